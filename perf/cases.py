@@ -131,16 +131,17 @@ def _nodes(case):
 
 def work(case):
     """A step reads and writes the 18 populations of every fluid node; the
-    fields that are read at the end, and a checkpoint's 18 populations, are
-    FP64 (FP32 in the host call, whose inputs are the mask and two FP32
-    densities). About 380 operations per
+    fields that are kept at the end, and a checkpoint's 18 populations, are
+    FP32 (FP64 for FP64 storage; the host call's inputs are the mask and two
+    FP32 densities). About 380 operations per
     node and step."""
     updates = case["steps"] * _nodes(case)
     if case["family"] == "batch_mixed":
         cells = 46_000 * case["n"]
     else:
         cells = case["nx"] * case["ny"] * (45 if case["family"] == "batch_study" else 1)
-    io = cells * (9 + 16 if case["reads"] == "host" else 32 + 144 if case["reads"] == "checkpoint" else 32)
+    values = 4 + (18 if case["reads"] == "checkpoint" else 0)
+    io = cells * (values * (8 if case["storage"] == "fp64" else 4) + (9 if case["reads"] == "host" else 0))
     return {"bytes": updates * 36 * _STORAGE_BYTES[case["storage"]] + io, "flops": 380 * updates}
 
 
@@ -246,15 +247,22 @@ def run(state):
         return state["outs"]
     if state["batch"] is not None:
         state["batch"].step(case["steps"])
-        return _joined([sim.moments() for sim in sims])
+        return _kept(case, _joined([sim.moments() for sim in sims]))
     sims[0].step(case["steps"])
     if case["reads"] == "diagnostics":
         d = sims[0].diagnostics(bridge=state["bridge"])
-        return {"bridge_radius": d["bridge_radius"], "max_u": d["max_u"], "com": d["com"],
-                "com_velocity": d["com_velocity"], "fields": sims[0].moments()}
+        sample = np.array([d["bridge_radius"], d["max_u"], *d["com"], *d["com_velocity"]],
+                          np.float64 if case["storage"] == "fp64" else np.float32)
+        return {"sample": sample, "fields": _kept(case, sims[0].moments())}
     if case["reads"] == "checkpoint":
-        return sims[0].moments(), sims[0].populations()
-    return sims[0].moments()
+        return _kept(case, sims[0].moments()), _kept(case, [sims[0].populations()])[0]
+    return _kept(case, sims[0].moments())
+
+
+def _kept(case, fields):
+    """What a study keeps of the FP64 fields it is given: the precision the
+    simulation computes in."""
+    return [f if case["storage"] == "fp64" else f.float() for f in fields]
 
 
 def _joined(fields):
@@ -387,8 +395,7 @@ def exact(case, seed):
         return _joined(moments)
     if case["reads"] == "checkpoint":
         x, y, nx, ny = boxes[0]
-        return moments[0], torch.stack([torch.stack([a[y:y + ny, x:x + nx] for a in f[s]]) for s in range(2)])
+        return list(moments[0]), torch.stack([torch.stack([a[y:y + ny, x:x + nx] for a in f[s]]) for s in range(2)])
     if case["reads"] == "diagnostics":
-        return {"bridge_radius": None, "max_u": None, "com": (None, None), "com_velocity": (None, None),
-                "fields": moments[0]}
-    return moments[0]
+        return {"sample": None, "fields": list(moments[0])}
+    return list(moments[0])
