@@ -116,11 +116,14 @@ typedef enum {
  *   lbm_step_profiled. Slower than TILED on GB300 (the windows also carry
  *   the solid slots that the tiled kernel's lists skip).
  * AUTO picks the schedule measured fastest on GB300, at each step from the
- * installed wetting scheme: for 4- and 8-byte storage TILED under the
+ * installed wetting scheme: for FP64 storage TWO_PASS (bound by the FP64
+ * pipe: the single passes update the nodes around a tile again); for 4-byte
+ * storage TILED under the
  * improved scheme (a quarter fewer bytes than TWO_PASS and 8% faster on the
  * 8192^2 porous medium) and HALO under Martys-Chen, LLKC and the constant
- * solid density (6% faster than TILED there); the workspace keeps both sets
- * of lists and the halo lists are built at the first step that needs them.
+ * solid density (6% faster than TILED there); the workspace of 4- and 8-byte
+ * storage keeps both sets of lists and the halo lists are built at the first
+ * step that needs them.
  * TWO_PASS for 16-bit storage. */
 typedef enum {
   LBM_KERNEL_AUTO = 0,

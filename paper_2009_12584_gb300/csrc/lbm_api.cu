@@ -206,7 +206,39 @@ lbm_status launch(lbm_ctx* c, int cls, const char* where, Fn&& fn) {
   return s;
 }
 
+}  // namespace
+
+// Before work that reads the density planes under a scheme without virtual
+// densities: zero the rho~ an earlier scheme of this context left in them.
+lbm_status clear_virtual(lbm_ctx* c, cudaStream_t stream) {
+  if (!c->virt_written || c->ph.bc == BC_VAVG) return LBM_OK;
+  const int nb = (c->n_iface + 127) / 128;
+  if (c->prm.storage == LBM_STORE_FP64)
+    k_clear_virtual<double><<<nb, 128, 0, stream>>>((double*)c->Pbuf[0], (double*)c->Pbuf[1], (double*)c->Pbuf[2],
+                                                    c->iface_list, c->n_iface, c->g);
+  else
+    k_clear_virtual<float><<<nb, 128, 0, stream>>>((float*)c->Pbuf[0], (float*)c->Pbuf[1], (float*)c->Pbuf[2],
+                                                   c->iface_list, c->n_iface, c->g);
+  lbm_status s = after_launch(c, "k_clear_virtual");
+  if (!s) c->virt_written = false;
+  return s;
+}
+
+namespace {
+
 dim3 node_grid(const Geo& g, int bx) { return dim3((g.nx + bx - 1) / bx, g.ny); }
+
+// rho~ of Eq. 8 into the interface-solid cells of density plane P (improved
+// scheme only).
+template <typename C>
+lbm_status launch_virtual(lbm_ctx* c, C* P) {
+  if (c->ph.bc != BC_VAVG || c->n_iface == 0) return LBM_OK;
+  c->virt_written = true;
+  return launch(c, LBM_KC_VIRTUAL, "k_virtual_density", [&] {
+    k_virtual_density<C><<<(c->n_iface + 127) / 128, 128, 0, c->stream>>>(P, c->iface_mask, c->iface_list, c->n_iface,
+                                                                           c->g, kphys<C>(c->ph));
+  });
+}
 
 // Densities of the current state (and rho~ at interface-solid nodes) into
 // the spare density plane Pbuf[pcur ^ 1]; Pbuf[pcur] keeps the references
@@ -222,13 +254,7 @@ lbm_status launch_density_and_virtual(lbm_ctx* c, const T* f) {
   });
   if (s) return s;
   c->p_valid = false;
-  if (c->ph.bc == BC_VAVG && c->n_iface > 0) {
-    s = launch(c, LBM_KC_VIRTUAL, "k_virtual_density", [&] {
-      k_virtual_density<C><<<(c->n_iface + 127) / 128, 128, 0, c->stream>>>(P, c->iface_mask, c->iface_list,
-                                                                             c->n_iface, c->g, kphys<C>(c->ph));
-    });
-  }
-  return s;
+  return launch_virtual<C>(c, P);
 }
 
 // Two-pass step: densities of the pulled populations into the spare plane,
@@ -238,7 +264,8 @@ template <typename T>
 lbm_status step_two_pass(lbm_ctx* c, int nsteps) {
   using C = typename Pop<T>::C;
   const int nb = (c->n_fluid + 255) / 256;
-  const int nbc = (c->n_fluid + COLLIDE_THREADS - 1) / COLLIDE_THREADS;
+  const int ntc = collide_threads<T>(c->n_fluid, c->num_sms);
+  const int nbc = (c->n_fluid + ntc - 1) / ntc;
   for (int t = 0; t < nsteps && c->n_fluid > 0; ++t) {
     const T* fin = (const T*)c->f[c->cur];
     T* fout = (T*)c->f[c->cur ^ 1];
@@ -252,16 +279,10 @@ lbm_status step_two_pass(lbm_ctx* c, int nsteps) {
                                     kphys<C>(c->ph));
     });
     if (s) return s;
-    if (c->ph.bc == BC_VAVG && c->n_iface > 0) {
-      s = launch(c, LBM_KC_VIRTUAL, "k_virtual_density", [&] {
-        k_virtual_density<C><<<(c->n_iface + 127) / 128, 128, 0, c->stream>>>(P, c->iface_mask, c->iface_list,
-                                                                               c->n_iface, c->g, kphys<C>(c->ph));
-      });
-      if (s) return s;
-    }
+    if ((s = launch_virtual<C>(c, P))) return s;
     s = launch(c, LBM_KC_COLLIDE, "k_collide_list", [&] {
       auto kc = vr ? k_collide_list<T, kDev<T>> : k_collide_list<T, false>;
-      kc<<<nbc, COLLIDE_THREADS, 0, c->stream>>>(fin, fout, P, Pref, c->Ubuf[c->cur], c->Ubuf[c->cur ^ 1], c->flags,
+      kc<<<nbc, ntc, 0, c->stream>>>(fin, fout, P, Pref, c->Ubuf[c->cur], c->Ubuf[c->cur ^ 1], c->flags,
                                                  c->fluid_list, c->n_fluid, c->g, kphys<C>(c->ph));
     });
     if (s) return s;
@@ -291,14 +312,8 @@ lbm_status step_fused(lbm_ctx* c, int nsteps) {
     C* Pin = (C*)c->Pbuf[c->pcur];
     C* Pout = (C*)c->Pbuf[c->pcur ^ 1];
     lbm_status s;
-    if (c->ph.bc == BC_VAVG && c->n_iface > 0) {
-      // rho~(t) of Eq. 8 into the solid cells of the plane the step reads
-      s = launch(c, LBM_KC_VIRTUAL, "k_virtual_density", [&] {
-        k_virtual_density<C><<<(c->n_iface + 127) / 128, 128, 0, c->stream>>>(Pin, c->iface_mask, c->iface_list,
-                                                                               c->n_iface, c->g, kphys<C>(c->ph));
-      });
-      if (s) return s;
-    }
+    // rho~(t) of Eq. 8 into the solid cells of the plane the step reads
+    if ((s = launch_virtual<C>(c, Pin))) return s;
     lbm_status ls = LBM_OK;
     if constexpr (sizeof(T) == 4) {
       if (c->tma) {
@@ -372,13 +387,7 @@ lbm_status step_tiled16(lbm_ctx* c, int nsteps) {
     C* P = (C*)c->Pbuf[c->pcur ^ 1];
     C* Po = (C*)c->Pbuf[2];
     lbm_status s;
-    if (c->ph.bc == BC_VAVG && c->n_iface > 0) {
-      s = launch(c, LBM_KC_VIRTUAL, "k_virtual_density", [&] {
-        k_virtual_density<C><<<(c->n_iface + 127) / 128, 128, 0, c->stream>>>(P, c->iface_mask, c->iface_list,
-                                                                               c->n_iface, c->g, kphys<C>(c->ph));
-      });
-      if (s) return s;
-    }
+    if ((s = launch_virtual<C>(c, P))) return s;
     lbm_status ls = LBM_OK;
     s = launch(c, LBM_KC_FUSED, "k_tile", [&] {
       ls = launch_tiled<T>(c->g, c->ph, fin, fout, P, Pref, c->Ubuf[c->cur], c->Ubuf[c->cur ^ 1], Po, c->flags,
@@ -441,7 +450,17 @@ lbm_status step_halo(lbm_ctx* c, int nsteps) {
 
 template <typename T>
 lbm_status do_step(lbm_ctx* c, int nsteps) {
+  if (nsteps > 0) {
+    lbm_status s = clear_virtual(c, c->stream);
+    if (s) return s;
+  }
   if constexpr (sizeof(T) >= 4) {  // the marching kernel stores 4- and 8-byte populations only
+    // AUTO with FP64 storage: bound by the FP64 pipe, so the schedule that
+    // updates every node once (the single passes update a tile's ring again):
+    // before the update's operations were halved too, 100 x 50 took 20.5
+    // against 61 us per step, 800 x 600 207 against 298 us, 1400 x 1000 553
+    // against 701 us
+    if (sizeof(T) == 8 && c->prm.kernel == LBM_KERNEL_AUTO) return step_two_pass<T>(c, nsteps);
     // HALO always; AUTO under the one-node-reach schemes (the improved
     // scheme's Eq. 8 reaches three rings, where the tiled schedule wins)
     const bool halo = c->prm.kernel == LBM_KERNEL_HALO || (c->prm.kernel == LBM_KERNEL_AUTO && c->ph.bc != BC_VAVG);
@@ -464,7 +483,8 @@ lbm_status do_step(lbm_ctx* c, int nsteps) {
 template <typename T, int MODE, typename O = double>
 lbm_status do_eval(lbm_ctx* c, O* out) {
   const T* fin = (const T*)c->f[c->cur];
-  lbm_status s = launch_density_and_virtual<T>(c, fin);
+  lbm_status s = clear_virtual(c, c->stream);
+  if (!s) s = launch_density_and_virtual<T>(c, fin);
   if (s) return s;
   using C = typename Pop<T>::C;
   k_collide<T, MODE, O><<<node_grid(c->g, 128), 128, 0, c->stream>>>(
@@ -674,6 +694,7 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const uint8_t* d_mask) {
   }
   // clear the density planes so solid cells read as zero
   c->p_valid = false;
+  c->virt_written = false;
   s = check_cuda(c, cudaMemsetAsync(c->Pbase, 0, (c->Pbuf[2] ? 6 : 4) * (size_t)g.plane * compute_size(c->prm.storage),
                                     c->stream), "cudaMemsetAsync");
   if (s) return s;

@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB)
 }
 
 template <typename T, bool VR = false>
-__global__ void __launch_bounds__(256, 4) k_collide_batch(const BatchDesc<typename Pop<T>::C>* __restrict__ d,
+__global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_collide_batch(const BatchDesc<typename Pop<T>::C>* __restrict__ d,
                                                        const int2* __restrict__ blk, int parity) {
   using C = typename Pop<T>::C;
   const int2 b = blk[blockIdx.x];
@@ -336,6 +336,12 @@ template <typename T>
 lbm_status batch_step(lbm_batch* b, int nsteps) {
   using C = typename Pop<T>::C;
   fill_descs<C>(b);
+  for (int s = 0; s < b->n && nsteps > 0; ++s) {
+    lbm_ctx* c = b->ctx[s];
+    lbm_status cs = clear_virtual(c, b->stream);
+    if (cs) return bfail(b, cs, c->err);
+    if (c->ph.bc == BC_VAVG && c->n_iface > 0) c->virt_written = true;
+  }
   lbm_status st = bcuda(b, cudaMemcpyAsync(b->d_desc, b->h_desc, (size_t)b->n * sizeof(BatchDesc<C>),
                                            cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
   // the staging buffer is rewritten by the next call: wait for the copy

@@ -242,7 +242,11 @@ struct Phys {
 // the host (an FP32 kernel then does no FP64 conversions).
 template <typename C>
 struct PhysK {
-  C omega[2], kF[2], G_AB, G_s[2], chi[2], rho_s[2], rho_ref[2];
+  C omega[2];
+  C kF[2];   // 1 - 1 / (2 tau)
+  C k3[2];   // kF / 3
+  C h[2];    // (1 - omega) / 2
+  C G_AB, G_s[2], chi[2], rho_s[2];
   int bc, pairing, avg9, uniform;
 };
 
@@ -252,10 +256,11 @@ inline PhysK<C> kphys(const Phys& p) {
   for (int s = 0; s < 2; ++s) {
     k.omega[s] = C(p.omega[s]);
     k.kF[s] = C(p.kF[s]);
+    k.k3[s] = C(p.kF[s] / 3.0);
+    k.h[s] = C(0.5 * (1.0 - p.omega[s]));
     k.G_s[s] = C(p.G_s[s]);
     k.chi[s] = C(p.chi[s]);
     k.rho_s[s] = C(p.rho_s[s]);
-    k.rho_ref[s] = C(p.rho_ref[s]);
   }
   k.G_AB = C(p.G_AB);
   k.bc = p.bc;
@@ -265,44 +270,79 @@ inline PhysK<C> kphys(const Phys& p) {
   return k;
 }
 
-// sum_i w_i c_i q_i over the eight moving directions, as paired
-// differences (q[0] unused).
+// 36 sum_i w_i c_i phi(x + c_i) for the eight neighbour bits of a node's
+// flags: small integers, exact in either type. One 8-byte load (2 KB table,
+// resident in L1) in place of eight selects and a weighted sum.
+struct WallPush {
+  float2 v[256];
+  constexpr WallPush() : v() {
+    for (int m = 0; m < 256; ++m) {
+      int sx = 0, sy = 0;
+      for (int i = 1; i < 9; ++i)
+        if (m >> (i - 1) & 1) {
+          sx += (i <= 4 ? 4 : 1) * cx_of(i);
+          sy += (i <= 4 ? 4 : 1) * cy_of(i);
+        }
+      v[m].x = (float)sx;
+      v[m].y = (float)sy;
+    }
+  }
+};
+static __device__ const WallPush WALL_PUSH = WallPush();
+__device__ __forceinline__ float2 wall_push(uint16_t fl) { return __ldg(&WALL_PUSH.v[(fl >> 1) & 0xFF]); }
+
+// 36 sum_i w_i c_i q_i over the eight moving directions (q[0] unused).
 template <typename C>
-__device__ __forceinline__ void weighted_sum(const C q[9], C& sx, C& sy) {
-  sx = (q[1] - q[3]) * C(1.0 / 9.0) + ((q[5] - q[7]) + (q[8] - q[6])) * C(1.0 / 36.0);
-  sy = (q[2] - q[4]) * C(1.0 / 9.0) + ((q[5] - q[7]) + (q[6] - q[8])) * C(1.0 / 36.0);
+__device__ __forceinline__ void weighted_sum36(const C q[9], C& sx, C& sy) {
+  const C d57 = q[5] - q[7], d68 = q[6] - q[8];
+  sx = fma(C(4), q[1] - q[3], d57 - d68);
+  sy = fma(C(4), q[2] - q[4], d57 + d68);
 }
 
 // Interaction force on both components at a fluid node (Eq. 5 restricted to
 // fluid neighbours plus Eq. 7). nbP[s][i] is the value of the density plane
-// of component s at x + c_i (the density at fluid nodes, rho~ at interface-
-// solid nodes under the improved scheme); fl holds the neighbour bits.
-// Values at solid neighbours are only used under the improved scheme.
-// BULK_FAST: take the short path when no neighbour is solid (callers that
-// know their whole warp is bulk pass fl = 0; others pass false so that a
-// warp does not split between the two paths). The general path splits the
-// neighbour values by select into a fluid and a solid part and sums each
-// with the bulk formula. With ph.uniform (see Phys) every node takes the
-// short path.
-template <typename C, bool BULK_FAST = true>
-__device__ __forceinline__ void interaction_force(const PhysK<C>& ph, uint16_t fl, const C rho[2],
+// of component s at x + c_i: the density at fluid nodes, rho~ at interface-
+// solid nodes under the improved scheme, 0 at every other solid node; fl
+// holds the neighbour bits (unused when !walls: no neighbour is solid). The
+// zeros make the sum of Eq. 5 the same weighted sum at every node; with
+// ph.uniform (see Phys) that sum also holds the solid part of Eq. 7. A node
+// without solid neighbours gets the same bits whatever `walls` says.
+template <typename C>
+__device__ __forceinline__ void interaction_force(const PhysK<C>& ph, uint16_t fl, bool walls, const C rho[2],
                                                   const C nbP[2][9], C F[2][2]) {
-  const C G = ph.G_AB;
-  if ((BULK_FAST && !(fl & NB_ANY)) || ph.uniform) {
-    // bulk node: every neighbour is fluid, Eq. 5 over all eight
+  C ax[2], ay[2], r36[2];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) r36[s] = rho[s] * C(-1.0 / 36.0);
+  if (ph.bc != BC_VAVG || ph.uniform || !walls) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s) weighted_sum36(nbP[s], ax[s], ay[s]);
+    if (ph.bc == BC_VAVG || !walls) {
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        const C rg = r36[s] * ph.G_AB;
+        F[s][0] = rg * ax[1 - s];
+        F[s][1] = rg * ay[1 - s];
+      }
+      return;
+    }
+    const float2 v = wall_push(fl);
+    const C vx = C(v.x), vy = C(v.y);
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
-      C ax, ay;
-      weighted_sum(nbP[1 - s], ax, ay);
-      F[s][0] = -rho[s] * (G * ax);
-      F[s][1] = -rho[s] * (G * ay);
+      // the component whose solid pseudopotential enters Eq. 7
+      const C rho_c = ph.pairing != 0 ? rho[s] : rho[1 - s];
+      const C rs_c = ph.pairing != 0 ? ph.rho_s[s] : ph.rho_s[1 - s];
+      const C gs = ph.bc == BC_MC ? ph.G_s[s] : ph.G_s[s] * (ph.bc == BC_LLKC ? rho_c : rs_c);
+      const C rg = r36[s] * ph.G_AB, rs = r36[s] * gs;
+      F[s][0] = fma(rg, ax[1 - s], rs * vx);
+      F[s][1] = fma(rg, ay[1 - s], rs * vy);
     }
     return;
   }
-  C ax[2], ay[2];                    // fluid-weighted sums per component
-  C sx[2] = {0, 0}, sy[2] = {0, 0};  // solid-weighted sums (improved scheme)
-  C qf[9], qs[9], b[9];
-  qf[0] = qs[0] = b[0] = C(0);
+  // the improved scheme with other strengths or the self pairing: the fluid
+  // and the solid part are summed apart
+  C sx[2], sy[2], qf[9], qs[9];
+  qf[0] = qs[0] = C(0);
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
 #pragma unroll
@@ -311,39 +351,16 @@ __device__ __forceinline__ void interaction_force(const PhysK<C>& ph, uint16_t f
       qf[i] = solid ? C(0) : nbP[s][i];
       qs[i] = solid ? nbP[s][i] : C(0);
     }
-    weighted_sum(qf, ax[s], ay[s]);
-    if (ph.bc == BC_VAVG) weighted_sum(qs, sx[s], sy[s]);
+    weighted_sum36(qf, ax[s], ay[s]);
+    weighted_sum36(qs, sx[s], sy[s]);
   }
-#pragma unroll
-  for (int i = 1; i < 9; ++i) b[i] = (fl & nb_bit(i)) ? C(1) : C(0);
-  C vx, vy;  // sum_i w_i phi(x + c_i) c_i
-  weighted_sum(b, vx, vy);
+  const bool self = ph.pairing != 0;
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
-    const int o = 1 - s;
-    // the component whose solid pseudopotential enters Eq. 7 (selects only
-    // between compile-time indices so the arrays stay in registers)
-    const bool self = ph.pairing != 0;
-    const C rho_c = self ? rho[s] : rho[o];
-    const C sx_c = self ? sx[s] : sx[o], sy_c = self ? sy[s] : sy[o];
-    const C rs_c = self ? ph.rho_s[s] : ph.rho_s[o];
-    C bx, by;
-    if (ph.bc == BC_MC) {
-      bx = vx;
-      by = vy;
-    } else if (ph.bc == BC_LLKC) {
-      bx = rho_c * vx;
-      by = rho_c * vy;
-    } else if (ph.bc == BC_VAVG) {
-      bx = sx_c;
-      by = sy_c;
-    } else {
-      bx = rs_c * vx;
-      by = rs_c * vy;
-    }
-    const C Gs = ph.G_s[s];
-    F[s][0] = -rho[s] * (G * ax[o] + Gs * bx);
-    F[s][1] = -rho[s] * (G * ay[o] + Gs * by);
+    const C bx = self ? sx[s] : sx[1 - s], by = self ? sy[s] : sy[1 - s];
+    const C rg = r36[s] * ph.G_AB, rs = r36[s] * ph.G_s[s];
+    F[s][0] = fma(rg, ax[1 - s], rs * bx);
+    F[s][1] = fma(rg, ay[1 - s], rs * by);
   }
 }
 
@@ -376,51 +393,75 @@ __device__ __forceinline__ float rho_over_9<float>(float rho) {
 }
 template <>
 __device__ __forceinline__ double rho_over_9<double>(double rho) {
-  return rho / 9.0;
+  constexpr double HI = 1.0 / 9.0;
+  constexpr double LO = HI * 0x1p-54;  // 9 HI = 1 - 2^-54
+  return fma(rho, HI, rho * LO);
 }
 
-// BGK relaxation towards Eq. 2 plus the Guo source of Eq. 4, in place:
-//   f_i <- f_i + Delta_i,  Delta_i = omega (f^eq_i - f_i) + S_i,
-// with f^eq_i - f_i evaluated as (rho w_i - f_i) + rho w_i p_i, where p_i =
-// 3 c.u + 4.5 (c.u)^2 - 1.5 u^2 is the small part of Eq. 2's bracket, so the
-// O(1) part of the bracket is never rounded, and S_i of Eq. 4 written as
-// w_i (1 - 1/(2 tau)) [3 c.F - 3 u.F + 9 (c.u)(c.F)]. The moving populations
-// take their increments and the rest population takes minus their sum:
-// exactly what the method gives (sum_i Delta_i = 0 by Eqs. 2 and 4), and in
-// floating point the mass of each component changes only by the rounding
-// of the nine final additions, whatever the rounding of rho.
+// Force, velocity u of Eq. 3, BGK relaxation towards Eq. 2 and the Guo
+// source of Eq. 4 at one fluid node in the FP64 compute type, in place
+// (f: pulled populations on entry, f* on exit). FP64 instructions run at
+// 1/32 of the FP32 rate on this GPU and bound every FP64 pass, so the
+// update is written for their number: opposite directions go as pairs, with
+// S = f_i + f_-i and D = f_i - f_-i shared by rho, the momentum and the
+// relaxation,
+//   P = (f*_i + f*_-i) / 2 = (1 - omega) S / 2 + omega r (1 + e) + E,
+//   M = (f*_i - f*_-i) / 2 = (1 - omega) D / 2 + omega r 3 c.u + g,
+// r = w_i rho, e = 4.5 (c.u)^2 - 1.5 u^2, g = 3 w_i (1 - 1/(2 tau)) c.F,
+// E = 3 c.u g - 3 w_i (1 - 1/(2 tau)) u.F; the rest population takes minus
+// what the pairs gained (sum_i Delta_i = 0 by Eqs. 2 and 4), so that each
+// component's mass changes only by rounding. About 180 FP64 instructions
+// per node where one direction at a time took 366; with the two-pass
+// schedule, 800 x 600 went from 207 to 178 us per step (128 registers, no
+// spills).
 template <typename C>
-__device__ __forceinline__ void collide(C f[2][9], const C rho[2], C ux, C uy, const C F[2][2],
-                                        const C omega[2], const C kF[2]) {
-  const C usq15 = C(1.5) * (ux * ux + uy * uy);
-  C r9[2], r36[2], k9[2], k36[2], uF3[2];
+__device__ __forceinline__ void update_node(C f[2][9], const C nbP[2][9], uint16_t fl, bool walls,
+                                            const PhysK<C>& ph, C rho[2], C u[2]) {
+  C S[2][4], D[2][4], jx[2], jy[2];
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
-    r9[s] = rho_over_9(rho[s]);
-    r36[s] = C(0.25) * r9[s];  // exact
-    k9[s] = kF[s] * C(1.0 / 9.0);
-    k36[s] = kF[s] * C(1.0 / 36.0);
-    uF3[s] = C(3) * (ux * F[s][0] + uy * F[s][1]);
-  }
-  C acc[2] = {0, 0};
 #pragma unroll
-  for (int i = 1; i < 9; ++i) {
-    const C cu = C(cx_of(i)) * ux + C(cy_of(i)) * uy;
-    const C p = cu * (C(3) + C(4.5) * cu) - usq15;
-    const C cu9 = C(9) * cu;
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const C cF = C(cx_of(i)) * F[s][0] + C(cy_of(i)) * F[s][1];
-      const C src = (i <= 4 ? k9[s] : k36[s]) * ((C(3) * cF - uF3[s]) + cu9 * cF);
-      const C ri = i <= 4 ? r9[s] : r36[s];
-      const C d = (ri - f[s][i]) + ri * p;
-      const C delta = omega[s] * d + src;
-      acc[s] += delta;
-      f[s][i] = f[s][i] + delta;
+    for (int a = 0; a < 4; ++a) {
+      const int i = a < 2 ? a + 1 : a + 3;  // 1, 2, 5, 6
+      S[s][a] = f[s][i] + f[s][opp_of(i)];
+      D[s][a] = f[s][i] - f[s][opp_of(i)];
     }
+    rho[s] = ((f[s][0] + S[s][0]) + S[s][1]) + (S[s][2] + S[s][3]);  // as density()
+    jx[s] = D[s][0] + (D[s][2] - D[s][3]);
+    jy[s] = D[s][1] + (D[s][2] + D[s][3]);
   }
-  f[0][0] = f[0][0] - acc[0];
-  f[1][0] = f[1][0] - acc[1];
+  C F[2][2];
+  interaction_force<C>(ph, fl, walls, rho, nbP, F);
+  const C inv = C(1) / (rho[0] + rho[1]);
+  const C ux = fma(C(0.5), F[0][0] + F[1][0], jx[0] + jx[1]) * inv;
+  const C uy = fma(C(0.5), F[0][1] + F[1][1], jy[0] + jy[1]) * inv;
+  const C c3[4] = {C(3) * ux, C(3) * uy, C(3) * (ux + uy), C(3) * (uy - ux)};
+  const C base = fma(C(-1.5), fma(ux, ux, uy * uy), C(1));
+  C e1[4];  // 1 + e
+#pragma unroll
+  for (int a = 0; a < 4; ++a) e1[a] = fma(C(0.5) * c3[a], c3[a], base);
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const C w9 = ph.omega[s] * rho_over_9(rho[s]), w36 = C(0.25) * w9;
+    const C gx = ph.k3[s] * F[s][0], gy = ph.k3[s] * F[s][1];
+    const C uF = fma(ux, gx, uy * gy), gx4 = C(0.25) * gx, gy4 = C(0.25) * gy;
+    const C g[4] = {gx, gy, gx4 + gy4, gy4 - gx4};
+    C acc = C(0);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      const int i = a < 2 ? a + 1 : a + 3;
+      const C r = a < 2 ? w9 : w36;
+      const C E = fma(c3[a], g[a], a < 2 ? -uF : C(-0.25) * uF);
+      const C P = fma(ph.h[s], S[s][a], fma(r, e1[a], E));
+      const C M = fma(ph.h[s], D[s][a], fma(r, c3[a], g[a]));
+      acc += fma(C(2), P, -S[s][a]);
+      f[s][i] = P + M;
+      f[s][opp_of(i)] = P - M;
+    }
+    f[s][0] -= acc;
+  }
+  u[0] = ux;
+  u[1] = uy;
 }
 
 // Halfway bounce-back done by the writer. When the upstream node x - c_i of

@@ -60,20 +60,7 @@ __device__ __forceinline__ void march_update(C fv[2][9], const C nbP[2][9], uint
       fv[1][i] = fp[i].y;
     }
   } else {
-    const C rho[2] = {density(fv[0]), density(fv[1])};
-    rho_out[0] = rho[0];
-    rho_out[1] = rho[1];
-    C F[2][2];
-    interaction_force<C, true>(ph, fl, rho, nbP, F);
-    C jxA, jyA, jxB, jyB;
-    momentum(fv[0], jxA, jyA);
-    momentum(fv[1], jxB, jyB);
-    const C inv = C(1) / (rho[0] + rho[1]);
-    const C ux = ((jxA + jxB) + C(0.5) * (F[0][0] + F[1][0])) * inv;
-    const C uy = ((jyA + jyB) + C(0.5) * (F[0][1] + F[1][1])) * inv;
-    collide(fv, rho, ux, uy, F, ph.omega, ph.kF);
-    u_out[0] = ux;
-    u_out[1] = uy;
+    update_node<C>(fv, nbP, fl, general, ph, rho_out, u_out);
   }
 }
 

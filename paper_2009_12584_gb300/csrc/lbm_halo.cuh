@@ -175,6 +175,16 @@ __global__ void __launch_bounds__(HALO_THREADS, HALO_MINB)
   if (vavg && threadIdx.x < HALO_MW) fm[threadIdx.x] = __ldg(fmask + (int64_t)tile * HALO_MW + threadIdx.x);
   const int x0 = (tile % ntx) * HALO_W, y0 = (tile / ntx) * HALO_H;
   const int korg = g.idx(x0 - HALO_R, y0 - HALO_R);  // padded index of slot 0
+  if (sizeof(C) == 8 && !vavg) {
+    // the schemes without virtual densities read 0 at solid slots
+    for (int w = threadIdx.x >> 5; w < HALO_MW; w += HALO_THREADS / 32) {
+      const uint32_t bits = __ldg(fmask + (int64_t)tile * HALO_MW + w);
+      const int slot = w * 32 + (threadIdx.x & 31);
+      V z;
+      z.x = z.y = C(0);
+      if (slot < HALO_RS && !(bits >> (threadIdx.x & 31) & 1u)) rho[slot] = z;
+    }
+  }
   const C zr[2][9] = {};  // storage references: unused for 4- and 8-byte populations
 
   // phase A: rho(t) of the tile and its rings

@@ -41,6 +41,7 @@ struct lbm_ctx {
                        // written with (16-bit encoding references); after a
                        // single-pass step, the densities of the current state
   int pcur;
+  bool virt_written;   // some density plane may hold rho~ at interface-solid cells
   bool p_valid;        // P holds the densities of the current state (single-pass)
   uint16_t* flags;
   int* iface_list;
@@ -85,3 +86,7 @@ struct lbm_ctx {
   int prof_n, prof_cap;
   char err[512];
 };
+
+// Zero the rho~ that an earlier improved-scheme step left in the density
+// planes when the installed scheme has none (lbm_api.cu).
+lbm_status clear_virtual(lbm_ctx* c, cudaStream_t stream);

@@ -26,10 +26,9 @@ __device__ __forceinline__ void gather(const T* __restrict__ f, const Geo& g, in
 // it. A CTA asks L2 for the list lines of the CTA LIST_AHEAD launches after
 // it (one 128-byte line per 32 entries), so that CTA finds them there.
 constexpr int LIST_AHEAD = 1024;
-template <int NT>
 __device__ __forceinline__ void prefetch_list_ahead(const int* __restrict__ list, int n) {
-  if (threadIdx.x < NT / 32) {
-    const int64_t t = ((int64_t)blockIdx.x + LIST_AHEAD) * NT + threadIdx.x * 32;
+  if (threadIdx.x < blockDim.x / 32) {
+    const int64_t t = ((int64_t)blockIdx.x + LIST_AHEAD) * blockDim.x + threadIdx.x * 32;
     if (t < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(list + t));
   }
 }
@@ -316,6 +315,19 @@ __device__ __forceinline__ void collide_node_pair(const T* __restrict__ f, T* __
 // with 256 threads when its warps finish at different times.
 constexpr int COLLIDE_THREADS = 128;
 
+// Threads per CTA for n nodes. FP64 passes are bound by each SM's FP64 pipe,
+// so what counts is that every SM gets the same share of the nodes: one warp
+// per CTA until 16 CTAs of 128 fall to each SM (above that the last wave is
+// under 6% of the work). Other storage is bound by latency there; smaller
+// CTAs only spread lists of less than two CTAs per SM.
+template <typename T>
+inline int collide_threads(int n, int num_sms) {
+  if (sizeof(T) == 8) return n < 16 * COLLIDE_THREADS * num_sms ? 32 : COLLIDE_THREADS;
+  int nt = COLLIDE_THREADS;
+  while (nt > 32 && n < 2 * num_sms * nt) nt /= 2;
+  return nt;
+}
+
 // Three paths, chosen per warp so that a warp never splits between them: a
 // warp whose 32 nodes are all bulk (eight fluid neighbours, away from
 // periodic borders) loads no flags and has no adhesion and no bounce-back;
@@ -347,22 +359,10 @@ __device__ __forceinline__ void collide_node(const T* __restrict__ f, T* __restr
   pull_refs<T>(Pref, Uref, g, k, fl, warp_edge, ref);
   C fv[2][9];
   gather<T>(f, g, k, ref, fv);
-  const C rho[2] = {density(fv[0]), density(fv[1])};
   C nbP[2][9];
   neighbour_P(P, g, k, nbP);
-  C F[2][2];
-  if (!warp_edge) {
-    interaction_force<C, true>(ph, 0, rho, nbP, F);
-  } else {
-    interaction_force<C, false>(ph, fl, rho, nbP, F);
-  }
-  C jxA, jyA, jxB, jyB;
-  momentum(fv[0], jxA, jyA);
-  momentum(fv[1], jxB, jyB);
-  const C inv = C(1) / (rho[0] + rho[1]);
-  const C ux = ((jxA + jxB) + C(0.5) * (F[0][0] + F[1][0])) * inv;
-  const C uy = ((jyA + jyB) + C(0.5) * (F[0][1] + F[1][1])) * inv;
-  collide(fv, rho, ux, uy, F, ph.omega, ph.kF);
+  C rho[2], u[2];
+  update_node<C>(fv, nbP, fl, warp_edge, ph, rho, u);
   write_refs<T>(rho, false, UVal{}, ref);  // the FP64 compute type stores 8-byte populations
   if (!warp_border) {
 #pragma unroll
@@ -377,9 +377,11 @@ __device__ __forceinline__ void collide_node(const T* __restrict__ f, T* __restr
   }
 }
 
-// VR as for k_density_list (Uref and Uo untouched without it).
+// VR as for k_density_list (Uref and Uo untouched without it). FP64: 128
+// registers without spills (64 spill 264 bytes); 16 warps per SM fill the
+// FP64 pipe.
 template <typename T, bool VR = false>
-__global__ void __launch_bounds__(COLLIDE_THREADS, 8) k_collide_list(const T* __restrict__ f, T* __restrict__ fo,
+__global__ void __launch_bounds__(COLLIDE_THREADS, sizeof(T) == 8 ? 4 : 8) k_collide_list(const T* __restrict__ f, T* __restrict__ fo,
                                                          const typename Pop<T>::C* __restrict__ P,
                                                          const typename Pop<T>::C* __restrict__ Pref,
                                                          const UPair* __restrict__ Uref,
@@ -387,7 +389,7 @@ __global__ void __launch_bounds__(COLLIDE_THREADS, 8) k_collide_list(const T* __
                                                          const uint16_t* __restrict__ flags,
                                                          const int* __restrict__ list, int nfluid, Geo g,
                                                          PhysK<typename Pop<T>::C> ph) {
-  prefetch_list_ahead<COLLIDE_THREADS>(list, nfluid);
+  prefetch_list_ahead(list, nfluid);
   collide_node<T>(f, fo, P, Pref, VR ? Uref : nullptr, VR ? Uo : nullptr, flags, list,
                   blockIdx.x * blockDim.x + threadIdx.x, nfluid, g, ph);
 }
@@ -471,6 +473,20 @@ __device__ __forceinline__ void virtual_density_node(C* __restrict__ P, const ui
   stP_ghosts(P, g, x, y, v0, v1);
 }
 
+// Zero the interface-solid cells (and their images) of up to three density
+// planes: a scheme without virtual densities reads 0 at every solid cell.
+template <typename C>
+__global__ void __launch_bounds__(128) k_clear_virtual(C* __restrict__ P0, C* __restrict__ P1, C* __restrict__ P2,
+                                                       const int* __restrict__ list, int n, Geo g) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  int x, y;
+  coords(g, list[t], x, y);
+  stP_ghosts(P0, g, x, y, C(0), C(0));
+  stP_ghosts(P1, g, x, y, C(0), C(0));
+  if (P2) stP_ghosts(P2, g, x, y, C(0), C(0));
+}
+
 template <typename C>
 __global__ void __launch_bounds__(128) k_virtual_density(C* __restrict__ P, const uint32_t* __restrict__ mask,
                                                          const int* __restrict__ list, int n, Geo g,
@@ -506,11 +522,22 @@ __global__ void __launch_bounds__(128) k_collide(const T* __restrict__ f, const 
   pull_refs<T>(Pref, Uref, g, k, fl, true, ref);
   C fv[2][9];
   gather<T>(f, g, k, ref, fv);
-  C rho[2] = {density(fv[0]), density(fv[1])};
+  const C rho[2] = {density(fv[0]), density(fv[1])};
   C nbP[2][9];
   neighbour_P(P, g, k, nbP);
   C F[2][2];
-  interaction_force(ph, fl, rho, nbP, F);
+  if constexpr (sizeof(C) == 4) {
+    float2 q[9], Fx, Fy;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) q[i] = f2(nbP[0][i], nbP[1][i]);
+    interaction_force2<true>(ph, fl, f2(rho[0], rho[1]), q, Fx, Fy);
+    F[0][0] = Fx.x;
+    F[1][0] = Fx.y;
+    F[0][1] = Fy.x;
+    F[1][1] = Fy.y;
+  } else {
+    interaction_force<C>(ph, fl, true, rho, nbP, F);
+  }
   C jxA, jyA, jxB, jyB;
   momentum(fv[0], jxA, jyA);
   momentum(fv[1], jxB, jyB);

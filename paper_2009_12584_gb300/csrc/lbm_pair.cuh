@@ -22,6 +22,12 @@ __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y
 __device__ __forceinline__ float2 swap2(float2 a) { return make_float2(a.y, a.x); }
 __device__ __forceinline__ float2 sel2(bool p, float2 a, float2 b) { return p ? a : b; }
 
+// sum_i w_i c_i q_i over the eight moving directions, as paired differences.
+__device__ __forceinline__ void weighted_sum(const float q[9], float& sx, float& sy) {
+  sx = (q[1] - q[3]) * (1.0f / 9.0f) + ((q[5] - q[7]) + (q[8] - q[6])) * (1.0f / 36.0f);
+  sy = (q[2] - q[4]) * (1.0f / 9.0f) + ((q[5] - q[7]) + (q[6] - q[8])) * (1.0f / 36.0f);
+}
+
 // sum_i w_i c_i q_i over the eight moving directions for both components.
 __device__ __forceinline__ void weighted_sum2(const float2 q[9], float2& sx, float2& sy) {
   const float2 d57 = sub2(q[5], q[7]), d86 = sub2(q[8], q[6]);
