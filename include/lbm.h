@@ -96,14 +96,15 @@ typedef enum {
  *   bytes per ring-extended region slot (about 2.4 bytes per node), and for
  *   16-bit storage by a third density plane (8 bytes per padded node), since
  *   a 16-bit step decodes with the densities of the step before.
- * HALO: one kernel per step and no density plane: each CTA takes a 32 x 14
- *   tile, recomputes rho(t) from the pulled populations for the tile and the
- *   1 to 3 node rings its force and Eq. 8 reach (3 for the D2Q25 average, 2
- *   for the D2Q9 average, 1 for the other schemes), evaluates Eq. 8 in
- *   shared memory and updates its own nodes. 4- and 8-byte storage (16-bit
- *   storage runs TWO_PASS); the workspace grows by about 4 bytes per node.
- *   The fastest schedule under Martys-Chen, LLKC and the constant solid
- *   density (one ring); slower than TILED under the improved scheme.
+ * HALO: one kernel per step, and for 4- and 8-byte storage no density plane:
+ *   each CTA takes a tile of 32 x 14 nodes (32 x 20 with 16-bit storage), whose
+ *   populations the Tensor Memory Accelerator copies into shared memory with
+ *   the 2 or 4 nodes around it, computes rho(t) of the tile and of the rings
+ *   its force and Eq. 8 reach (3 under the improved scheme, 1 under the
+ *   others), evaluates Eq. 8 there and updates its own nodes. Its lists take
+ *   the parts of the workspace that the geometry leaves unused (4- and 8-byte
+ *   storage: the workspace grows by about 4 bytes per node); where they do
+ *   not fit, TWO_PASS runs. The copies' wait is bounded as for TMA.
  * TMA: the TILED schedule (same lists, same results bit for bit) with two
  *   persistent CTAs per SM walking a list of the tiles that own fluid
  *   nodes; each tile's inputs, the nine population planes and the density
@@ -113,18 +114,16 @@ typedef enum {
  *   storage runs TILED); the workspace grows by 16 bytes per tile. A copy
  *   not seen to complete within about a second stops the kernel and is
  *   reported as LBM_ERR_TIMEOUT by the next lbm_sync, lbm_mass or
- *   lbm_step_profiled. Slower than TILED on GB300 (the windows also carry
+ *   lbm_step_profiled (until then further halo steps do nothing). Slower than
+ *   TILED on GB300 (the windows also carry
  *   the solid slots that the tiled kernel's lists skip).
- * AUTO picks the schedule measured fastest on GB300, at each step from the
- * installed wetting scheme: for FP64 storage TWO_PASS (bound by the FP64
- * pipe: the single passes update the nodes around a tile again); for 4-byte
- * storage TILED under the
- * improved scheme (a quarter fewer bytes than TWO_PASS and 8% faster on the
- * 8192^2 porous medium) and HALO under Martys-Chen, LLKC and the constant
- * solid density (6% faster than TILED there); the workspace of 4- and 8-byte
- * storage keeps both sets of lists and the halo lists are built at the first
- * step that needs them.
- * TWO_PASS for 16-bit storage. */
+ * AUTO picks the schedule measured fastest on GB300: TWO_PASS for FP64 storage
+ * (bound by the FP64 pipe: the single passes compute densities around a tile
+ * again) and HALO for the others (porous 4096^2, us per step under the
+ * improved scheme / LLKC: FP32 406 / 363 against 449 / 427 for TILED and 514 /
+ * 488 for TWO_PASS; FP16 376 / 337 against 434 / 412 for TWO_PASS); the
+ * workspace of 4- and 8-byte storage also keeps room for the tiled lists,
+ * which batches use. */
 typedef enum {
   LBM_KERNEL_AUTO = 0,
   LBM_KERNEL_TWO_PASS = 1,
@@ -256,8 +255,8 @@ lbm_status lbm_mass(lbm_ctx* ctx, double* h_out);
  * paper has no counterpart. */
 lbm_status lbm_set_l2_fetch_granularity(int32_t bytes, int32_t* previous);
 
-/* Test hook of the TMA schedule's bounded wait (not for production use):
- * from the next step on, the barrier of every tile's copies expects `bytes`
+/* Test hook of the bounded wait of the TMA and halo schedules (not for
+ * production use): from the next step on, the barrier of every tile's copies expects `bytes`
  * (0 ... 4096) more than the copies deliver, so that its wait runs out
  * after about a second, each CTA stops after waiting (bounded) for the
  * copies it has in flight, and the next lbm_sync, lbm_mass or

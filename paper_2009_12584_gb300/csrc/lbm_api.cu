@@ -39,7 +39,7 @@ bool make_geo(const lbm_params* p, Geo* g) {
 }
 
 struct Layout {
-  size_t f, P, U, flags, list, imask, flist, tent, toff, tcnt, twork, hent, hoff, hcnt, hmask, counts, small, partial, mass,
+  size_t f, P, U, flags, list, imask, flist, tent, toff, tcnt, twork, hlists, hend, counts, small, partial, mass,
       smask, stage, dpart, total;
 };
 
@@ -56,11 +56,10 @@ bool uses_tma(const lbm_params* p) {
   return TMA_AVAILABLE && p->kernel == LBM_KERNEL_TMA && p->storage == LBM_STORE_FP32;
 }
 
-// Whether a context keeps the per-tile lists of the halo schedule (4- and
-// 8-byte storage; 16-bit storage runs the two-pass schedule instead). AUTO
-// keeps room for them: it runs the halo schedule under the wetting schemes
-// whose force reaches one node (Martys-Chen, LLKC, constant rho_s), where
-// it is the fastest, and builds the lists at the first such step.
+// Whether the workspace has an area of its own for the lists of the halo
+// schedule (4- and 8-byte storage). The lists themselves go wherever they
+// fit (place_halo_lists): the part of the interface arrays that the geometry
+// leaves unused usually holds them all, with any storage.
 bool uses_halo(const lbm_params* p) {
   const bool wide = p->storage == LBM_STORE_FP32 || p->storage == LBM_STORE_FP64;
   return (p->kernel == LBM_KERNEL_HALO || p->kernel == LBM_KERNEL_AUTO) && wide;
@@ -95,11 +94,14 @@ bool layout(const lbm_params* p, const Geo& g, Layout* L) {
   L->toff = off;     off = align_up(off + (size_t)(nt ? nt + 1 : 0) * 4, A);
   L->tcnt = off;     off = align_up(off + (size_t)nt * 8, A);
   L->twork = off;    off = align_up(off + (size_t)(uses_tma(p) ? nt : 0) * 16, A);
-  const int64_t nh = uses_halo(p) ? halo_tile_count(g) : 0;
-  L->hent = off;     off = align_up(off + (size_t)nh * HALO_RS * 2, A);
-  L->hoff = off;     off = align_up(off + (size_t)(nh ? nh + 1 : 0) * 4, A);
-  L->hcnt = off;     off = align_up(off + (size_t)nh * 16, A);
-  L->hmask = off;    off = align_up(off + (size_t)nh * HALO_MW * 4, A);
+  // per 32 x 14 cells: 1520 + 4 + 16 + 96 bytes
+  const int64_t nh = uses_halo(p) ? ((int64_t)((g.nx + 31) / 32) * ((g.ny + 13) / 14)) : 0;
+  L->hlists = off;
+  off = align_up(off + (size_t)nh * 1520, A);
+  off = align_up(off + (size_t)(nh ? nh + 1 : 0) * 4, A);
+  off = align_up(off + (size_t)nh * 16, A);
+  off = align_up(off + (size_t)nh * 96, A);
+  L->hend = off;
   L->counts = off;   off = align_up(off + (size_t)scan_blocks * 4, A);
   L->small = off;    off = align_up(off + 64, A);
   L->partial = off;  off = align_up(off + 2 * MASS_BLOCKS * 8, A);
@@ -170,10 +172,11 @@ lbm_status check_cuda(lbm_ctx* c, cudaError_t e, const char* where) {
   return LBM_ERR_CUDA;
 }
 
-// The TMA schedule's bounded waits set small[4] when a copy was not seen to
-// complete; synchronising calls report it (and clear it).
+// The bounded waits of the TMA and halo schedules set small[4] when a copy was
+// not seen to complete; synchronising calls report it (and clear it).
 lbm_status check_timeout(lbm_ctx* c) {
-  if (!c->tma) return LBM_OK;
+  if (!c->tma && !c->halo_used) return LBM_OK;
+  c->halo_used = false;
   int v = 0;
   lbm_status s = check_cuda(c, cudaMemcpyAsync(&v, c->small + 4, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
                             "cudaMemcpyAsync");
@@ -181,7 +184,7 @@ lbm_status check_timeout(lbm_ctx* c) {
   if (s) return s;
   if (v) {
     s = check_cuda(c, cudaMemsetAsync(c->small + 4, 0, sizeof(int), c->stream), "cudaMemsetAsync");
-    return s ? s : fail(c, LBM_ERR_TIMEOUT, "a TMA copy of the tiled step did not complete within its bounded wait");
+    return s ? s : fail(c, LBM_ERR_TIMEOUT, "a TMA copy of a step did not complete within its bounded wait");
   }
   return LBM_OK;
 }
@@ -207,6 +210,35 @@ lbm_status launch(lbm_ctx* c, int cls, const char* where, Fn&& fn) {
 }
 
 }  // namespace
+
+// Per-tile lists of the tiled schedule for the installed geometry: counts,
+// offsets (fixed-order scan, total at tile_off[n_tiles]), entries. AUTO keeps
+// room for them and builds them when a batch runs its tiled schedule. The TMA
+// schedule's work list is read back (synchronises).
+lbm_status build_tile_lists(lbm_ctx* c, cudaStream_t stream) {
+  const Geo& g = c->g;
+  const int ntx = (g.nx + TILE_W - 1) / TILE_W;
+  const int nt = (int)c->n_tiles;
+  lbm_status s;
+  k_tile_lists<<<nt, TILE_LIST_THREADS, 0, stream>>>(c->flags, g, ntx, nullptr, c->tile_off, c->tile_cnt, nullptr);
+  if ((s = after_launch(c, "k_tile_lists(count)"))) return s;
+  k_iface_scan<<<1, 1024, 0, stream>>>(c->tile_off, nt, c->tile_off + nt);
+  if ((s = after_launch(c, "k_iface_scan(tiles)"))) return s;
+  k_tile_lists<<<nt, TILE_LIST_THREADS, 0, stream>>>(c->flags, g, ntx, c->tile_off, nullptr, nullptr, c->tile_entries);
+  if ((s = after_launch(c, "k_tile_lists(write)"))) return s;
+  if (c->tile_work) {
+    // the tiles with owned nodes, in order
+    k_tile_work<<<1, 1024, 0, stream>>>(c->tile_cnt, c->tile_off, nt, c->tile_work, c->small + 5);
+    if ((s = after_launch(c, "k_tile_work"))) return s;
+    int nw = 0;
+    s = check_cuda(c, cudaMemcpyAsync(&nw, c->small + 5, sizeof(int), cudaMemcpyDeviceToHost, stream), "cudaMemcpyAsync");
+    if (!s) s = check_cuda(c, cudaStreamSynchronize(stream), "cudaStreamSynchronize");
+    if (s) return s;
+    c->n_work = nw;
+  }
+  c->tiles_built = true;
+  return LBM_OK;
+}
 
 // Before work that reads the density planes under a scheme without virtual
 // densities: zero the rho~ an earlier scheme of this context left in them.
@@ -408,42 +440,140 @@ lbm_status step_tiled16(lbm_ctx* c, int nsteps) {
   return LBM_OK;
 }
 
-// Per-tile lists of the halo schedule for the current geometry: counts and
-// fluid bitmasks, offsets (fixed-order scan, total at halo_off[n_halo_tiles]),
-// entries. Built by lbm_set_geometry for HALO, at the first halo step for AUTO.
+// Tensor map of `planes` planes of the padded grid whose nodes are
+// `node_bytes` wide, with the box of a halo tile's window (HaloSmem: R rings,
+// H owned rows, O more columns on each side).
+bool encode_halo_map(CUtensorMap* map, const Geo& g, void* base, int node_bytes, int planes, int R, int O, int H) {
+  EncodeTiledFn enc = encode_tiled();
+  if (!enc) return false;
+  const cuuint32_t m = node_bytes > 8 ? node_bytes / 8 : 1;  // elements per node
+  const cuuint64_t dim[3] = {(cuuint64_t)m * g.px, (cuuint64_t)g.py, (cuuint64_t)planes};
+  const cuuint64_t str[2] = {(cuuint64_t)node_bytes * g.px, (cuuint64_t)node_bytes * g.plane};
+  const cuuint32_t box[3] = {(cuuint32_t)(m * (HALO_W + 2 * O)), (cuuint32_t)(H + 2 * (R + 1)), 1};
+  const cuuint32_t ones[3] = {1, 1, 1};
+  return enc(map, node_bytes >= 8 ? CU_TENSOR_MAP_DATA_TYPE_UINT64 : CU_TENSOR_MAP_DATA_TYPE_UINT32, planes > 1 ? 3 : 2,
+             base, dim, str, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Tensor maps of the halo schedule: both population buffers, and the planes
+// that hold their references (16-bit storage), for one and three rings.
+bool encode_halo_maps(lbm_ctx* c) {
+  const int es = (int)elem_size(c->prm.storage);
+  for (int r = 0; r < 2; ++r)
+    for (int b = 0; b < 2; ++b) {
+      const int R = r ? 3 : 1, O = es == 2 ? 4 : R + 1, H = halo_rows(es);
+      if (!encode_halo_map(&c->hmap_f[r][b], c->g, c->f[b], 2 * es, 9, R, O, H)) return false;
+      if (es == 2 && !(c->Ubuf[0] ? encode_halo_map(&c->hmap_ref[r][b], c->g, c->Ubuf[b], (int)sizeof(UPair), 1, R, O, H)
+                                  : encode_halo_map(&c->hmap_ref[r][b], c->g, c->Pbuf[b], 8, 1, R, O, H)))
+        return false;
+    }
+  return true;
+}
+
+// Whether the context steps (or, in a batch, may step) by the halo schedule.
+bool wants_halo(const lbm_ctx* c) {
+  return c->prm.kernel == LBM_KERNEL_HALO ||
+         (c->prm.kernel == LBM_KERNEL_AUTO && c->prm.storage != LBM_STORE_FP64);
+}
+
+// The halo schedule's lists for the installed geometry, in the unused parts
+// of the workspace: behind the interface cells (their arrays have room for
+// every node) and in the area halo contexts keep. Leaves halo_ready false,
+// and the two-pass schedule runs instead, if they do not fit. Synchronises.
 lbm_status build_halo_lists(lbm_ctx* c) {
   const Geo& g = c->g;
+  c->halo_ready = false;
+  if (!c->hmaps_ok || c->n_fluid == 0) return LBM_OK;
   const int ntx = (g.nx + HALO_W - 1) / HALO_W;
-  const int nt = (int)c->n_halo_tiles;
+  const int H = halo_rows((int)elem_size(c->prm.storage));
+  const int64_t nt = halo_tile_count(g, H);
+  if (nt * HALO_RW * (H + 6) > 0x7fffffff) return LBM_OK;  // 32-bit places in the lists
+  char* from[2] = {(char*)align_up((size_t)(c->iface_mask + c->n_iface), 256), c->halo_area[0]};
+  char* const end[2] = {c->iface_end, c->halo_area[1]};
+  auto take = [&](size_t bytes) -> char* {
+    for (int r = 1; r >= 0; --r)
+      if (from[r] < end[r] && (size_t)(end[r] - from[r]) >= bytes) {
+        char* p = from[r];
+        from[r] = (char*)align_up((size_t)(p + bytes), 256);
+        return p;
+      }
+    return nullptr;
+  };
+  HaloTile* work = (HaloTile*)take((size_t)nt * sizeof(HaloTile));
+  int* off[3];  // entries, cells, work list
+  for (int i = 0; i < 3; ++i)
+    if (!(off[i] = (int*)take((size_t)nt * 4))) return LBM_OK;
+  if (!work) return LBM_OK;
   lbm_status s;
-  k_halo_lists<<<nt, HALO_LIST_THREADS, 0, c->stream>>>(c->flags, g, ntx, nullptr, c->halo_off, c->halo_cnt,
-                                                        c->halo_fmask, nullptr);
+  k_halo_lists<<<(unsigned)nt, HALO_LIST_THREADS, 0, c->stream>>>(c->flags, g, ntx, H, off[0], off[1], off[2], nullptr,
+                                                                  nullptr, nullptr);
   if ((s = after_launch(c, "k_halo_lists(count)"))) return s;
-  k_iface_scan<<<1, 1024, 0, c->stream>>>(c->halo_off, nt, c->halo_off + nt);
-  if ((s = after_launch(c, "k_iface_scan(halo)"))) return s;
-  k_halo_lists<<<nt, HALO_LIST_THREADS, 0, c->stream>>>(c->flags, g, ntx, c->halo_off, nullptr, nullptr, nullptr,
-                                                        c->halo_entries);
+  for (int i = 0; i < 3; ++i) {
+    k_iface_scan<<<1, 1024, 0, c->stream>>>(off[i], (int)nt, c->small + 6 + i);
+    if ((s = after_launch(c, "k_iface_scan(halo)"))) return s;
+  }
+  int h[3];
+  s = check_cuda(c, cudaMemcpyAsync(h, c->small + 6, sizeof(h), cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync");
+  if (!s) s = check_cuda(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+  if (s) return s;
+  uint32_t* entries = (uint32_t*)take((size_t)h[0] * 4);
+  uint2* cells = (uint2*)take((size_t)(h[1] > 0 ? h[1] : 1) * 8);
+  if (!entries || !cells) return LBM_OK;
+  k_halo_lists<<<(unsigned)nt, HALO_LIST_THREADS, 0, c->stream>>>(c->flags, g, ntx, H, off[0], off[1], off[2], work,
+                                                                  entries, cells);
   if ((s = after_launch(c, "k_halo_lists(write)"))) return s;
-  c->halo_built = true;
+  c->halo = HaloLists{work, h[2], entries, cells};
+  c->halo_ready = true;
   return LBM_OK;
 }
 
+template <typename T, int R, bool VR>
+lbm_status launch_halo(lbm_ctx* c, const T* fin, T* fout, typename Pop<T>::C* P) {
+  using C = typename Pop<T>::C;
+  using S = HaloSmem<T, R, VR>;
+  auto kern = k_halo<T, R, VR>;
+  bool& set = c->halo_smem_set[R == 3];
+  if (!set) {
+    lbm_status s = check_cuda(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::BYTES),
+                              "cudaFuncSetAttribute");
+    if (s) return s;
+    set = true;
+  }
+  const int r = R == 3 ? 1 : 0;
+  const CUtensorMap& mref = kDev<T> ? c->hmap_ref[r][c->Ubuf[0] ? c->cur : c->pcur] : c->hmap_f[r][c->cur];
+  return launch(c, LBM_KC_FUSED, "k_halo", [&] {
+    kern<<<c->halo.n_work, halo_threads<T>, S::BYTES, c->stream>>>(
+        c->hmap_f[r][c->cur], mref, fout, StorePtrs<T>(fout, c->g), P, c->Ubuf[c->cur ^ 1], c->halo, c->g, (c->g.nx + HALO_W - 1) / HALO_W,
+        kphys<C>(c->ph), c->small + 4, c->tma_extra_tx);
+  });
+}
+
 // Halo schedule: one kernel per step, densities recomputed per tile from the
-// populations (no density plane).
+// populations. 16-bit storage: the spare density plane takes rho(t), the
+// references of the populations the step writes; the planes then swap roles
+// as in the two-pass schedule.
 template <typename T>
 lbm_status step_halo(lbm_ctx* c, int nsteps) {
+  using C = typename Pop<T>::C;
+  const bool three = halo_reach(c->ph) == 3;
   for (int t = 0; t < nsteps; ++t) {
     const T* fin = (const T*)c->f[c->cur];
     T* fout = (T*)c->f[c->cur ^ 1];
-    lbm_status ls = LBM_OK;
-    lbm_status s = launch(c, LBM_KC_FUSED, "k_halo", [&] {
-      ls = launch_halo<T>(c->g, c->ph, fin, fout, c->flags, c->halo_entries, c->halo_off, c->halo_cnt,
-                          c->halo_fmask, c->stream);
-    });
-    if (ls) return fail(c, ls, "halo kernel launch rejected");
+    C* P = (C*)c->Pbuf[c->pcur ^ 1];
+    lbm_status s;
+    if (kDev<T> && c->prm.velocity_refs)
+      s = three ? launch_halo<T, 3, kDev<T>>(c, fin, fout, P) : launch_halo<T, 1, kDev<T>>(c, fin, fout, P);
+    else
+      s = three ? launch_halo<T, 3, false>(c, fin, fout, P) : launch_halo<T, 1, false>(c, fin, fout, P);
     if (s) return s;
     c->cur ^= 1;
     c->p_valid = false;
+    c->halo_used = true;
+    if (kDev<T>) {
+      c->pcur ^= 1;
+      c->P = c->Pbuf[c->pcur];
+    }
   }
   return LBM_OK;
 }
@@ -454,26 +584,17 @@ lbm_status do_step(lbm_ctx* c, int nsteps) {
     lbm_status s = clear_virtual(c, c->stream);
     if (s) return s;
   }
+  const int k = c->prm.kernel;
+  // AUTO with FP64 storage: bound by the FP64 pipe, so the schedule that
+  // sums and updates every node once. Before the update's operations were
+  // halved too, 100 x 50 took 20.5 us per step against 61 for the single
+  // passes, 800 x 600 207 against 298 us, 1400 x 1000 553 against 701 us.
+  const bool halo = k == LBM_KERNEL_HALO || (k == LBM_KERNEL_AUTO && sizeof(T) != 8);
+  if (halo && c->halo_ready) return step_halo<T>(c, nsteps);
   if constexpr (sizeof(T) >= 4) {  // the marching kernel stores 4- and 8-byte populations only
-    // AUTO with FP64 storage: bound by the FP64 pipe, so the schedule that
-    // updates every node once (the single passes update a tile's ring again):
-    // before the update's operations were halved too, 100 x 50 took 20.5
-    // against 61 us per step, 800 x 600 207 against 298 us, 1400 x 1000 553
-    // against 701 us
-    if (sizeof(T) == 8 && c->prm.kernel == LBM_KERNEL_AUTO) return step_two_pass<T>(c, nsteps);
-    // HALO always; AUTO under the one-node-reach schemes (the improved
-    // scheme's Eq. 8 reaches three rings, where the tiled schedule wins)
-    const bool halo = c->prm.kernel == LBM_KERNEL_HALO || (c->prm.kernel == LBM_KERNEL_AUTO && c->ph.bc != BC_VAVG);
-    if (halo && c->n_halo_tiles > 0) {
-      if (!c->halo_built) {
-        lbm_status s = build_halo_lists(c);
-        if (s) return s;
-      }
-      return step_halo<T>(c, nsteps);
-    }
-    if (c->prm.kernel == LBM_KERNEL_FUSED && fused_supported<T>(c->g, c->ph)) return step_fused<T>(c, nsteps);
-    const bool tiled = c->prm.kernel == LBM_KERNEL_TILED || c->prm.kernel == LBM_KERNEL_AUTO || c->prm.kernel == LBM_KERNEL_TMA;
-    if (tiled && c->n_tiles > 0) return step_fused<T>(c, nsteps);
+    if (k == LBM_KERNEL_FUSED && fused_supported<T>(c->g, c->ph)) return step_fused<T>(c, nsteps);
+    if ((k == LBM_KERNEL_TILED || k == LBM_KERNEL_TMA) && c->n_tiles > 0)
+      return step_fused<T>(c, nsteps);
   } else {
     if (c->Pbuf[2] && c->n_tiles > 0) return step_tiled16<T>(c, nsteps);
   }
@@ -622,11 +743,9 @@ lbm_status lbm_create(const lbm_params* params, void* d_workspace, size_t bytes,
   c->tile_off = c->n_tiles ? (int*)(c->ws + L.toff) : nullptr;
   c->tile_cnt = c->n_tiles ? (int2*)(c->ws + L.tcnt) : nullptr;
   c->tile_work = c->n_tiles && uses_tma(params) ? (int4*)(c->ws + L.twork) : nullptr;
-  c->n_halo_tiles = uses_halo(params) ? halo_tile_count(g) : 0;
-  c->halo_entries = c->n_halo_tiles ? (uint16_t*)(c->ws + L.hent) : nullptr;
-  c->halo_off = c->n_halo_tiles ? (int*)(c->ws + L.hoff) : nullptr;
-  c->halo_cnt = c->n_halo_tiles ? (int4*)(c->ws + L.hcnt) : nullptr;
-  c->halo_fmask = c->n_halo_tiles ? (uint32_t*)(c->ws + L.hmask) : nullptr;
+  c->halo_area[0] = c->ws + L.hlists;
+  c->halo_area[1] = c->ws + L.hend;
+  c->iface_end = c->ws + L.flist;
   c->scan_counts = (int*)(c->ws + L.counts);
   c->small = (int*)(c->ws + L.small);
   c->partial = (double*)(c->ws + L.partial);
@@ -654,6 +773,7 @@ lbm_status lbm_create(const lbm_params* params, void* d_workspace, size_t bytes,
                          "cudaDeviceGetAttribute");
   if (!s) s = check_cuda(c, cudaMemsetAsync(c->ws, 0, L.total, c->stream), "cudaMemsetAsync");
   if (!s && c->tma && !encode_tma_maps(c)) s = LBM_ERR_CUDA;
+  if (!s) c->hmaps_ok = encode_halo_maps(c);  // without them the two-pass schedule runs
   if (s) {
     delete c;
     return s;
@@ -706,37 +826,16 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const uint8_t* d_mask) {
   if (h[1] > c->if_capacity) return fail(c, LBM_ERR_SPACE, "interface-solid list exceeds max_interface");
   c->n_iface = h[1];
   c->n_fluid = h[2];
+  c->iface_mask = (uint32_t*)align_up((size_t)(c->iface_list + c->n_iface), 256);
   if (c->n_iface > 0) {
     k_iface_mask<<<(c->n_iface + 127) / 128, 128, 0, c->stream>>>(c->flags, c->iface_list, c->n_iface, g,
                                                                   c->iface_mask);
     if ((s = after_launch(c, "k_iface_mask"))) return s;
   }
-  if (c->n_tiles > 0) {
-    // per-tile lists of the tiled schedule: counts, offsets (fixed-order
-    // scan, total at tile_off[n_tiles]), entries
-    const int ntx = (g.nx + TILE_W - 1) / TILE_W;
-    const int nt = (int)c->n_tiles;
-    k_tile_lists<<<nt, TILE_LIST_THREADS, 0, c->stream>>>(c->flags, g, ntx, nullptr, c->tile_off, c->tile_cnt, nullptr);
-    if ((s = after_launch(c, "k_tile_lists(count)"))) return s;
-    k_iface_scan<<<1, 1024, 0, c->stream>>>(c->tile_off, nt, c->tile_off + nt);
-    if ((s = after_launch(c, "k_iface_scan(tiles)"))) return s;
-    k_tile_lists<<<nt, TILE_LIST_THREADS, 0, c->stream>>>(c->flags, g, ntx, c->tile_off, nullptr, nullptr,
-                                                     c->tile_entries);
-    if ((s = after_launch(c, "k_tile_lists(write)"))) return s;
-    if (c->tile_work) {
-      // the TMA schedule's work list: the tiles with owned nodes, in order
-      k_tile_work<<<1, 1024, 0, c->stream>>>(c->tile_cnt, c->tile_off, nt, c->tile_work, c->small + 5);
-      if ((s = after_launch(c, "k_tile_work"))) return s;
-      int nw = 0;
-      s = check_cuda(c, cudaMemcpyAsync(&nw, c->small + 5, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
-                     "cudaMemcpyAsync");
-      if (!s) s = check_cuda(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-      if (s) return s;
-      c->n_work = nw;
-    }
-  }
-  c->halo_built = false;
-  if (c->n_halo_tiles > 0 && c->prm.kernel == LBM_KERNEL_HALO && (s = build_halo_lists(c))) return s;
+  c->tiles_built = false;
+  if (c->n_tiles > 0 && c->prm.kernel != LBM_KERNEL_AUTO && (s = build_tile_lists(c, c->stream))) return s;
+  c->halo_ready = false;
+  if (wants_halo(c) && (s = build_halo_lists(c))) return s;
   c->has_geometry = true;
   return LBM_OK;
 }

@@ -336,17 +336,18 @@ template <typename T>
 lbm_status batch_step(lbm_batch* b, int nsteps) {
   using C = typename Pop<T>::C;
   fill_descs<C>(b);
+  const bool tiled = b->schedule == LBM_KERNEL_TILED;
   for (int s = 0; s < b->n && nsteps > 0; ++s) {
     lbm_ctx* c = b->ctx[s];
     lbm_status cs = clear_virtual(c, b->stream);
     if (cs) return bfail(b, cs, c->err);
     if (c->ph.bc == BC_VAVG && c->n_iface > 0) c->virt_written = true;
+    if (tiled && !c->tiles_built && (cs = build_tile_lists(c, b->stream))) return bfail(b, cs, c->err);
   }
   lbm_status st = bcuda(b, cudaMemcpyAsync(b->d_desc, b->h_desc, (size_t)b->n * sizeof(BatchDesc<C>),
                                            cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
   // the staging buffer is rewritten by the next call: wait for the copy
   if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
-  const bool tiled = b->schedule == LBM_KERNEL_TILED;
   if (!st && tiled && nsteps > 0) {
     // the tiled step reads rho(t) from Pbuf[pcur]: compute it for every
     // member once (a member whose plane already holds it gets the same bits)

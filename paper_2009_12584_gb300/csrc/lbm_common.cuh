@@ -138,6 +138,9 @@ struct Pop;
 template <>
 struct Pop<float> {
   using C = float;
+  using V = float2;  // both components as stored
+  static __device__ __forceinline__ float2 unpack(float2 v, float, float) { return v; }
+  static __device__ __forceinline__ float2 pack(float a, float b, float, float) { return make_float2(a, b); }
   static __device__ __forceinline__ float ld(const float* p, int64_t k, float) { return p[k]; }
   static __device__ __forceinline__ void st(float* p, int64_t k, float v, float) { p[k] = v; }
   static __device__ __forceinline__ float enc(float v, float) { return v; }
@@ -154,6 +157,9 @@ struct Pop<float> {
 template <>
 struct Pop<double> {
   using C = double;
+  using V = double2;
+  static __device__ __forceinline__ double2 unpack(double2 v, double, double) { return v; }
+  static __device__ __forceinline__ double2 pack(double a, double b, double, double) { return make_double2(a, b); }
   static __device__ __forceinline__ double ld(const double* p, int64_t k, double) { return p[k]; }
   static __device__ __forceinline__ void st(double* p, int64_t k, double v, double) { p[k] = v; }
   static __device__ __forceinline__ double enc(double v, double) { return v; }
@@ -179,6 +185,13 @@ constexpr float HALF_SCALE = 4096.0f, HALF_UNSCALE = 1.0f / 4096.0f;
 template <>
 struct Pop<__half> {
   using C = float;
+  using V = __half2;
+  static __device__ __forceinline__ float2 unpack(__half2 v, float ra, float rb) {
+    return make_float2(fmaf(__low2float(v), HALF_UNSCALE, ra), fmaf(__high2float(v), HALF_UNSCALE, rb));
+  }
+  static __device__ __forceinline__ __half2 pack(float a, float b, float ra, float rb) {
+    return __floats2half2_rn(__fsub_rn(a, ra) * HALF_SCALE, __fsub_rn(b, rb) * HALF_SCALE);
+  }
   static __device__ __forceinline__ float ld(const __half* p, int64_t k, float ref) {
     return fmaf(__half2float(p[k]), HALF_UNSCALE, ref);
   }
@@ -199,6 +212,13 @@ struct Pop<__half> {
 template <>
 struct Pop<__nv_bfloat16> {
   using C = float;
+  using V = __nv_bfloat162;
+  static __device__ __forceinline__ float2 unpack(__nv_bfloat162 v, float ra, float rb) {
+    return make_float2(__fadd_rn(__low2float(v), ra), __fadd_rn(__high2float(v), rb));
+  }
+  static __device__ __forceinline__ __nv_bfloat162 pack(float a, float b, float ra, float rb) {
+    return __floats2bfloat162_rn(__fsub_rn(a, ra), __fsub_rn(b, rb));
+  }
   static __device__ __forceinline__ float ld(const __nv_bfloat16* p, int64_t k, float ref) {
     return __fadd_rn(__bfloat162float(p[k]), ref);
   }
@@ -215,6 +235,24 @@ struct Pop<__nv_bfloat16> {
   }
   static __device__ __forceinline__ void st2(__nv_bfloat16* p, int64_t j, float a, float b, float ra, float rb) {
     *reinterpret_cast<__nv_bfloat162*>(p + j) = __floats2bfloat162_rn(__fsub_rn(a, ra), __fsub_rn(b, rb));
+  }
+};
+
+// Where a step stores: the nine planes' base addresses, and those of the slots
+// x - c_i, formed on the host. As kernel parameters they sit in constant
+// memory, so that a store's address is one multiply-add of the node's padded
+// index k.
+template <typename T>
+struct StorePtrs {
+  char *own[9], *bounce[9];
+  StorePtrs(T* f, const Geo& g) {
+    for (int i = 0; i < 9; ++i) {
+      own[i] = (char*)(f + pslot(g, i, 0));
+      bounce[i] = (char*)(f + pslot(g, i, 0)) - (int64_t)(cx_of(i) + cy_of(i) * g.px) * 2 * (int64_t)sizeof(T);
+    }
+  }
+  static __device__ __forceinline__ void st(char* base, uint32_t k, typename Pop<T>::V v) {
+    *(typename Pop<T>::V*)(base + (uint64_t)k * (2 * sizeof(T))) = v;
   }
 };
 
@@ -270,26 +308,32 @@ inline PhysK<C> kphys(const Phys& p) {
   return k;
 }
 
-// 36 sum_i w_i c_i phi(x + c_i) for the eight neighbour bits of a node's
-// flags: small integers, exact in either type. One 8-byte load (2 KB table,
-// resident in L1) in place of eight selects and a weighted sum.
+// sum_i w_i c_i phi(x + c_i) for the eight neighbour bits of a node's flags,
+// in FP32 as the paired arithmetic forms it (a multiple of fl(1/9) plus one
+// of fl(1/36), rounded once) and as the integer 36 sum_i w_i c_i phi. One
+// 8-byte load (2 KB tables, resident in L1) in place of eight selects and a
+// weighted sum.
 struct WallPush {
-  float2 v[256];
-  constexpr WallPush() : v() {
+  float2 w[256], w36[256];
+  constexpr WallPush() : w(), w36() {
+    constexpr double A = (double)(1.0f / 9.0f), D = (double)(1.0f / 36.0f);
     for (int m = 0; m < 256; ++m) {
-      int sx = 0, sy = 0;
+      int ax = 0, ay = 0, dx = 0, dy = 0;
       for (int i = 1; i < 9; ++i)
         if (m >> (i - 1) & 1) {
-          sx += (i <= 4 ? 4 : 1) * cx_of(i);
-          sy += (i <= 4 ? 4 : 1) * cy_of(i);
+          (i <= 4 ? ax : dx) += cx_of(i);
+          (i <= 4 ? ay : dy) += cy_of(i);
         }
-      v[m].x = (float)sx;
-      v[m].y = (float)sy;
+      w[m].x = (float)(ax * A + dx * D);
+      w[m].y = (float)(ay * A + dy * D);
+      w36[m].x = (float)(4 * ax + dx);
+      w36[m].y = (float)(4 * ay + dy);
     }
   }
 };
 static __device__ const WallPush WALL_PUSH = WallPush();
-__device__ __forceinline__ float2 wall_push(uint16_t fl) { return __ldg(&WALL_PUSH.v[(fl >> 1) & 0xFF]); }
+__device__ __forceinline__ float2 wall_push(uint16_t fl) { return __ldg(&WALL_PUSH.w[(fl >> 1) & 0xFF]); }
+__device__ __forceinline__ float2 wall_push36(uint16_t fl) { return __ldg(&WALL_PUSH.w36[(fl >> 1) & 0xFF]); }
 
 // 36 sum_i w_i c_i q_i over the eight moving directions (q[0] unused).
 template <typename C>
@@ -325,7 +369,7 @@ __device__ __forceinline__ void interaction_force(const PhysK<C>& ph, uint16_t f
       }
       return;
     }
-    const float2 v = wall_push(fl);
+    const float2 v = wall_push36(fl);
     const C vx = C(v.x), vy = C(v.y);
 #pragma unroll
     for (int s = 0; s < 2; ++s) {

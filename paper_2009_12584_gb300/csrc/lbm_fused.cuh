@@ -64,6 +64,33 @@ __device__ __forceinline__ void march_update(C fv[2][9], const C nbP[2][9], uint
   }
 }
 
+// march_update on component pairs (fp, q: pairs of the compute type).
+template <typename C>
+__device__ __forceinline__ void update_pairs(typename CPair<C>::V fp[9], const typename CPair<C>::V q[9], uint16_t fl,
+                                             bool general, const PhysK<C>& ph, C rho_out[2], C u_out[2]) {
+  if constexpr (sizeof(C) == 4) {
+    const float2 r = general ? update_pair<true>(fp, q, fl, ph, u_out[0], u_out[1])
+                             : update_pair<false>(fp, q, fl, ph, u_out[0], u_out[1]);
+    rho_out[0] = r.x;
+    rho_out[1] = r.y;
+  } else {
+    C fv[2][9], nb[2][9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      fv[0][i] = fp[i].x;
+      fv[1][i] = fp[i].y;
+      nb[0][i] = q[i].x;
+      nb[1][i] = q[i].y;
+    }
+    update_node<C>(fv, nb, fl, general, ph, rho_out, u_out);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      fp[i].x = fv[0][i];
+      fp[i].y = fv[1][i];
+    }
+  }
+}
+
 // Neighbour value along x from the lane's own column value: lanes 1 ... 31
 // take it from the lane to the left (dx = -1) or right (dx = +1); the outer
 // lanes use the value they loaded for the column beyond the warp.

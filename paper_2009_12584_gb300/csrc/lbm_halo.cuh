@@ -1,31 +1,34 @@
-// Halo-tiled single-pass step: one kernel per time step and no density
-// plane (4- and 8-byte storage).
+// Halo-tiled single-pass step: one kernel per time step, every population
+// crosses HBM once, and (4- and 8-byte storage) no density plane.
 //
 // The step needs rho(t) at a fluid node's eight neighbours (Eq. 5) and,
 // under the improved scheme, rho~(t) at its solid neighbours, which Eq. 8
 // averages from rho(t) up to two nodes further out. Both are recomputed per
-// tile from the populations themselves: one CTA takes a HALO_W x HALO_H
-// tile and
-//   phase A: pulls f_i(x) = f*_i(x - c_i, t) at every fluid node of the tile
-//     and of the R rings around it (R = 3 for the D2Q25 average of Eq. 8,
-//     2 for the D2Q9 average, 1 for the other schemes) and keeps
-//     rho(t) = sum_i f_i (Eq. 3) in shared memory;
-//   phase B (improved scheme only): evaluates Eq. 8 at the interface-solid
-//     cells of the tile and its first ring from those densities;
-//   phase C: each fluid node of the tile pulls its populations again (now
-//     L1/L2 hits), takes rho or rho~ of its neighbours from shared memory,
-//     evaluates Eqs. 5 and 7, u of Eq. 3 and the collision (Eqs. 1, 2, 4),
-//     and stores f*(t+1) (with bounced slots and periodic images).
-// The ring nodes cost nine pulls and a sum each, not a collision; the
-// populations cross HBM once per step. Every value is computed with the
-// arithmetic, in the order, of the two-pass schedule, so the schedules agree
-// bit for bit.
+// tile from the populations themselves. One CTA takes a HALO_W x HALO_H
+// tile. Its inputs arrive by the Tensor Memory Accelerator: the nine
+// population planes over the tile's window, R + 1 nodes wider on each side
+// (nine 3-D boxes), the encoding references there (16-bit storage: one 2-D
+// box) and the tile's node list (one bulk copy), all counted on one
+// mbarrier. No load holds registers or is addressed by the threads, and
+// three or four CTAs per SM overlap one's copies with the others' updates.
+// Out of shared memory,
+//   phase A: rho(t) = sum_i f_i (Eq. 3), f_i(x) = f*_i(x - c_i, t), at every
+//     fluid node of the tile and of the R rings around it (R = 3 under the
+//     improved scheme, 1 otherwise);
+//   phase V (improved scheme): Eq. 8 at the interface-solid cells of the
+//     tile and its first ring (the other schemes keep 0 there);
+//   phase B: each node of the tile evaluates Eqs. 5 and 7, u of Eq. 3 and
+//     the collision (Eqs. 1, 2, 4) and stores f*(t+1) to HBM (with bounced
+//     slots and periodic images; with 16-bit storage also the references of
+//     what it stores).
+// Every value is computed with the arithmetic, in the order, of the two-pass
+// schedule, so the schedules agree bit for bit.
 //
-// Fluid nodes are listed per tile at set-up: the tile's own nodes first, then
-// the rings by distance, each in row order (16-bit entries: the slot in the
-// (HALO_W + 2 HALO_R) x (HALO_H + 2 HALO_R) region and two tags). A per-tile
-// bitmask of the region's fluid slots gives phase B the fluid neighbours of
-// each solid cell.
+// Lists of a geometry, per tile: its fluid nodes (own nodes, then ring 1,
+// then rings 2 and 3, each in row order), an entry holding the node's place
+// in the window, its eight solid-neighbour bits and a border tag; and its
+// interface-solid cells within ring 1 with their fluid neighbours (Eq. 8's
+// 5 x 5 bits).
 #pragma once
 
 #include "lbm.h"
@@ -33,98 +36,94 @@
 #include "lbm_fused.cuh"
 #include "lbm_geometry.cuh"
 #include "lbm_kernels.cuh"
+#include "lbm_tma.cuh"
 
 namespace lbm {
 
-#ifndef LBM_HALO_W
-#define LBM_HALO_W 32
-#endif
-#ifndef LBM_HALO_H
-#define LBM_HALO_H 14
-#endif
-// 128-thread CTAs, 8 per SM: on the 8192^2 porous medium 2.09 ms per step
-// against 2.34 ms with 256 threads at 4 per SM (improved scheme; Martys-Chen
-// 1.59 against 1.68 ms)
-#ifndef LBM_HALO_THREADS
-#define LBM_HALO_THREADS 128
-#endif
-#ifndef LBM_HALO_MINB
-#define LBM_HALO_MINB 8
-#endif
-#ifndef LBM_HALO_AHEAD
-#define LBM_HALO_AHEAD 512
-#endif
-constexpr int HALO_R = 3;  // widest halo: Eq. 8's D2Q25 reach (2) plus the force's (1)
-constexpr int HALO_W = LBM_HALO_W, HALO_H = LBM_HALO_H;  // owned nodes per tile
-constexpr int HALO_RW = HALO_W + 2 * HALO_R;  // region pitch
-constexpr int HALO_RH = HALO_H + 2 * HALO_R;
-constexpr int HALO_RS = HALO_RW * HALO_RH;    // region slots
-constexpr int HALO_MW = (HALO_RS + 31) / 32;  // words of a tile's fluid bitmask
-constexpr int HALO_THREADS = LBM_HALO_THREADS;
-constexpr int HALO_MINB = LBM_HALO_MINB;      // CTAs per SM the registers must allow
-constexpr int HALO_AHEAD = LBM_HALO_AHEAD;    // tiles between a CTA and the one whose entries it prefetches
-constexpr int HALO_LIST_THREADS = 256;        // k_halo_lists
-static_assert(HALO_RS <= 2048, "slots must fit the 11 slot bits of an entry");
-static_assert(HALO_MW <= HALO_THREADS, "one thread per bitmask word");
+constexpr int HALO_W = 32;  // owned columns of a tile
+// Owned rows and threads: three windows of three rings, or four of one ring,
+// fill an SM's shared memory, and the threads take the tile's own nodes of a
+// porous medium (60% fluid) in about one round at 64 to 96 registers each.
+// 4096^2 porous, us per step, improved scheme / LLKC: FP32 with 14 rows and
+// 224 threads 406 / 363 (256 threads 411 / 363, 12 rows 429 / 371, 16 rows
+// 480 / 383); FP16 with 20 rows and 256 threads 376 / 337 (16 rows 400 / 346,
+// 24 rows 356 / 352, and with velocity references 450 against 478 and 515).
+constexpr int HALO_H = 14, HALO_H16 = 20;
+template <typename T>
+constexpr int halo_h = sizeof(T) == 2 ? HALO_H16 : HALO_H;
+__host__ __device__ inline int halo_rows(int elem_size) { return elem_size == 2 ? HALO_H16 : HALO_H; }
+constexpr int HALO_O = 4;                        // entries count columns and rows from (x0 - 4, y0 - 4)
+template <typename T>
+constexpr int halo_threads = sizeof(T) == 2 ? 256 : 224;
+constexpr int HALO_AHEAD = 512;  // CTAs between one and that whose record it asks L2 for
+constexpr int HALO_LIST_THREADS = 256;
+constexpr int HALO_RW = HALO_W + 6;              // region of the lists: the tile and three rings
+static_assert(HALO_H + 2 * HALO_O <= 32 && HALO_H16 + 2 * HALO_O <= 32, "entries: 6 column bits, 5 row bits");
 
-constexpr uint16_t HE_SLOT = 0x07FFu;     // slot = row * HALO_RW + col in the region
-constexpr uint16_t HE_SOLIDNB = 0x2000u;  // own node with a solid D2Q9 neighbour
-constexpr uint16_t HE_BORDER = 0x4000u;   // own node within GH + 1 of a periodic border
+// List entry: column (bits 0-5) and row (6-10) from (x0 - 4, y0 - 4),
+// solid-neighbour bits 1 ... 8 of the flags (11-18), border tag.
+constexpr int HE_NB_SHIFT = 10;
+constexpr uint32_t HE_BORDER = 1u << 19;  // own node within GH + 1 of a periodic border
 
-inline int64_t halo_tile_count(const Geo& g) {
-  return (int64_t)((g.nx + HALO_W - 1) / HALO_W) * ((g.ny + HALO_H - 1) / HALO_H);
+inline int64_t halo_tile_count(const Geo& g, int H) {
+  return (int64_t)((g.nx + HALO_W - 1) / HALO_W) * ((g.ny + H - 1) / H);
 }
-
 // Rings a step needs for the installed wetting scheme.
-inline int halo_reach(const Phys& ph) { return ph.bc == BC_VAVG ? (ph.avg9 ? 2 : 3) : 1; }
+inline int halo_reach(const Phys& ph) { return ph.bc == BC_VAVG ? 3 : 1; }
 
-// Ring of region slot (col, row) of a tile with tw x th owned nodes: 0 for
-// an owned slot, else its distance (max norm) from the owned rectangle; -1
-// outside the region.
-__device__ __forceinline__ int halo_ring(int col, int row, int tw, int th) {
-  if (col > tw + 2 * HALO_R - 1 || row > th + 2 * HALO_R - 1) return -1;
-  const int dc = col < HALO_R ? HALO_R - col : (col >= HALO_R + tw ? col - (HALO_R + tw - 1) : 0);
-  const int dr = row < HALO_R ? HALO_R - row : (row >= HALO_R + th ? row - (HALO_R + th - 1) : 0);
-  return max(dc, dr);
+// A tile that owns fluid nodes: its counts (own nodes, + ring 1, + rings 2
+// and 3, interface-solid cells), its first entry (a multiple of 4: bulk
+// copies start on 16 bytes) and first cell, and its number.
+struct alignas(32) HaloTile {
+  int4 n;
+  int e0, i0, tile, pad;
+};
+struct HaloLists {
+  const HaloTile* work;  // in tile order
+  int n_work;
+  const uint32_t* entries;
+  const uint2* cells;  // (place in the window as in an entry, 5 x 5 fluid bits)
+};
+
+// Fluid neighbours of the cell at padded index k (k_iface_mask's bits).
+__device__ __forceinline__ uint32_t fluid_mask25(const uint16_t* __restrict__ flags, const Geo& g, int k) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int dy = -2; dy <= 2; ++dy)
+#pragma unroll
+    for (int dx = -2; dx <= 2; ++dx)
+      if ((dx != 0 || dy != 0) && !(flags[k + dx + dy * g.px] & F_SOLID)) m |= 1u << ((dy + 2) * 5 + (dx + 2));
+  return m;
 }
 
-// Per-tile lists, two passes over the same deterministic order (four
-// rounds: the owned nodes, then rings 1, 2, 3). Count pass (entries ==
-// nullptr): totals[tile] = fluid nodes of the region, cnt[tile] = the
-// cumulative counts after each round, fmask[tile] = the region's fluid
-// bitmask. Write pass: the entries from offsets[tile] on.
+// One CTA per tile, two passes over the same fixed order. Count pass
+// (entries == nullptr): the tile's sizes and whether it owns nodes, which the
+// scans turn into offsets and places in the work list. Write pass: work list,
+// entries and cells.
 static __global__ void __launch_bounds__(HALO_LIST_THREADS)
-    k_halo_lists(const uint16_t* __restrict__ flags, Geo g, int ntx, const int* __restrict__ offsets,
-                 int* __restrict__ totals, int4* __restrict__ cnt, uint32_t* __restrict__ fmask,
-                 uint16_t* __restrict__ entries) {
+    k_halo_lists(const uint16_t* __restrict__ flags, Geo g, int ntx, int H, int* __restrict__ eoff, int* __restrict__ ioff,
+                 int* __restrict__ woff, HaloTile* __restrict__ work, uint32_t* __restrict__ entries,
+                 uint2* __restrict__ cells) {
   __shared__ int warp_cnt[HALO_LIST_THREADS / 32];
   const int tile = blockIdx.x;
-  const int x0 = (tile % ntx) * HALO_W, y0 = (tile / ntx) * HALO_H;
-  const int tw = min(HALO_W, g.nx - x0), th = min(HALO_H, g.ny - y0);
+  const int x0 = (tile % ntx) * HALO_W, y0 = (tile / ntx) * H;
+  const int tw = min(HALO_W, g.nx - x0), th = min(H, g.ny - y0), RS = HALO_RW * (H + 6);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int base = 0;
   int cum[4];
-  for (int round = 0; round < 4; ++round) {
-    for (int c0 = 0; c0 < HALO_RS; c0 += HALO_LIST_THREADS) {
+  for (int round = 0; round < 4; ++round) {  // own nodes, ring 1, rings 2 and 3, interface-solid cells
+    if (round == 3) base = 0;
+    for (int c0 = 0; c0 < RS; c0 += HALO_LIST_THREADS) {
       const int slot = c0 + threadIdx.x;
       const int row = slot / HALO_RW, col = slot - row * HALO_RW;
-      const int ring = slot < HALO_RS ? halo_ring(col, row, tw, th) : -1;
-      bool fluid = false;
-      uint16_t e = 0;
-      if (ring >= 0) {
-        const int x = x0 - HALO_R + col, y = y0 - HALO_R + row;
-        const uint16_t fl = flags[g.idx(x, y)];
-        fluid = !(fl & F_SOLID);
-        e = (uint16_t)slot;
-        if (ring == 0 && (fl & NB_ANY)) e |= HE_SOLIDNB;
-        if (ring == 0 && near_border(g, x, y)) e |= HE_BORDER;
-      }
-      if (round == 0 && !entries) {
-        const unsigned bits = __ballot_sync(0xffffffffu, fluid);
-        const int word = (c0 >> 5) + wid;
-        if (lane == 0 && word < HALO_MW) fmask[(int64_t)tile * HALO_MW + word] = bits;
-      }
-      const bool hit = fluid && ring == round;
+      // distance (max norm) from the owned rectangle
+      const int dc = col < 3 ? 3 - col : (col >= 3 + tw ? col - (2 + tw) : 0);
+      const int dr = row < 3 ? 3 - row : (row >= 3 + th ? row - (2 + th) : 0);
+      const int ring = slot < RS ? max(dc, dr) : 99;
+      const int x = x0 - 3 + col, y = y0 - 3 + row;
+      const uint16_t fl = ring <= 3 ? flags[g.idx(x, y)] : F_SOLID;
+      const int cls = ring >= 2 ? 2 : ring;
+      const bool hit = round == 3 ? ring <= 1 && (fl & F_IFACE) : !(fl & F_SOLID) && cls == round;
       const unsigned ball = __ballot_sync(0xffffffffu, hit);
       if (lane == 0) warp_cnt[wid] = __popc(ball);
       __syncthreads();
@@ -134,160 +133,239 @@ static __global__ void __launch_bounds__(HALO_LIST_THREADS)
         before += w < wid ? v : 0;
         all += v;
       }
-      if (entries && hit) entries[offsets[tile] + base + before + __popc(ball & ((1u << lane) - 1u))] = e;
+      if (entries && hit && (round == 0 || cum[0] > 0)) {
+        const int pos = base + before + __popc(ball & ((1u << lane) - 1u));
+        uint32_t e = (uint32_t)(col + 1) | (uint32_t)(row + 1) << 6;
+        if (round == 3) {
+          cells[ioff[tile] + pos] = make_uint2(e, fluid_mask25(flags, g, g.idx(x, y)));
+        } else {
+          e |= (uint32_t)(fl & NB_ANY) << HE_NB_SHIFT;
+          if (ring == 0 && near_border(g, x, y)) e |= HE_BORDER;
+          entries[eoff[tile] + pos] = e;
+        }
+      }
       base += all;
       __syncthreads();
     }
     cum[round] = base;
   }
-  if (!entries && threadIdx.x == 0) {
-    totals[tile] = base;
-    cnt[tile] = make_int4(cum[0], cum[1], cum[2], cum[3]);
+  if (threadIdx.x == 0) {
+    if (!entries) {
+      eoff[tile] = cum[0] > 0 ? (cum[2] + 3) & ~3 : 0;
+      ioff[tile] = cum[0] > 0 ? cum[3] : 0;
+      woff[tile] = cum[0] > 0;
+    } else if (cum[0] > 0) {
+      work[woff[tile]] = HaloTile{make_int4(cum[0], cum[1], cum[2], cum[3]), eoff[tile], ioff[tile], tile, 0};
+    }
   }
 }
 
-// One CTA per tile. reach: the rings phase A covers (halo_reach).
-template <typename T>
-__global__ void __launch_bounds__(HALO_THREADS, HALO_MINB)
-    k_halo(const T* __restrict__ f, T* __restrict__ fo, const uint16_t* __restrict__ flags,
-           const uint16_t* __restrict__ entries, const int* __restrict__ offsets, const int4* __restrict__ cnt,
-           const uint32_t* __restrict__ fmask, Geo g, int ntx, int reach, PhysK<typename Pop<T>::C> ph) {
+// Shared memory of a CTA, in bytes from a 128-byte boundary.
+template <typename T, int R, bool VR>
+struct HaloSmem {
+  using C = typename Pop<T>::C;
+  // the window: R + 1 more nodes on each side, with 16-bit storage four more
+  // columns whatever R (copies start on 16 bytes)
+  static constexpr int H = halo_h<T>, O = kDev<T> ? 4 : R + 1, P = HALO_W + 2 * O;
+  static constexpr int ROWS = H + 2 * (R + 1), CELLS = P * ROWS;
+  static constexpr int pad(int n) { return (n + 127) / 128 * 128; }
+  static constexpr int FBYTES = CELLS * 2 * (int)sizeof(T), FSLOT = pad(FBYTES);
+  static constexpr int RBYTES = kDev<T> ? CELLS * (VR ? (int)sizeof(UPair) : 2 * (int)sizeof(C)) : 0;
+  static constexpr int REF = 9 * FSLOT, RHO = REF + pad(RBYTES), ENT = RHO + pad(CELLS * 2 * (int)sizeof(C));
+  static constexpr int BYTES = ENT + pad((HALO_W + 2 * R) * (H + 2 * R) * 4 + 16) + 128;
+};
+
+// mapf: tensor map of the populations (pairs; x in units of Pop<T>::V, FP64 of
+// 8 bytes), with a box of one tile's window; mapref: of the references. P: the
+// density plane that takes rho(t), the references of what a 16-bit step
+// stores. err: set to 1
+// when the copies were not seen to complete within the bound (the CTA then
+// stops, and those that start later do nothing); extra_tx: see tma_issue. FP64 is bound by its arithmetic, not by
+// the one CTA per SM that its windows allow.
+template <typename T, int R, bool VR>
+__global__ void __launch_bounds__(halo_threads<T>, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
+    k_halo(const __grid_constant__ CUtensorMap mapf, const __grid_constant__ CUtensorMap mapref, T* __restrict__ fo,
+           const __grid_constant__ StorePtrs<T> out, typename Pop<T>::C* __restrict__ P, UPair* __restrict__ Uo, HaloLists L, Geo g, int ntx,
+           PhysK<typename Pop<T>::C> ph, int* __restrict__ err, uint32_t extra_tx) {
   using C = typename Pop<T>::C;
   using V = typename CPair<C>::V;
-  static_assert(!kDev<T>, "the halo schedule stores 4- and 8-byte populations");
-  __shared__ V rho[HALO_RS];       // rho(t) at fluid slots, rho~(t) at interface-solid slots
-  __shared__ uint32_t fm[HALO_MW];  // fluid slots of the region
-  const int tile = blockIdx.x;
-  const int4 cn = cnt[tile];
-  const int n_own = cn.x;
-  if (n_own == 0) return;  // the whole CTA: nothing owned, nothing to store
-  const int n_a = reach <= 1 ? cn.y : (reach == 2 ? cn.z : cn.w);
-  const int e0 = offsets[tile];
-  // the entries are the first load of every node and its pulls depend on
-  // them: ask L2 for those of the tile HALO_AHEAD launches later
-  constexpr int ENTRY_LINES = (HALO_RS + 63) / 64;
-  static_assert(ENTRY_LINES <= HALO_THREADS, "one thread per line");
-  if (threadIdx.x < ENTRY_LINES && tile + HALO_AHEAD < (int)gridDim.x) {
-    const int e1 = __ldg(offsets + tile + HALO_AHEAD);
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(entries + e1 + threadIdx.x * 64));
+  using S = HaloSmem<T, R, VR>;
+  constexpr int NT = halo_threads<T>;
+  constexpr uint32_t FB = 2 * sizeof(T);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t bar;
+  unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+  V* rho = (V*)(sm + S::RHO);
+  const uint32_t* ent = (const uint32_t*)(sm + S::ENT);
+  const int tid = threadIdx.x;
+  const HaloTile* item = L.work + blockIdx.x;
+  if (tid == 0) {
+    mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  const bool vavg = ph.bc == BC_VAVG;
-  if (vavg && threadIdx.x < HALO_MW) fm[threadIdx.x] = __ldg(fmask + (int64_t)tile * HALO_MW + threadIdx.x);
-  const int x0 = (tile % ntx) * HALO_W, y0 = (tile / ntx) * HALO_H;
-  const int korg = g.idx(x0 - HALO_R, y0 - HALO_R);  // padded index of slot 0
-  if (sizeof(C) == 8 && !vavg) {
-    // the schemes without virtual densities read 0 at solid slots
-    for (int w = threadIdx.x >> 5; w < HALO_MW; w += HALO_THREADS / 32) {
-      const uint32_t bits = __ldg(fmask + (int64_t)tile * HALO_MW + w);
-      const int slot = w * 32 + (threadIdx.x & 31);
-      V z;
-      z.x = z.y = C(0);
-      if (slot < HALO_RS && !(bits >> (threadIdx.x & 31) & 1u)) rho[slot] = z;
-    }
-  }
-  const C zr[2][9] = {};  // storage references: unused for 4- and 8-byte populations
-
-  // phase A: rho(t) of the tile and its rings
-  for (int t = threadIdx.x; t < n_a; t += HALO_THREADS) {
-    const int slot = __ldg(entries + e0 + t) & HE_SLOT;
-    const int row = slot / HALO_RW, col = slot - row * HALO_RW;
-    const int k = korg + row * g.px + col;
-    C fv[2][9];
-    gather<T>(f, g, k, zr, fv);
-    V v;
-    v.x = density(fv[0]);
-    v.y = density(fv[1]);
-    rho[slot] = v;
-  }
-  __syncthreads();
-
-  // phase B: Eq. 8 at the interface-solid cells of the tile and its first
-  // ring (the solid neighbours of the owned nodes); it reads the densities
-  // of fluid slots only and writes solid slots only
-  if (vavg) {
-    const int tw = min(HALO_W, g.nx - x0), th = min(HALO_H, g.ny - y0);
-    const int cw = tw + 2, ch = th + 2;
-    auto fluid = [&](int s) { return (fm[s >> 5] >> (s & 31)) & 1u; };
-    for (int j = threadIdx.x; j < cw * ch; j += HALO_THREADS) {
-      const int row = HALO_R - 1 + j / cw, col = HALO_R - 1 + j % cw;
-      const int slot = row * HALO_RW + col;
-      if (fluid(slot)) continue;
-      uint32_t msk = 0;
-      bool iface = false;
+  const int4 cn = __ldg(&item->n), it = __ldg((const int4*)&item->e0);
+  if (*(volatile int*)err) return;  // the whole CTA, or it waits (bounded) like the ones before it
+  const int n_own = cn.x, n_a = R == 1 ? cn.y : cn.z, n_if = cn.w, i0 = it.y, tile = it.z;
+  const int x0 = (tile % ntx) * HALO_W, y0 = (tile / ntx) * S::H;
+  if (tid == 0) {
+    // the window's first node: column x0 - O + LP (a multiple of 4 nodes with
+    // 16-bit storage, of 2 otherwise: 16-byte aligned), row y0 - (R + 1) + GH
+    const int xw = x0 - S::O + LP, yw = y0 - (R + 1) + GH;
+    const uint32_t ebytes = (uint32_t)((n_a + 3) & ~3) * 4;
+    mbar_expect_tx(&bar, 9u * S::FBYTES + S::RBYTES + ebytes + extra_tx);
+    bulk_load(sm + S::ENT, L.entries + it.x, ebytes, &bar);
 #pragma unroll
-      for (int dy = -2; dy <= 2; ++dy)
+    for (int i = 0; i < 9; ++i) tma_load_3d(sm + i * S::FSLOT, &mapf, sizeof(T) == 8 ? 2 * xw : xw, yw, i, &bar);
+    if (kDev<T>) tma_load_2d(sm + S::REF, &mapref, VR ? 2 * xw : xw, yw, &bar);
+  }
+  if (tid == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(item + HALO_AHEAD));
+  // this thread's interface-solid cell, needed after phase A
+  uint2 cell = make_uint2(0, 0);
+  if (tid < n_if) cell = __ldg(L.cells + i0 + tid);
+  // An entry's node in the window held in shared memory, and in cells of
+  // the padded grid from the entries' node (0, 0).
+  auto place = [](uint32_t e) {
+    return (int)(e >> 6 & 31u) * S::P + (int)(e & 63u) - ((3 - R) * S::P + HALO_O - S::O);
+  };
+  auto cells = [&](uint32_t e) { return (e >> 6 & 31u) * (uint32_t)g.px + (e & 63u); };
+  // Post-streaming populations of the node at window place w.
+  auto gather_node = [&](int w, uint16_t fl, V fp[9]) {
+    const typename Pop<T>::V* win = (const typename Pop<T>::V*)sm;
 #pragma unroll
-        for (int dx = -2; dx <= 2; ++dx) {
-          if (dx == 0 && dy == 0) continue;
-          if (fluid(slot + dx + dy * HALO_RW)) {
-            msk |= 1u << ((dy + 2) * 5 + (dx + 2));
-            if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) iface = true;
-          }
+    for (int i = 0; i < 9; ++i) {
+      const int up = -(cx_of(i) + cy_of(i) * S::P);  // to x - c_i
+      const auto v = win[i * (S::FSLOT / (int)FB) + w + up];
+      C ra = C(0), rb = C(0);
+      if constexpr (kDev<T>) {
+        // the writer: x - c_i, or the node itself where that is solid (its
+        // bounced value, sent along -c_i)
+        const bool back = i != 0 && (fl & nb_bit(opp_of(i)));
+        const int m = back ? w : w + up;
+        if constexpr (VR) {
+          const UVal u = u_unpack(((const UPair*)(sm + S::REF))[m]);
+          const float ca = cdot(i, u.v[0]), cb = cdot(i, u.v[1]);
+          ra = ref_of(i, u.r[0], back ? -ca : ca);
+          rb = ref_of(i, u.r[1], back ? -cb : cb);
+        } else {
+          const V r = ((const V*)(sm + S::REF))[m];
+          ra = w_of<C>(i) * r.x;
+          rb = w_of<C>(i) * r.y;
         }
-      if (!iface) continue;
+      }
+      fp[i] = Pop<T>::unpack(v, ra, rb);
+    }
+  };
+
+  __syncthreads();  // the barrier is initialised
+  bool ok = mbar_wait(&bar, 0);
+  if (!ok) ok = mbar_wait(&bar, 0);  // the copies in flight, once more
+
+  // phase A
+  if (ok) {
+    for (int t = tid; t < n_a; t += NT) {
+      const uint32_t e = ent[t];
+      const int w = place(e);
+      V fp[9];
+      gather_node(w, (e >> HE_NB_SHIFT) & NB_ANY, fp);
+      rho[w] = density_pair(fp);
+    }
+    if (R == 1)
+      for (int t = tid; t < n_if; t += NT) {
+        V z;
+        z.x = z.y = C(0);
+        rho[place(t == tid ? cell.x : __ldg(L.cells + i0 + t).x)] = z;
+      }
+  }
+  if (__syncthreads_or(!ok)) {
+    if (tid == 0) atomicExch(err, 1);
+    return;
+  }
+
+  // phase V
+  if (R == 3) {
+    for (int t = tid; t < n_if; t += NT) {
+      const uint2 cl = t == tid ? cell : __ldg(L.cells + i0 + t);
+      const int w = place(cl.x);
       auto load = [&](int dx, int dy, C& a, C& b) {
-        const V v = rho[slot + dx + dy * HALO_RW];
+        const V v = rho[w + dx + dy * S::P];
         a = v.x;
         b = v.y;
       };
       V v;
       if (ph.avg9)
-        virtual_density_at<C, true>(msk, ph, load, v.x, v.y);
+        virtual_density_at<C, true, 1>(cl.y, ph, load, v.x, v.y);
       else
-        virtual_density_at<C, false>(msk, ph, load, v.x, v.y);
-      rho[slot] = v;
+        virtual_density_at<C, false, 1>(cl.y, ph, load, v.x, v.y);
+      rho[w] = v;
     }
     __syncthreads();
   }
 
-  // phase C: force, velocity, collision and stores of the owned nodes
-  for (int b = 0; b < n_own; b += HALO_THREADS) {
-    const int t = b + threadIdx.x;
-    const bool valid = t < n_own;
-    const uint16_t e = valid ? __ldg(entries + e0 + t) : uint16_t(0);
-    const bool warp_edge = __any_sync(0xffffffffu, (e & HE_SOLIDNB) != 0);
+  // phase B
+  const int korg = g.idx(x0 - HALO_O, y0 - HALO_O);  // padded index of the entries' node (0, 0)
+  for (int b = 0; b < n_own; b += NT) {
+    const bool valid = b + tid < n_own;
+    const uint32_t e = valid ? ent[b + tid] : 0u;
+    const uint16_t fl = (e >> HE_NB_SHIFT) & NB_ANY;
+    const bool warp_edge = __any_sync(0xffffffffu, fl != 0);
     const bool warp_border = __any_sync(0xffffffffu, (e & HE_BORDER) != 0);
     if (!valid) continue;
-    const int slot = e & HE_SLOT;
-    const int row = slot / HALO_RW, col = slot - row * HALO_RW;
-    const int k = korg + row * g.px + col;
-    const uint16_t fl = warp_edge ? __ldg(flags + k) : uint16_t(0);
-    C fv[2][9];
-    gather<T>(f, g, k, zr, fv);
-    C nbP[2][9];
-    nbP[0][0] = nbP[1][0] = C(0);
+    const int w = place(e);
+    const uint32_t kp = (uint32_t)korg + cells(e);  // padded index
+    V fp[9], q[9];
+    gather_node(w, fl, fp);
+    q[0].x = q[0].y = C(0);
 #pragma unroll
-    for (int i = 1; i < 9; ++i) {
-      const V v = rho[slot + cx_of(i) + cy_of(i) * HALO_RW];
-      nbP[0][i] = v.x;
-      nbP[1][i] = v.y;
+    for (int i = 1; i < 9; ++i) q[i] = rho[w + cx_of(i) + cy_of(i) * S::P];
+    C ref[2][9], rh[2], u[2];
+    UVal U{};
+    update_pairs<C>(fp, q, fl, warp_edge, ph, rh, u);
+    const int x = x0 - HALO_O + (int)(e & 63u), y = y0 - HALO_O + (int)(e >> 6 & 31u);
+    if constexpr (kDev<T>) {
+      // the references of what this node stores, for its readers
+      const V rv = f2(rh[0], rh[1]);
+      UPair up{};
+      if constexpr (VR) {
+        // momentum of each component's post-collision populations
+        const float2 d57 = sub2(fp[5], fp[7]), d86 = sub2(fp[8], fp[6]);
+        up = u_pack(add2(sub2(fp[1], fp[3]), add2(d57, d86)), add2(sub2(fp[2], fp[4]), sub2(d57, d86)), rv);
+        U = u_unpack(up);
+        Uo[kp] = up;
+      } else {
+        stP(P, kp, rh[0], rh[1]);
+      }
+      if (warp_border) {
+        for_ghost_images(g, x, y, [&](int kk) {
+          if constexpr (VR)
+            Uo[kk] = up;
+          else
+            stP(P, kk, rh[0], rh[1]);
+        });
+      }
     }
-    C rh[2], uu[2];
-    march_update<C>(fv, nbP, fl, warp_edge, ph, rh, uu);
+    write_refs<T>(rh, VR, U, ref);
     if (!warp_border) {
 #pragma unroll
-      for (int i = 0; i < 9; ++i) Pop<T>::st2(fo, pslot(g, i, k), fv[0][i], fv[1][i], C(0), C(0));
-      if (warp_edge) store_bounced_near(fo, g, k, fl, fv, zr);
+      for (int i = 0; i < 9; ++i) out.st(out.own[i], kp, Pop<T>::pack(fp[i].x, fp[i].y, ref[0][i], ref[1][i]));
+      if (warp_edge) {
+        // the solid neighbours are owned nodes without images: slot i of x - c_i
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+          const int o = opp_of(i);
+          if (fl & nb_bit(o)) out.st(out.bounce[i], kp, Pop<T>::pack(fp[o].x, fp[o].y, ref[0][o], ref[1][o]));
+        }
+      }
     } else {
-      const int x = x0 - HALO_R + col, y = y0 - HALO_R + row;
-      store_node(fo, g, x, y, k, fv, zr);
-      store_bounced(fo, g, x, y, fl, fv, zr);
+      C fv[2][9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        fv[0][i] = fp[i].x;
+        fv[1][i] = fp[i].y;
+      }
+      store_node(fo, g, x, y, (int)kp, fv, ref);
+      store_bounced(fo, g, x, y, fl, fv, ref);
     }
-  }
-}
-
-template <typename T>
-inline lbm_status launch_halo(const Geo& g, const Phys& ph, const T* fin, T* fout, const uint16_t* flags,
-                              const uint16_t* entries, const int* offsets, const int4* cnt, const uint32_t* fmask,
-                              cudaStream_t stream) {
-  if constexpr (kDev<T>) {
-    return LBM_ERR_ARG;
-  } else {
-    const int ntx = (g.nx + HALO_W - 1) / HALO_W;
-    const int64_t nt = halo_tile_count(g);
-    k_halo<T><<<(unsigned)nt, HALO_THREADS, 0, stream>>>(fin, fout, flags, entries, offsets, cnt, fmask, g, ntx,
-                                                         halo_reach(ph), kphys<typename Pop<T>::C>(ph));
-    return LBM_OK;
   }
 }
 

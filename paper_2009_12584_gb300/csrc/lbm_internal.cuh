@@ -20,6 +20,10 @@ struct lbm_ctx {
   // (rank 2), encoded at creation
   alignas(64) CUtensorMap tmap_f[2];
   alignas(64) CUtensorMap tmap_P[2];
+  // halo schedule: maps of f[0], f[1] and of the planes with their
+  // references (16-bit storage), boxes for one ring [0] and three rings [1]
+  alignas(64) CUtensorMap hmap_f[2][2];
+  alignas(64) CUtensorMap hmap_ref[2][2];
   bool tma;            // the TMA schedule runs (FP32 storage, LBM_KERNEL_TMA)
   bool tma_smem_set;   // k_tile_tma's dynamic shared memory limit raised
   lbm_params prm;
@@ -45,7 +49,8 @@ struct lbm_ctx {
   bool p_valid;        // P holds the densities of the current state (single-pass)
   uint16_t* flags;
   int* iface_list;
-  uint32_t* iface_mask; // fluid neighbours of each interface-solid cell (5 x 5 stencil bits)
+  uint32_t* iface_mask; // fluid neighbours of each interface-solid cell (5 x 5 stencil bits), behind
+                        // iface_list
   int* fluid_list;     // fluid nodes in node order, edge nodes tagged (padded indices)
   uint16_t* tile_entries; // tiled schedule: per-tile lists of region slots (null if unused)
   int* tile_off;       // tiled schedule: first entry of each tile, total at [ntiles]
@@ -56,13 +61,15 @@ struct lbm_ctx {
   int64_t n_tiles;
   bool tile_smem_set;  // k_tile's dynamic shared memory limit raised on this context's device
   bool march_smem_set;  // k_march's (FP64: above 48 KB) likewise
-  bool halo_built;      // the halo lists match the current geometry
+  bool tiles_built;     // the tiled schedule's lists match the current geometry
+  bool halo_used;       // a halo step ran since the last look at the error word
+  bool halo_ready;      // the halo schedule's lists match the current geometry
+  bool hmaps_ok;        // its tensor maps are encoded
+  bool halo_smem_set[2];  // k_halo's dynamic shared memory limit raised (one ring, three rings)
   uint32_t tma_extra_tx;  // test hook of the TMA schedule's bounded wait (lbm_debug_tma_expect_extra); 0
-  uint16_t* halo_entries; // halo schedule: per-tile lists of region slots (null if unused)
-  int* halo_off;       // halo schedule: first entry of each tile, total at [n_halo_tiles]
-  int4* halo_cnt;      // halo schedule: cumulative counts (own, +ring 1, +ring 2, +ring 3) per tile
-  uint32_t* halo_fmask; // halo schedule: fluid bitmask of each tile's region
-  int64_t n_halo_tiles;
+  lbm::HaloLists halo;  // halo schedule: per-tile lists, placed by lbm_set_geometry
+  char* halo_area[2];  // an area of the workspace for these lists (may be empty)
+  char* iface_end;     // end of the interface arrays, whose unused part also holds them
   int* scan_counts;    // per-block interface counts / offsets
   int* small;          // [0] error count, [1] interface total, [2] fluid total
   double* partial;     // mass partial sums
@@ -90,3 +97,5 @@ struct lbm_ctx {
 // Zero the rho~ that an earlier improved-scheme step left in the density
 // planes when the installed scheme has none (lbm_api.cu).
 lbm_status clear_virtual(lbm_ctx* c, cudaStream_t stream);
+// The tiled schedule's lists of the installed geometry (lbm_api.cu).
+lbm_status build_tile_lists(lbm_ctx* c, cudaStream_t stream);

@@ -414,22 +414,32 @@ __device__ __forceinline__ void ldP_line(const C* __restrict__ P, int64_t k, C& 
 // neighbour (dx, dy); the sums run in a fixed order, so every caller (the
 // plane-based pass and the shared-memory pass of the halo schedule) gets
 // the same bits.
-template <typename C, bool AVG9, typename Load>
+// ROWS: rows of the stencil whose loads go out together: all of them for
+// loads from memory (one round trip), one at a time out of shared memory
+// (registers).
+template <typename C, bool AVG9, int ROWS = 5, typename Load>
 __device__ __forceinline__ void virtual_density_at(uint32_t msk, const PhysK<C>& ph, Load&& load, C& v0, C& v1) {
   constexpr int REACH = AVG9 ? 1 : 2;
   constexpr int NB = (2 * REACH + 1) * (2 * REACH + 1);
   C p0[NB], p1[NB];
-#pragma unroll
-  for (int dy = -REACH; dy <= REACH; ++dy)
+  auto load_row = [&](int dy) {
 #pragma unroll
     for (int dx = -REACH; dx <= REACH; ++dx) {
       const int j = (dy + REACH) * (2 * REACH + 1) + (dx + REACH);
       p0[j] = p1[j] = C(0);
       if ((msk >> ((dy + 2) * 5 + (dx + 2))) & 1u) load(dx, dy, p0[j], p1[j]);
     }
+  };
+  if (ROWS >= 5)
+#pragma unroll
+    for (int dy = -REACH; dy <= REACH; ++dy) load_row(dy);
   C num0 = 0, num1 = 0, den = 0;
 #pragma unroll
-  for (int dy = -REACH; dy <= REACH; ++dy)
+  for (int dy = -REACH; dy <= REACH; ++dy) {
+    if (ROWS < 5) {
+      load_row(dy);
+      asm volatile("" ::: "memory");  // the next row's loads stay behind this row's
+    }
 #pragma unroll
     for (int dx = -REACH; dx <= REACH; ++dx) {
       if (dx == 0 && dy == 0) continue;
@@ -446,6 +456,7 @@ __device__ __forceinline__ void virtual_density_at(uint32_t msk, const PhysK<C>&
       num1 += fluid ? w * p1[j] : C(0);
       den += fluid ? w : C(0);
     }
+  }
   v0 = ph.chi[0] * num0 / den;
   v1 = ph.chi[1] * num1 / den;
 }

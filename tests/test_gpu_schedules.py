@@ -59,3 +59,72 @@ def test_fp64_auto_matches_tiled(nx, ny):
     b.step(4)
     assert torch.equal(a.populations(), b.populations())
     assert np.all(np.isfinite(a.mass()))
+
+
+# Tile edges of the halo schedule: 32 columns, 14 rows (20 with 16-bit
+# storage), one tile, one node more, a ragged last tile, windows that reach
+# across a whole small periodic box.
+@pytest.mark.parametrize("storage,vref", [("fp32", False), ("fp64", False), ("fp16", False), ("bf16", False),
+                                          ("fp16", True), ("bf16", True)])
+@pytest.mark.parametrize("nx,ny", [(4, 4), (32, 14), (33, 15), (32, 20), (65, 41), (100, 61), (31, 13)])
+@pytest.mark.parametrize("periodic", [True, False])
+@pytest.mark.parametrize("scheme", ["improved", "improved_d2q9_self", "llkc", "constant"])
+def test_halo_matches_two_pass_bitwise(storage, vref, nx, ny, periodic, scheme):
+    wet = {"improved": IMPROVED,
+           "improved_d2q9_self": ("virtual_avg", dict(G_s=(2.5, 3.5), chi=(0.9, 1.3), pairing=lbm.PAIR_SELF,
+                                                      avg_stencil=9))}.get(scheme) or SCHEMES[scheme]
+    mask = inputs.random_solid_mask(nx, ny, seed=nx + ny, fraction=0.12, periodic_x=periodic, periodic_y=periodic)
+    rA, rB, ux, uy = inputs.random_fields(nx, ny, 11, umax=0.05)
+    out = []
+    for kernel in ("two_pass", "halo"):
+        sim = lbm.Simulation(nx, ny, storage=storage, velocity_refs=vref, kernel=kernel, periodic_x=periodic,
+                             periodic_y=periodic)
+        sim.set_geometry(mask).set_wetting(wet[0], **wet[1]).init_fields(rA, rB, ux, uy)
+        sim.step(3)
+        m = sim.moments()  # in the middle: the next steps start from the same state
+        sim.step(4)
+        sim.sync()
+        out.append([*m, sim.populations(), torch.from_numpy(sim.mass())])
+        sim.close()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+
+
+def test_halo_without_room_for_its_lists_runs_two_pass():
+    """A workspace with a small interface list leaves no room for the lists
+    of a 16-bit context: the same results, by the two-pass schedule."""
+    nx, ny = 96, 70
+    mask = inputs.flat_wall_mask(nx, ny)
+    rA, rB, ux, uy = inputs.random_fields(nx, ny, 2, umax=0.05)
+    out = []
+    for cap in (0, 2 * nx):
+        sim = lbm.Simulation(nx, ny, storage="fp16", kernel="halo", periodic_x=True, max_interface=cap)
+        sim.set_geometry(mask).set_wetting(IMPROVED[0], **IMPROVED[1]).init_fields(rA, rB, ux, uy)
+        n0 = sim.launch_count
+        sim.step(5)
+        out.append((sim.launch_count - n0, sim.populations()))
+        sim.close()
+    assert out[0][0] == 5 and out[1][0] == 15  # one launch a step; density, Eq. 8, collide
+    assert torch.equal(out[0][1], out[1][1])
+
+
+def test_halo_wait_runs_out_and_context_recovers():
+    """A tile whose copies do not complete within the bound is reported, later
+    steps do nothing until then, and the context steps on afterwards."""
+    nx, ny = 70, 50
+    mask = inputs.inclined_wall_mask(nx, ny, 20.0, 9)
+    rA, rB = inputs.sharp_droplet(nx, ny, nx / 2, ny / 2, 9)
+    sims = []
+    for kernel in ("halo", "two_pass"):
+        sim = lbm.Simulation(nx, ny, kernel=kernel)
+        sims.append(sim.set_geometry(mask).set_wetting(IMPROVED[0], **IMPROVED[1]).init_fields(rA, rB))
+    sims[0].step(2).debug_tma_expect_extra(16)
+    sims[0].step(3)
+    with pytest.raises(lbm.LbmError) as e:
+        sims[0].sync()
+    assert e.value.status == lbm.ERR_TIMEOUT
+    sims[0].debug_tma_expect_extra(0).sync()
+    sims[0].init_fields(rA, rB).step(7)
+    sims[1].step(7)
+    sims[0].sync()
+    assert torch.equal(sims[0].populations(), sims[1].populations())
