@@ -387,8 +387,11 @@ lbm_status lbm_field_mass_noalloc(const double* d_rhoA, const double* d_rhoB,
  * and size, all of the same storage type on one device) advance together:
  * each step is one launch per kernel class over all of them, and repeated
  * steps replay a CUDA graph (kernel nodes, one per launch; the batch is not
- * one persistent kernel). Two schedules: TWO_PASS (density, Eq. 8 and
- * collide launches over the members' fluid lists, any storage) and TILED
+ * one persistent kernel). Two schedules: TWO_PASS, the list schedule (members
+ * with FP32 or 16-bit storage created with LBM_KERNEL_AUTO or
+ * LBM_KERNEL_HALO step by the halo kernel, one launch for those whose step
+ * needs one ring and one for those that need three; the others by density,
+ * Eq. 8 and collide launches over their fluid lists) and TILED
  * (the Eq. 8 launch and one tiled single-pass launch over all members'
  * 32 x 14 tiles; 4- and 8-byte storage, members created with
  * LBM_KERNEL_AUTO or LBM_KERNEL_TILED so that they keep tile lists). The batch keeps pointers to the contexts; they

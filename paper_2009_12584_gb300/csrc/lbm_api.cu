@@ -529,8 +529,7 @@ lbm_status build_halo_lists(lbm_ctx* c) {
 }
 
 template <typename T, int R, bool VR>
-lbm_status launch_halo(lbm_ctx* c, const T* fin, T* fout, typename Pop<T>::C* P) {
-  using C = typename Pop<T>::C;
+lbm_status launch_halo(lbm_ctx* c) {
   using S = HaloSmem<T, R, VR>;
   auto kern = k_halo<T, R, VR>;
   bool& set = c->halo_smem_set[R == 3];
@@ -540,12 +539,11 @@ lbm_status launch_halo(lbm_ctx* c, const T* fin, T* fout, typename Pop<T>::C* P)
     if (s) return s;
     set = true;
   }
-  const int r = R == 3 ? 1 : 0;
-  const CUtensorMap& mref = kDev<T> ? c->hmap_ref[r][c->Ubuf[0] ? c->cur : c->pcur] : c->hmap_f[r][c->cur];
+  const CUtensorMap* mf = &c->hmap_f[R == 3][c->cur];
+  const CUtensorMap* mr = kDev<T> ? &c->hmap_ref[R == 3][c->Ubuf[0] ? c->cur : c->pcur] : mf;
+  const HaloArgs<T> a = halo_args<T>(c, c->cur, c->pcur);
   return launch(c, LBM_KC_FUSED, "k_halo", [&] {
-    kern<<<c->halo.n_work, halo_threads<T>, S::BYTES, c->stream>>>(
-        c->hmap_f[r][c->cur], mref, fout, StorePtrs<T>(fout, c->g), P, c->Ubuf[c->cur ^ 1], c->halo, c->g, (c->g.nx + HALO_W - 1) / HALO_W,
-        kphys<C>(c->ph), c->small + 4, c->tma_extra_tx);
+    kern<<<c->halo.n_work, HALO_THREADS, S::BYTES, c->stream>>>(*mf, *mr, a, c->halo.work, c->tma_extra_tx);
   });
 }
 
@@ -555,17 +553,13 @@ lbm_status launch_halo(lbm_ctx* c, const T* fin, T* fout, typename Pop<T>::C* P)
 // as in the two-pass schedule.
 template <typename T>
 lbm_status step_halo(lbm_ctx* c, int nsteps) {
-  using C = typename Pop<T>::C;
   const bool three = halo_reach(c->ph) == 3;
   for (int t = 0; t < nsteps; ++t) {
-    const T* fin = (const T*)c->f[c->cur];
-    T* fout = (T*)c->f[c->cur ^ 1];
-    C* P = (C*)c->Pbuf[c->pcur ^ 1];
     lbm_status s;
     if (kDev<T> && c->prm.velocity_refs)
-      s = three ? launch_halo<T, 3, kDev<T>>(c, fin, fout, P) : launch_halo<T, 1, kDev<T>>(c, fin, fout, P);
+      s = three ? launch_halo<T, 3, kDev<T>>(c) : launch_halo<T, 1, kDev<T>>(c);
     else
-      s = three ? launch_halo<T, 3, false>(c, fin, fout, P) : launch_halo<T, 1, false>(c, fin, fout, P);
+      s = three ? launch_halo<T, 3, false>(c) : launch_halo<T, 1, false>(c);
     if (s) return s;
     c->cur ^= 1;
     c->p_valid = false;

@@ -1,9 +1,13 @@
 // Batched stepping of many independent simulations (contexts): each step is
 // one launch per kernel class over all members, through block tables that
 // map a CTA to (member, first list entry) or (member, tile), replayed from
-// a CUDA graph. Two schedules, as for a single simulation: the two-pass one
-// (density pass, Eq. 8 pass, collide pass) and, for 4- and 8-byte storage
-// with tile lists, the tiled single pass (Eq. 8 pass, tiled step).
+// a CUDA graph. Two schedules, as for a single simulation: the list one and,
+// for 4- and 8-byte storage with tile lists, the tiled single pass (Eq. 8
+// pass, tiled step). Under the list schedule, members that keep halo lists
+// (FP32 and 16-bit storage created with AUTO or HALO) step by the halo kernel,
+// one launch for those of one ring and one for those of three; the others by
+// the two passes (density pass, Eq. 8 pass, collide pass). The bits are the
+// same.
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -95,6 +99,76 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_collide_batch(c
                   D.n_fluid, D.g, D.ph);
 }
 
+// The halo step of every member with R rings; 45 simulations of 400 x 200 in
+// FP32 116 -> 95 us per step (two passes before), 512 of 64^2 to 512 x 256 in
+// FP16 641 -> 508. CTA -> record of a tile and its
+// member. args: two per member (buffer parity of the step), copied to shared
+// memory while the copies are under way; maps: four tensor maps per member
+// (populations of buffers 0 and 1, references of buffers 0 and 1), in global
+// memory, hence the fence. cur: two indices per member, into its maps.
+template <typename T, int R, bool VR>
+__global__ void __launch_bounds__(HALO_THREADS, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
+    k_halo_batch(const HaloArgs<T>* __restrict__ args, const CUtensorMap* __restrict__ maps,
+                 const HaloTile* __restrict__ work, const int2* __restrict__ cur, const int* __restrict__ stop,
+                 int parity) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ HaloArgs<T> a;
+  static_assert(sizeof(a) % 4 == 0 && sizeof(a) / 4 <= HALO_THREADS, "one thread per word");
+  HaloTile h;
+  h.n = __ldg(&work[blockIdx.x].n);
+  *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
+  if (*(const volatile int*)stop) return;
+  if (threadIdx.x == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(work + blockIdx.x + HALO_AHEAD));
+  const HaloArgs<T>* src = args + 2 * h.member + parity;
+  const CUtensorMap *mf = maps, *mr = maps;
+  if (threadIdx.x == 0) {
+    const int2 b = __ldg(cur + h.member);
+    mf = maps + 4 * h.member + (b.x ^ parity);
+    mr = maps + 4 * h.member + 2 + (b.y ^ parity);
+    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(mf) : "memory");
+    if (kDev<T>) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(mr) : "memory");
+  }
+  const uint32_t* entries = (const uint32_t*)__ldg((const unsigned long long*)&src->entries);
+  halo_tile<T, R, VR>(h, mf, mr, entries, a, __ldg(&src->ntx), smem_raw, 0u,
+                      [&] {
+                        if (threadIdx.x < sizeof(a) / 4)
+                          ((uint32_t*)&a)[threadIdx.x] = __ldg((const uint32_t*)src + threadIdx.x);
+                      });
+}
+
+// A member's tile records into the batch's list.
+__global__ void __launch_bounds__(256) k_halo_gather(const HaloTile* __restrict__ from, int n, int member,
+                                                     HaloTile* __restrict__ to) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  HaloTile h = from[i];
+  h.member = member;
+  to[i] = h;
+}
+
+// Members of a halo launch: rings of the step and velocity references.
+constexpr int HALO_CLASSES = 4;
+int halo_class(const lbm_ctx* c) { return (halo_reach(c->ph) == 3 ? 2 : 0) + (c->Ubuf[0] ? 1 : 0); }
+template <typename T>
+const void* halo_kernel(int cls) {
+  switch (cls) {
+    case 0: return (const void*)k_halo_batch<T, 1, false>;
+    case 1: return (const void*)k_halo_batch<T, 1, kDev<T>>;
+    case 2: return (const void*)k_halo_batch<T, 3, false>;
+    default: return (const void*)k_halo_batch<T, 3, kDev<T>>;
+  }
+}
+template <typename T>
+int halo_smem(int cls) {
+  switch (cls) {
+    case 0: return HaloSmem<T, 1, false>::BYTES;
+    case 1: return HaloSmem<T, 1, kDev<T>>::BYTES;
+    case 2: return HaloSmem<T, 3, false>::BYTES;
+    default: return HaloSmem<T, 3, kDev<T>>::BYTES;
+  }
+}
+
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 size_t desc_bytes(int storage) {
   return storage == LBM_STORE_FP64 ? sizeof(BatchDesc<double>) : sizeof(BatchDesc<float>);
@@ -124,6 +198,16 @@ struct lbm_batch {
   int schedule;         // LBM_KERNEL_TWO_PASS or LBM_KERNEL_TILED
   bool tiled_ok;        // 4- or 8-byte storage and every member keeps tile lists
   bool vr;              // 16-bit storage and some member keeps velocity references
+  // halo steps of the list schedule
+  bool* halo;           // per member: it steps by the halo kernel
+  void* d_hargs;        // HaloArgs[2 n], and their host staging
+  void* h_hargs;
+  CUtensorMap* d_hmaps; // [4 n]
+  int2* d_hcur;         // [n], and host staging
+  int2* h_hcur;
+  HaloTile* d_hwork[HALO_CLASSES];
+  int n_hwork[HALO_CLASSES];
+  int* d_stop;
   int bs;               // threads per block of the density and collide kernels
   void* h_desc;         // host staging of the descriptors
   int2* h_tab;          // host staging of the block tables
@@ -150,8 +234,13 @@ lbm_status bcuda(lbm_batch* b, cudaError_t e, const char* where) {
 // Device layout of a batch workspace: descriptors, fluid block table (sized
 // for the smallest block size), interface block table, tile block table.
 struct BLayout {
-  size_t desc, fblk, iblk, tblk, total;
+  size_t desc, fblk, iblk, tblk, hargs, hmaps, hcur, hwork[HALO_CLASSES], stop, total;
+  int n_hwork[HALO_CLASSES];
 };
+size_t hargs_bytes(int storage) {
+  return storage == LBM_STORE_FP64 ? sizeof(HaloArgs<double>)
+                                   : storage == LBM_STORE_FP32 ? sizeof(HaloArgs<float>) : sizeof(HaloArgs<__half>);
+}
 
 // The tiled schedule runs when the storage is 4 or 8 bytes and every member
 // keeps the per-tile lists (contexts created with LBM_KERNEL_AUTO or TILED).
@@ -161,6 +250,10 @@ bool batch_tiled_ok(int n, lbm_ctx* const* ctxs) {
     if (ctxs[s]->n_tiles <= 0) return false;
   return true;
 }
+
+// Whether a member of the list schedule steps by the halo kernel. FP64 members
+// keep the two passes (bound by the FP64 pipe).
+bool batch_halo(const lbm_ctx* c) { return c->halo_ready && c->prm.storage != LBM_STORE_FP64; }
 
 BLayout blayout(int n, lbm_ctx* const* ctxs) {
   int* lf = (int*)malloc(sizeof(int) * n);
@@ -178,6 +271,17 @@ BLayout blayout(int n, lbm_ctx* const* ctxs) {
   if (batch_tiled_ok(n, ctxs))
     for (int s = 0; s < n; ++s) nt += ctxs[s]->n_tiles;
   L.tblk = off;  off = align_up(off + (size_t)nt * sizeof(int2), 256);
+  L.hargs = off; off = align_up(off + 2 * (size_t)n * hargs_bytes(ctxs[0]->prm.storage), 256);
+  L.hmaps = off; off = align_up(off + 4 * (size_t)n * sizeof(CUtensorMap), 256);
+  L.hcur = off;  off = align_up(off + (size_t)n * sizeof(int2), 256);
+  for (int k = 0; k < HALO_CLASSES; ++k) L.n_hwork[k] = 0;
+  for (int s = 0; s < n; ++s)
+    if (batch_halo(ctxs[s])) L.n_hwork[halo_class(ctxs[s])] += ctxs[s]->halo.n_work;
+  for (int k = 0; k < HALO_CLASSES; ++k) {
+    L.hwork[k] = off;
+    off = align_up(off + (size_t)L.n_hwork[k] * sizeof(HaloTile), 256);
+  }
+  L.stop = off;  off = align_up(off + 4, 256);
   L.total = off;
   free(lf);
   free(li);
@@ -193,13 +297,41 @@ int build_table(int2* h_tab, int n, int bs, LenFn len) {
   return e;
 }
 
-lbm_status upload_fluid_table(lbm_batch* b, int bs) {
+// Block tables of the density, collide and Eq. 8 launches, bs threads per
+// block: every member under the tiled schedule, those of the two passes under
+// the list schedule.
+lbm_status upload_tables(lbm_batch* b, int bs) {
+  const bool all = b->schedule == LBM_KERNEL_TILED;
   b->bs = bs;
-  b->n_fblk = build_table(b->h_tab, b->n, bs, [&](int s) { return b->ctx[s]->n_fluid; });
+  b->n_fblk = build_table(b->h_tab, b->n, bs, [&](int s) { return all || !b->halo[s] ? b->ctx[s]->n_fluid : 0; });
   lbm_status st = bcuda(b, cudaMemcpyAsync(b->d_fblk, b->h_tab, (size_t)b->n_fblk * sizeof(int2),
                                            cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
   if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
+  if (st) return st;
+  // interface blocks (128 threads), only for simulations with the improved scheme
+  b->n_iblk = build_table(b->h_tab, b->n, 128, [&](int s) {
+    return b->ctx[s]->ph.bc == BC_VAVG && (all || !b->halo[s]) ? b->ctx[s]->n_iface : 0;
+  });
+  st = bcuda(b, cudaMemcpyAsync(b->d_iblk, b->h_tab, (size_t)b->n_iblk * sizeof(int2), cudaMemcpyHostToDevice,
+                                b->stream), "cudaMemcpyAsync");
+  if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
   return st;
+}
+
+template <typename T>
+void fill_halo(lbm_batch* b) {
+  HaloArgs<T>* h = (HaloArgs<T>*)b->h_hargs;
+  for (int s = 0; s < b->n; ++s) {
+    const lbm_ctx* c = b->ctx[s];
+    for (int p = 0; p < 2; ++p) h[2 * s + p] = halo_args<T>(c, c->cur ^ p, c->pcur ^ p, b->d_stop);
+    b->h_hcur[s] = make_int2(c->cur, c->Ubuf[0] ? c->cur : c->pcur);
+  }
+}
+
+bool any_halo(const lbm_batch* b) {
+  for (int k = 0; k < HALO_CLASSES; ++k)
+    if (b->n_hwork[k] > 0) return true;
+  return false;
 }
 
 template <typename C>
@@ -231,6 +363,22 @@ void fill_descs(lbm_batch* b) {
     d.ph = kphys<C>(c->ph);
   }
 }
+
+// Arguments of one halo launch (class k, parity p).
+template <typename T>
+struct HaloLaunch {
+  const HaloArgs<T>* hargs;
+  const CUtensorMap* maps;
+  const HaloTile* work;
+  const int2* cur;
+  const int* stop;
+  int parity;
+  void* args[6];
+  HaloLaunch(const lbm_batch* b, int k, int p)
+      : hargs((const HaloArgs<T>*)b->d_hargs), maps(b->d_hmaps), work(b->d_hwork[k]), cur(b->d_hcur), stop(b->d_stop),
+        parity(p), args{&hargs, &maps, &work, &cur, &stop, &parity} {}
+  HaloLaunch(const HaloLaunch&) = delete;
+};
 
 // Enqueue one step (parity p) directly on the stream.
 template <typename T>
@@ -265,13 +413,25 @@ lbm_status launch_step(lbm_batch* b, int p) {
     kc<<<b->n_fblk, b->bs, 0, b->stream>>>(d, b->d_fblk, p);
     b->launches++;
   }
+  if constexpr (sizeof(T) <= 4) {
+    for (int k = 0; k < HALO_CLASSES; ++k) {
+      if (b->n_hwork[k] == 0) continue;
+      HaloLaunch<T> L(b, k, p);
+      lbm_status st = bcuda(b, cudaLaunchKernel(halo_kernel<T>(k), dim3(b->n_hwork[k]), dim3(HALO_THREADS), L.args,
+                                                halo_smem<T>(k), b->stream), "batched halo launch");
+      if (st) return st;
+      b->launches++;
+    }
+  }
   return bcuda(b, cudaGetLastError(), "batched step launch");
 }
 
 // Kernel launches per step of the current schedule.
 int launches_per_step(const lbm_batch* b) {
   if (b->schedule == LBM_KERNEL_TILED) return (b->n_iblk > 0) + (b->n_tblk > 0);
-  return (b->n_fblk > 0) * 2 + (b->n_iblk > 0);
+  int n = (b->n_fblk > 0) * 2 + (b->n_iblk > 0);
+  for (int k = 0; k < HALO_CLASSES; ++k) n += b->n_hwork[k] > 0;
+  return n;
 }
 
 void drop_graph(lbm_batch* b) {
@@ -322,6 +482,23 @@ lbm_status build_graph(lbm_batch* b, int steps) {
                  "cudaGraphAddKernelNode");
       prev = node;
     }
+    if constexpr (sizeof(T) <= 4) {
+      for (int q = 0; q < HALO_CLASSES && !st && !tiled; ++q) {
+        if (b->n_hwork[q] == 0) continue;
+        HaloLaunch<T> L(b, q, p);
+        cudaKernelNodeParams kp;
+        memset(&kp, 0, sizeof(kp));
+        kp.func = (void*)halo_kernel<T>(q);
+        kp.gridDim = dim3(b->n_hwork[q]);
+        kp.blockDim = dim3(HALO_THREADS);
+        kp.sharedMemBytes = (unsigned)halo_smem<T>(q);
+        kp.kernelParams = L.args;
+        cudaGraphNode_t node;
+        st = bcuda(b, cudaGraphAddKernelNode(&node, b->graph, prev ? &prev : nullptr, prev ? 1 : 0, &kp),
+                   "cudaGraphAddKernelNode");
+        prev = node;
+      }
+    }
   }
   if (!st) st = bcuda(b, cudaGraphInstantiate(&b->exec, b->graph, 0), "cudaGraphInstantiate");
   if (st) {
@@ -346,7 +523,18 @@ lbm_status batch_step(lbm_batch* b, int nsteps) {
   }
   lbm_status st = bcuda(b, cudaMemcpyAsync(b->d_desc, b->h_desc, (size_t)b->n * sizeof(BatchDesc<C>),
                                            cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
-  // the staging buffer is rewritten by the next call: wait for the copy
+  const bool halo = !tiled && any_halo(b);
+  if constexpr (sizeof(T) <= 4) {
+    if (halo && !st) {
+      fill_halo<T>(b);
+      st = bcuda(b, cudaMemcpyAsync(b->d_hargs, b->h_hargs, 2 * (size_t)b->n * sizeof(HaloArgs<T>),
+                                    cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
+      if (!st) st = bcuda(b, cudaMemcpyAsync(b->d_hcur, b->h_hcur, (size_t)b->n * sizeof(int2),
+                                             cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
+      if (!st) st = bcuda(b, cudaMemsetAsync(b->d_stop, 0, 4, b->stream), "cudaMemsetAsync");
+    }
+  }
+  // the staging buffers are rewritten by the next call: wait for the copies
   if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
   if (!st && tiled && nsteps > 0) {
     // the tiled step reads rho(t) from Pbuf[pcur]: compute it for every
@@ -374,6 +562,7 @@ lbm_status batch_step(lbm_batch* b, int nsteps) {
       c->pcur ^= 1;
       c->P = c->Pbuf[c->pcur];
     }
+    if (halo && b->halo[s] && nsteps > 0) c->halo_used = true;
     // after tiled steps Pbuf[pcur] holds rho of the current state
     c->p_valid = tiled && (nsteps > 0 || c->p_valid);
   }
@@ -387,6 +576,59 @@ lbm_status batch_step(lbm_batch* b, int nsteps) {
     case LBM_STORE_FP16: { using T = __half; CALL; }     \
     default: { using T = __nv_bfloat16; CALL; }          \
   }
+
+void free_batch(lbm_batch* b) {
+  free(b->ctx);
+  free(b->h_desc);
+  free(b->h_tab);
+  free(b->halo);
+  free(b->h_hargs);
+  free(b->h_hcur);
+  delete b;
+}
+
+// Tensor maps and tile records of the members that step by the halo kernel.
+// Synchronises.
+lbm_status create_halo(lbm_batch* b) {
+  CUtensorMap* h = (CUtensorMap*)malloc(4 * (size_t)b->n * sizeof(CUtensorMap));
+  if (!h) return LBM_ERR_SPACE;
+  size_t off[HALO_CLASSES] = {};
+  lbm_status st = LBM_OK;
+  for (int s = 0; s < b->n && !st; ++s) {
+    const lbm_ctx* c = b->ctx[s];
+    if (!b->halo[s]) continue;
+    const int k = halo_class(c), r = halo_reach(c->ph) == 3;
+    for (int i = 0; i < 2; ++i) {
+      h[4 * s + i] = c->hmap_f[r][i];
+      h[4 * s + 2 + i] = c->hmap_ref[r][i];
+    }
+    k_halo_gather<<<(c->halo.n_work + 255) / 256, 256, 0, b->stream>>>(c->halo.work, c->halo.n_work, s,
+                                                                       b->d_hwork[k] + off[k]);
+    off[k] += c->halo.n_work;
+    st = bcuda(b, cudaGetLastError(), "k_halo_gather");
+  }
+  if (!st) st = bcuda(b, cudaMemcpyAsync(b->d_hmaps, h, 4 * (size_t)b->n * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
+                                         b->stream), "cudaMemcpyAsync");
+  if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
+  for (int k = 0; k < HALO_CLASSES && !st; ++k) {
+    if (b->n_hwork[k] == 0) continue;
+    switch (b->storage) {
+      case LBM_STORE_FP32:
+        st = bcuda(b, cudaFuncSetAttribute(halo_kernel<float>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           halo_smem<float>(k)), "cudaFuncSetAttribute");
+        break;
+      case LBM_STORE_FP16:
+        st = bcuda(b, cudaFuncSetAttribute(halo_kernel<__half>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           halo_smem<__half>(k)), "cudaFuncSetAttribute");
+        break;
+      default:
+        st = bcuda(b, cudaFuncSetAttribute(halo_kernel<__nv_bfloat16>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           halo_smem<__nv_bfloat16>(k)), "cudaFuncSetAttribute");
+    }
+  }
+  free(h);
+  return st;
+}
 
 lbm_status check_members(int32_t n, lbm_ctx* const* ctxs) {
   if (n < 1 || !ctxs) return LBM_ERR_ARG;
@@ -449,22 +691,27 @@ lbm_status lbm_batch_create(int32_t n, lbm_ctx* const* ctxs, void* d_workspace, 
     tab_cap += ef > ei ? (ef > et ? ef : et) : (ei > et ? ei : et);
   }
   b->h_tab = (int2*)malloc((size_t)tab_cap * sizeof(int2));
-  if (!b->ctx || !b->h_desc || !b->h_tab) {
-    free(b->ctx);
-    free(b->h_desc);
-    free(b->h_tab);
-    delete b;
+  b->halo = (bool*)malloc((size_t)n);
+  b->h_hargs = malloc(2 * (size_t)n * hargs_bytes(b->storage));
+  b->h_hcur = (int2*)malloc((size_t)n * sizeof(int2));
+  b->d_hargs = b->ws + L.hargs;
+  b->d_hmaps = (CUtensorMap*)(b->ws + L.hmaps);
+  b->d_hcur = (int2*)(b->ws + L.hcur);
+  b->d_stop = (int*)(b->ws + L.stop);
+  for (int k = 0; k < HALO_CLASSES; ++k) {
+    b->d_hwork[k] = (HaloTile*)(b->ws + L.hwork[k]);
+    b->n_hwork[k] = L.n_hwork[k];
+  }
+  if (!b->ctx || !b->h_desc || !b->h_tab || !b->halo || !b->h_hargs || !b->h_hcur) {
+    free_batch(b);
     return LBM_ERR_SPACE;
   }
-  for (int s = 0; s < n; ++s) b->ctx[s] = ctxs[s];
-  // interface blocks (128 threads), only for simulations with the improved scheme
-  b->n_iblk = build_table(b->h_tab, n, 128, [&](int s) {
-    return b->ctx[s]->ph.bc == BC_VAVG ? b->ctx[s]->n_iface : 0;
-  });
-  st = bcuda(b, cudaMemcpyAsync(b->d_iblk, b->h_tab, (size_t)b->n_iblk * sizeof(int2), cudaMemcpyHostToDevice,
-                                b->stream), "cudaMemcpyAsync");
-  if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
-  if (!st) st = upload_fluid_table(b, 256);
+  for (int s = 0; s < n; ++s) {
+    b->ctx[s] = ctxs[s];
+    b->halo[s] = batch_halo(ctxs[s]);
+  }
+  st = upload_tables(b, 256);
+  if (!st && any_halo(b)) st = create_halo(b);
   if (!st && b->tiled_ok) {
     // tile blocks: every tile of every member, member by member
     int e = 0;
@@ -479,10 +726,7 @@ lbm_status lbm_batch_create(int32_t n, lbm_ctx* const* ctxs, void* d_workspace, 
                                          (int)tile_smem<double>()), "cudaFuncSetAttribute");
   }
   if (st) {
-    free(b->ctx);
-    free(b->h_desc);
-    free(b->h_tab);
-    delete b;
+    free_batch(b);
     return st;
   }
   *out = b;
@@ -510,7 +754,11 @@ lbm_status lbm_batch_set_schedule(lbm_batch* b, int32_t kernel) {
   if (kernel != LBM_KERNEL_TWO_PASS && kernel != LBM_KERNEL_TILED) return bfail(b, LBM_ERR_ARG, "unknown schedule");
   if (kernel == LBM_KERNEL_TILED && !b->tiled_ok)
     return bfail(b, LBM_ERR_ARG, "tiled schedule needs 4- or 8-byte storage and members with tile lists");
-  b->schedule = kernel;
+  if (b->schedule != kernel) {
+    b->schedule = kernel;
+    lbm_status st = upload_tables(b, b->bs);
+    if (st) return st;
+  }
   return b->graph_steps > 0 ? lbm_batch_set_graph_steps(b, b->graph_steps) : LBM_OK;
 }
 
@@ -542,7 +790,7 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int32_t trial_steps, int32_t* h_choi
   int best_steps = 2;
   for (int ic = 0; ic < 3 && !st; ++ic) {
     if (kCand[ic].schedule == LBM_KERNEL_TILED && !b->tiled_ok) continue;
-    st = upload_fluid_table(b, kCand[ic].bs);
+    st = upload_tables(b, kCand[ic].bs);
     if (!st) st = lbm_batch_set_schedule(b, kCand[ic].schedule);
     for (int is = 0; is < 3 && !st; ++is) {
       const int S = kSteps[is];
@@ -564,7 +812,7 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int32_t trial_steps, int32_t* h_choi
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (!st) st = upload_fluid_table(b, best_c.bs);
+  if (!st) st = upload_tables(b, best_c.bs);
   if (!st) st = lbm_batch_set_schedule(b, best_c.schedule);
   if (!st) st = lbm_batch_set_graph_steps(b, best_steps);
   if (!st && h_choice) {
@@ -581,10 +829,7 @@ const char* lbm_batch_last_error(const lbm_batch* b) { return b ? b->err : ""; }
 lbm_status lbm_batch_destroy(lbm_batch* b) {
   if (!b) return LBM_ERR_ARG;
   drop_graph(b);
-  free(b->ctx);
-  free(b->h_desc);
-  free(b->h_tab);
-  delete b;
+  free_batch(b);
   return LBM_OK;
 }
 

@@ -245,6 +245,7 @@ struct Pop<__nv_bfloat16> {
 template <typename T>
 struct StorePtrs {
   char *own[9], *bounce[9];
+  StorePtrs() = default;
   StorePtrs(T* f, const Geo& g) {
     for (int i = 0; i < 9; ++i) {
       own[i] = (char*)(f + pslot(g, i, 0));

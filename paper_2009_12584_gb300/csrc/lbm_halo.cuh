@@ -43,18 +43,18 @@ namespace lbm {
 constexpr int HALO_W = 32;  // owned columns of a tile
 // Owned rows and threads: three windows of three rings, or four of one ring,
 // fill an SM's shared memory, and the threads take the tile's own nodes of a
-// porous medium (60% fluid) in about one round at 64 to 96 registers each.
+// porous medium (60% fluid) in about one round at 72 to 80 registers each.
 // 4096^2 porous, us per step, improved scheme / LLKC: FP32 with 14 rows and
 // 224 threads 406 / 363 (256 threads 411 / 363, 12 rows 429 / 371, 16 rows
-// 480 / 383); FP16 with 20 rows and 256 threads 376 / 337 (16 rows 400 / 346,
-// 24 rows 356 / 352, and with velocity references 450 against 478 and 515).
+// 480 / 383); FP16 with 20 rows and 224 threads 387 / 330 (192 threads 388 /
+// 338, 256 threads 384 / 343, 16 rows and 256 threads 400 / 346, 24 rows 356 /
+// 352, but with velocity references 515 against 464).
 constexpr int HALO_H = 14, HALO_H16 = 20;
 template <typename T>
 constexpr int halo_h = sizeof(T) == 2 ? HALO_H16 : HALO_H;
 __host__ __device__ inline int halo_rows(int elem_size) { return elem_size == 2 ? HALO_H16 : HALO_H; }
 constexpr int HALO_O = 4;                        // entries count columns and rows from (x0 - 4, y0 - 4)
-template <typename T>
-constexpr int halo_threads = sizeof(T) == 2 ? 256 : 224;
+constexpr int HALO_THREADS = 224;
 constexpr int HALO_AHEAD = 512;  // CTAs between one and that whose record it asks L2 for
 constexpr int HALO_LIST_THREADS = 256;
 constexpr int HALO_RW = HALO_W + 6;              // region of the lists: the tile and three rings
@@ -76,13 +76,32 @@ inline int halo_reach(const Phys& ph) { return ph.bc == BC_VAVG ? 3 : 1; }
 // copies start on 16 bytes) and first cell, and its number.
 struct alignas(32) HaloTile {
   int4 n;
-  int e0, i0, tile, pad;
+  int e0, i0, tile, member;  // member: in a batch's list, the simulation it belongs to
 };
 struct HaloLists {
   const HaloTile* work;  // in tile order
   int n_work;
   const uint32_t* entries;
   const uint2* cells;  // (place in the window as in an entry, 5 x 5 fluid bits)
+};
+
+// What a step needs of one simulation besides its tensor maps. P: the density
+// plane that takes rho(t), the references of what a 16-bit step stores; Uo:
+// with velocity references the velocity plane that does. err: the
+// simulation's error word; stop: the word that keeps later CTAs of the step
+// from starting (of a batch; err itself otherwise).
+template <typename T>
+struct HaloArgs {
+  using C = typename Pop<T>::C;
+  StorePtrs<T> out;
+  C* P;
+  UPair* Uo;
+  const uint32_t* entries;
+  const uint2* cells;
+  int *err, *stop;
+  int ntx;
+  Geo g;
+  PhysK<C> ph;
 };
 
 // Fluid neighbours of the cell at padded index k (k_iface_mask's bits).
@@ -175,54 +194,49 @@ struct HaloSmem {
   static constexpr int BYTES = ENT + pad((HALO_W + 2 * R) * (H + 2 * R) * 4 + 16) + 128;
 };
 
-// mapf: tensor map of the populations (pairs; x in units of Pop<T>::V, FP64 of
-// 8 bytes), with a box of one tile's window; mapref: of the references. P: the
-// density plane that takes rho(t), the references of what a 16-bit step
-// stores. err: set to 1
-// when the copies were not seen to complete within the bound (the CTA then
-// stops, and those that start later do nothing); extra_tx: see tma_issue. FP64 is bound by its arithmetic, not by
-// the one CTA per SM that its windows allow.
-template <typename T, int R, bool VR>
-__global__ void __launch_bounds__(halo_threads<T>, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
-    k_halo(const __grid_constant__ CUtensorMap mapf, const __grid_constant__ CUtensorMap mapref, T* __restrict__ fo,
-           const __grid_constant__ StorePtrs<T> out, typename Pop<T>::C* __restrict__ P, UPair* __restrict__ Uo, HaloLists L, Geo g, int ntx,
-           PhysK<typename Pop<T>::C> ph, int* __restrict__ err, uint32_t extra_tx) {
+// The work of one CTA on a tile with record h. mapf: tensor map of the
+// populations (pairs; x in units of Pop<T>::V, FP64 of 8 bytes), with a box of
+// one tile's window; mapref: of the references. a: the simulation's arguments,
+// and entries its list, which the thread that issues the copies has at hand.
+// stage: shared memory of HaloSmem::BYTES. The error word is set to 1 when
+// the copies were not seen to complete within the bound; extra_tx: see
+// tma_issue. ready(): called once by every thread before the first use of a.
+template <typename T, int R, bool VR, typename Ready>
+__device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* mapf, const CUtensorMap* mapref,
+                                          const uint32_t* entries, const HaloArgs<T>& a, int ntx,
+                                          unsigned char* smem_raw, uint32_t extra_tx, Ready&& ready) {
   using C = typename Pop<T>::C;
   using V = typename CPair<C>::V;
   using S = HaloSmem<T, R, VR>;
-  constexpr int NT = halo_threads<T>;
+  constexpr int NT = HALO_THREADS;
   constexpr uint32_t FB = 2 * sizeof(T);
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar;
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
   V* rho = (V*)(sm + S::RHO);
   const uint32_t* ent = (const uint32_t*)(sm + S::ENT);
   const int tid = threadIdx.x;
-  const HaloTile* item = L.work + blockIdx.x;
+  const int n_own = h.n.x, n_a = R == 1 ? h.n.y : h.n.z, n_if = h.n.w, i0 = h.i0;
+  const int x0 = (h.tile % ntx) * HALO_W, y0 = (h.tile / ntx) * S::H;
   if (tid == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  const int4 cn = __ldg(&item->n), it = __ldg((const int4*)&item->e0);
-  if (*(volatile int*)err) return;  // the whole CTA, or it waits (bounded) like the ones before it
-  const int n_own = cn.x, n_a = R == 1 ? cn.y : cn.z, n_if = cn.w, i0 = it.y, tile = it.z;
-  const int x0 = (tile % ntx) * HALO_W, y0 = (tile / ntx) * S::H;
-  if (tid == 0) {
     // the window's first node: column x0 - O + LP (a multiple of 4 nodes with
     // 16-bit storage, of 2 otherwise: 16-byte aligned), row y0 - (R + 1) + GH
     const int xw = x0 - S::O + LP, yw = y0 - (R + 1) + GH;
     const uint32_t ebytes = (uint32_t)((n_a + 3) & ~3) * 4;
     mbar_expect_tx(&bar, 9u * S::FBYTES + S::RBYTES + ebytes + extra_tx);
-    bulk_load(sm + S::ENT, L.entries + it.x, ebytes, &bar);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) tma_load_3d(sm + i * S::FSLOT, &mapf, sizeof(T) == 8 ? 2 * xw : xw, yw, i, &bar);
-    if (kDev<T>) tma_load_2d(sm + S::REF, &mapref, VR ? 2 * xw : xw, yw, &bar);
+    for (int i = 0; i < 9; ++i) tma_load_3d(sm + i * S::FSLOT, mapf, sizeof(T) == 8 ? 2 * xw : xw, yw, i, &bar);
+    if (kDev<T>) tma_load_2d(sm + S::REF, mapref, VR ? 2 * xw : xw, yw, &bar);
+    bulk_load(sm + S::ENT, entries + h.e0, ebytes, &bar);
   }
-  if (tid == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(item + HALO_AHEAD));
+  ready();
+  __syncthreads();  // the barrier is initialised
+  const Geo& g = a.g;
+  const PhysK<C>& ph = a.ph;
   // this thread's interface-solid cell, needed after phase A
   uint2 cell = make_uint2(0, 0);
-  if (tid < n_if) cell = __ldg(L.cells + i0 + tid);
+  if (tid < n_if) cell = __ldg(a.cells + i0 + tid);
   // An entry's node in the window held in shared memory, and in cells of
   // the padded grid from the entries' node (0, 0).
   auto place = [](uint32_t e) {
@@ -257,7 +271,6 @@ __global__ void __launch_bounds__(halo_threads<T>, sizeof(T) == 8 ? 1 : R == 1 ?
     }
   };
 
-  __syncthreads();  // the barrier is initialised
   bool ok = mbar_wait(&bar, 0);
   if (!ok) ok = mbar_wait(&bar, 0);  // the copies in flight, once more
 
@@ -274,18 +287,21 @@ __global__ void __launch_bounds__(halo_threads<T>, sizeof(T) == 8 ? 1 : R == 1 ?
       for (int t = tid; t < n_if; t += NT) {
         V z;
         z.x = z.y = C(0);
-        rho[place(t == tid ? cell.x : __ldg(L.cells + i0 + t).x)] = z;
+        rho[place(t == tid ? cell.x : __ldg(a.cells + i0 + t).x)] = z;
       }
   }
   if (__syncthreads_or(!ok)) {
-    if (tid == 0) atomicExch(err, 1);
+    if (tid == 0) {
+      atomicExch(a.err, 1);
+      atomicExch(a.stop, 1);
+    }
     return;
   }
 
   // phase V
   if (R == 3) {
     for (int t = tid; t < n_if; t += NT) {
-      const uint2 cl = t == tid ? cell : __ldg(L.cells + i0 + t);
+      const uint2 cl = t == tid ? cell : __ldg(a.cells + i0 + t);
       const int w = place(cl.x);
       auto load = [&](int dx, int dy, C& a, C& b) {
         const V v = rho[w + dx + dy * S::P];
@@ -331,29 +347,29 @@ __global__ void __launch_bounds__(halo_threads<T>, sizeof(T) == 8 ? 1 : R == 1 ?
         const float2 d57 = sub2(fp[5], fp[7]), d86 = sub2(fp[8], fp[6]);
         up = u_pack(add2(sub2(fp[1], fp[3]), add2(d57, d86)), add2(sub2(fp[2], fp[4]), sub2(d57, d86)), rv);
         U = u_unpack(up);
-        Uo[kp] = up;
+        a.Uo[kp] = up;
       } else {
-        stP(P, kp, rh[0], rh[1]);
+        stP(a.P, kp, rh[0], rh[1]);
       }
       if (warp_border) {
         for_ghost_images(g, x, y, [&](int kk) {
           if constexpr (VR)
-            Uo[kk] = up;
+            a.Uo[kk] = up;
           else
-            stP(P, kk, rh[0], rh[1]);
+            stP(a.P, kk, rh[0], rh[1]);
         });
       }
     }
     write_refs<T>(rh, VR, U, ref);
     if (!warp_border) {
 #pragma unroll
-      for (int i = 0; i < 9; ++i) out.st(out.own[i], kp, Pop<T>::pack(fp[i].x, fp[i].y, ref[0][i], ref[1][i]));
+      for (int i = 0; i < 9; ++i) StorePtrs<T>::st(a.out.own[i], kp, Pop<T>::pack(fp[i].x, fp[i].y, ref[0][i], ref[1][i]));
       if (warp_edge) {
         // the solid neighbours are owned nodes without images: slot i of x - c_i
 #pragma unroll
         for (int i = 1; i < 9; ++i) {
           const int o = opp_of(i);
-          if (fl & nb_bit(o)) out.st(out.bounce[i], kp, Pop<T>::pack(fp[o].x, fp[o].y, ref[0][o], ref[1][o]));
+          if (fl & nb_bit(o)) StorePtrs<T>::st(a.out.bounce[i], kp, Pop<T>::pack(fp[o].x, fp[o].y, ref[0][o], ref[1][o]));
         }
       }
     } else {
@@ -363,10 +379,29 @@ __global__ void __launch_bounds__(halo_threads<T>, sizeof(T) == 8 ? 1 : R == 1 ?
         fv[0][i] = fp[i].x;
         fv[1][i] = fp[i].y;
       }
+      T* fo = (T*)a.out.own[0];
       store_node(fo, g, x, y, (int)kp, fv, ref);
       store_bounced(fo, g, x, y, fl, fv, ref);
     }
   }
+}
+
+// A step of one simulation, a CTA per tile that owns fluid nodes. A CTA that
+// finds the error word set does nothing (it would wait like the one that set
+// it). FP64 is bound by its arithmetic, not by the one CTA per SM that its
+// windows allow.
+template <typename T, int R, bool VR>
+__global__ void __launch_bounds__(HALO_THREADS, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
+    k_halo(const __grid_constant__ CUtensorMap mapf, const __grid_constant__ CUtensorMap mapref,
+           const __grid_constant__ HaloArgs<T> a, const HaloTile* __restrict__ work, uint32_t extra_tx) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  HaloTile h;
+  h.n = __ldg(&work[blockIdx.x].n);
+  *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
+  if (*(volatile int*)a.stop) return;
+  if (threadIdx.x == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(work + blockIdx.x + HALO_AHEAD));
+  halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, a.ntx, smem_raw, extra_tx, [] {});
 }
 
 }  // namespace lbm

@@ -99,3 +99,20 @@ struct lbm_ctx {
 lbm_status clear_virtual(lbm_ctx* c, cudaStream_t stream);
 // The tiled schedule's lists of the installed geometry (lbm_api.cu).
 lbm_status build_tile_lists(lbm_ctx* c, cudaStream_t stream);
+
+// The halo step's arguments for a context whose current state is in buffer
+// cur, its density plane pcur (the spare one takes a 16-bit step's rho(t)).
+template <typename T>
+inline lbm::HaloArgs<T> halo_args(const lbm_ctx* c, int cur, int pcur, int* stop = nullptr) {
+  using C = typename lbm::Pop<T>::C;
+  return lbm::HaloArgs<T>{lbm::StorePtrs<T>((T*)c->f[cur ^ 1], c->g),
+                          (C*)c->Pbuf[pcur ^ 1],
+                          c->Ubuf[cur ^ 1],
+                          c->halo.entries,
+                          c->halo.cells,
+                          c->small + 4,
+                          stop ? stop : c->small + 4,
+                          (c->g.nx + lbm::HALO_W - 1) / lbm::HALO_W,
+                          c->g,
+                          lbm::kphys<C>(c->ph)};
+}

@@ -128,3 +128,37 @@ def test_halo_wait_runs_out_and_context_recovers():
     sims[1].step(7)
     sims[0].sync()
     assert torch.equal(sims[0].populations(), sims[1].populations())
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp64", "fp16", "bf16"])
+@pytest.mark.parametrize("graph", [0, 2])
+def test_batch_of_mixed_members_matches_members_alone(storage, graph):
+    """One batch over everything its list schedule tells apart: one ring and
+    three, with and without velocity references, members of the two passes
+    among those of the halo kernel, sizes below and above a tile; odd step
+    counts, and a member that starts from the other buffer."""
+    kinds = [(4, 4, "auto", IMPROVED, False), (33, 21, "two_pass", IMPROVED, False),
+             (70, 45, "auto", SCHEMES["llkc"], False), (64, 40, "halo", IMPROVED, True),
+             (32, 14, "auto", SCHEMES["mc"], True), (100, 61, "two_pass", SCHEMES["constant"], True)]
+    pairs = []
+    for i, (nx, ny, kernel, wet, vref) in enumerate(kinds):
+        two = []
+        for _ in range(2):
+            sim = lbm.Simulation(nx, ny, storage=storage, kernel=kernel, periodic_x=True, periodic_y=True,
+                                 velocity_refs=vref and storage in ("fp16", "bf16"))
+            sim.set_geometry(inputs.random_solid_mask(nx, ny, seed=i, fraction=0.1)).set_wetting(wet[0], **wet[1])
+            rA, rB, ux, uy = inputs.random_fields(nx, ny, 20 + i, umax=0.05)
+            two.append(sim.init_fields(rA, rB, ux, uy).step(i % 2))
+        pairs.append(two)
+    batch = lbm.Batch([p[0] for p in pairs])
+    if graph:
+        batch.set_graph_steps(graph)
+    for n in (1, 4, 3):
+        batch.step(n)
+        for a, b in pairs:
+            b.step(n)
+            a.sync()
+            assert torch.equal(a.populations(), b.populations())
+    for a, b in pairs:  # and alone again
+        assert torch.equal(a.step(2).populations(), b.step(2).populations())
+    batch.close()
