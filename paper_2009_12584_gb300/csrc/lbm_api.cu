@@ -595,17 +595,50 @@ lbm_status do_step(lbm_ctx* c, int nsteps) {
   return step_two_pass<T>(c, nsteps);
 }
 
-template <typename T, int MODE, typename O = double>
-lbm_status do_eval(lbm_ctx* c, O* out) {
+// Moments by the halo schedule's kernel (contexts with its lists).
+template <typename T, int R, bool VR, typename O>
+lbm_status launch_halo_moments(lbm_ctx* c, const EvalOut<O>& out) {
+  using S = HaloSmem<T, R, VR>;
+  auto kern = k_halo_moments<T, R, VR, O>;
+  // (per call: an evaluation is one of several kernels)
+  lbm_status s = check_cuda(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::BYTES),
+                            "cudaFuncSetAttribute");
+  if (s) return s;
+  const CUtensorMap* mf = &c->hmap_f[R == 3][c->cur];
+  const CUtensorMap* mr = kDev<T> ? &c->hmap_ref[R == 3][c->Ubuf[0] ? c->cur : c->pcur] : mf;
+  k_zero_solid<O><<<node_grid(c->g, 128), 128, 0, c->stream>>>(c->flags, c->g, out);
+  if ((s = after_launch(c, "k_zero_solid"))) return s;
+  kern<<<c->halo.n_work, HALO_THREADS, S::BYTES, c->stream>>>(*mf, *mr, halo_args<T>(c, c->cur, c->pcur), c->halo.work,
+                                                              c->tma_extra_tx, out);
+  c->halo_used = true;
+  return after_launch(c, "k_halo_moments");
+}
+
+template <typename T, int MODE, typename O>
+lbm_status do_eval(lbm_ctx* c, const EvalOut<O>& out) {
+  using C = typename Pop<T>::C;
+  if constexpr (MODE == 1 && sizeof(T) <= 4) {
+    if (c->halo_ready) {
+      const bool three = halo_reach(c->ph) == 3;
+      if (kDev<T> && c->prm.velocity_refs)
+        return three ? launch_halo_moments<T, 3, kDev<T>>(c, out) : launch_halo_moments<T, 1, kDev<T>>(c, out);
+      return three ? launch_halo_moments<T, 3, false>(c, out) : launch_halo_moments<T, 1, false>(c, out);
+    }
+  }
   const T* fin = (const T*)c->f[c->cur];
   lbm_status s = clear_virtual(c, c->stream);
   if (!s) s = launch_density_and_virtual<T>(c, fin);
   if (s) return s;
-  using C = typename Pop<T>::C;
   k_collide<T, MODE, O><<<node_grid(c->g, 128), 128, 0, c->stream>>>(
       fin, (const C*)c->Pbuf[c->pcur ^ 1], (const C*)c->Pbuf[c->pcur], c->Ubuf[c->cur], c->flags, c->g,
       kphys<C>(c->ph), out);
   return after_launch(c, "k_collide(eval)");
+}
+
+// Four consecutive fields of n values.
+template <typename O>
+EvalOut<O> fields(O* base, int64_t n) {
+  return EvalOut<O>{{base, base + n, base + 2 * n, base + 3 * n}};
 }
 
 template <typename T>
@@ -939,15 +972,18 @@ lbm_status lbm_step_profiled(lbm_ctx* c, int32_t nsteps, double* h_ms, int64_t* 
 lbm_status lbm_moments(lbm_ctx* c, double* rA, double* rB, double* ux, double* uy) {
   if (!c) return LBM_ERR_ARG;
   if (!c->has_geometry || !c->has_fields) return fail(c, LBM_ERR_STATE, "lbm_moments before geometry and fields");
+  if (!rA && !rB && !ux && !uy) return LBM_OK;
   const int64_t N = (int64_t)c->g.nx * c->g.ny;
-  double* tmp = c->stage;  // 4 * N doubles
-  lbm_status s;
-  LBM_DISPATCH(c, s = (do_eval<T, 1>(c, tmp)); break);
-  if (s) return s;
   double* outs[4] = {rA, rB, ux, uy};
+  EvalOut<double> out{{rA, rB, ux, uy}};
+  // an array that is not on 8 bytes gets its field as a copy
+  for (int a = 0; a < 4; ++a)
+    if ((uintptr_t)outs[a] % 8) out.p[a] = c->stage + a * N;
+  lbm_status s;
+  LBM_DISPATCH(c, s = (do_eval<T, 1>(c, out)); break);
   for (int a = 0; a < 4 && !s; ++a)
-    if (outs[a])
-      s = check_cuda(c, cudaMemcpyAsync(outs[a], tmp + a * N, N * 8, cudaMemcpyDeviceToDevice, c->stream),
+    if (outs[a] && out.p[a] != outs[a])
+      s = check_cuda(c, cudaMemcpyAsync(outs[a], out.p[a], N * 8, cudaMemcpyDeviceToDevice, c->stream),
                      "cudaMemcpyAsync");
   return s;
 }
@@ -956,7 +992,8 @@ lbm_status lbm_forces(lbm_ctx* c, double* F) {
   if (!c || !F) return LBM_ERR_ARG;
   if (!c->has_geometry || !c->has_fields) return fail(c, LBM_ERR_STATE, "lbm_forces before geometry and fields");
   lbm_status s;
-  LBM_DISPATCH(c, s = (do_eval<T, 2>(c, F)); break);
+  const EvalOut<double> out = fields(F, (int64_t)c->g.nx * c->g.ny);
+  LBM_DISPATCH(c, s = (do_eval<T, 2>(c, out)); break);
   return s;
 }
 
@@ -1015,12 +1052,14 @@ lbm_status lbm_diagnostics(lbm_ctx* c, const lbm_diag_params* p, lbm_diag* h_out
   a.bridge_x = p->bridge_x;
   a.bridge_y0 = p->bridge_y0;
   lbm_status s;
-  LBM_DISPATCH(c, s = (do_eval<T, 1>(c, c->stage)); break);
+  const EvalOut<double> ev = fields(c->stage, (int64_t)c->g.nx * c->g.ny);
+  LBM_DISPATCH(c, s = (do_eval<T, 1>(c, ev)); break);
   if (s) return s;
   double* out_d = c->dpart + (size_t)DIAG_BLOCKS * DIAG_NRED;
-  k_diag_partial<<<DIAG_BLOCKS, DIAG_THREADS, 0, c->stream>>>(c->stage, c->flags, c->g, a, c->dpart);
+  const int nb = diag_blocks(c->g);
+  k_diag_partial<<<nb, DIAG_THREADS, 0, c->stream>>>(c->stage, c->flags, c->g, a, c->dpart);
   if ((s = after_launch(c, "k_diag_partial"))) return s;
-  k_diag_final<<<1, 32, 0, c->stream>>>(c->dpart, c->stage, c->g, a, out_d);
+  k_diag_final<<<1, 32 * DIAG_NQ, 0, c->stream>>>(c->dpart, nb, c->stage, c->g, a, out_d);
   if ((s = after_launch(c, "k_diag_final"))) return s;
   double q[DIAG_NQ];
   s = check_cuda(c, cudaMemcpyAsync(q, out_d, sizeof(q), cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync");
@@ -1114,7 +1153,8 @@ lbm_status lbm_run_host(lbm_ctx* c, const lbm_wetting_params* w, const uint8_t* 
   if (!s) s = lbm_init_fields(c, in, in + N, nullptr, nullptr);
   if (!s) s = lbm_step(c, nsteps);
   if (s) return s;
-  LBM_DISPATCH(c, s = (do_eval<T, 1>(c, c->stage)); break);
+  const EvalOut<double> ev = fields(c->stage, (int64_t)c->g.nx * c->g.ny);
+  LBM_DISPATCH(c, s = (do_eval<T, 1>(c, ev)); break);
   double* outs[4] = {oA, oB, oux, ouy};
   for (int a = 0; a < 4 && !s; ++a)
     if (outs[a])
@@ -1146,7 +1186,8 @@ lbm_status lbm_run_host_f32(lbm_ctx* c, const lbm_wetting_params* w, const uint8
   if (!s) s = lbm_step(c, nsteps);
   if (s) return s;
   float* out = reinterpret_cast<float*>(c->stage);
-  LBM_DISPATCH(c, s = (do_eval<T, 1, float>(c, out)); break);
+  const EvalOut<float> ev = fields(out, N);
+  LBM_DISPATCH(c, s = (do_eval<T, 1>(c, ev)); break);
   float* outs[4] = {oA, oB, oux, ouy};
   for (int a = 0; a < 4 && !s; ++a)
     if (outs[a])

@@ -507,6 +507,25 @@ __global__ void __launch_bounds__(128) k_virtual_density(C* __restrict__ P, cons
 }
 
 
+// Where an evaluation writes its four fields ([ny][nx] each; null: not wanted).
+template <typename O>
+struct EvalOut {
+  O* p[4];
+  __device__ __forceinline__ void put(int64_t n, O a, O b, O c, O d) const {
+    if (p[0]) p[0][n] = a;
+    if (p[1]) p[1][n] = b;
+    if (p[2]) p[2][n] = c;
+    if (p[3]) p[3][n] = d;
+  }
+};
+
+// The zeros of an evaluation at solid nodes.
+template <typename O>
+__global__ void __launch_bounds__(128) k_zero_solid(const uint16_t* __restrict__ flags, Geo g, EvalOut<O> out) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  if (x < g.nx && (__ldg(flags + g.idx(x, y)) & F_SOLID)) out.put((int64_t)y * g.nx + x, O(0), O(0), O(0), O(0));
+}
+
 // ---- Evaluation of the current state: moments or forces -----------------
 // MODE 1: write the moments (rho^A, rho^B, u of Eq. 3). MODE 2: write the
 // forces (Eq. 5 + Eq. 7). The populations are not changed. O: the type of
@@ -516,7 +535,7 @@ __global__ void __launch_bounds__(128) k_collide(const T* __restrict__ f, const 
                                                  const typename Pop<T>::C* __restrict__ Pref,
                                                  const UPair* __restrict__ Uref,
                                                  const uint16_t* __restrict__ flags, Geo g,
-                                                 PhysK<typename Pop<T>::C> ph, O* __restrict__ out) {
+                                                 PhysK<typename Pop<T>::C> ph, EvalOut<O> out) {
   static_assert(MODE == 1 || MODE == 2, "evaluation modes only");
   using C = typename Pop<T>::C;
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
@@ -524,9 +543,8 @@ __global__ void __launch_bounds__(128) k_collide(const T* __restrict__ f, const 
   const int k = g.idx(x, y);
   const uint16_t fl = flags[k];
   const int64_t n = (int64_t)y * g.nx + x;
-  const int64_t N = (int64_t)g.nx * g.ny;
   if (fl & F_SOLID) {
-    out[n] = 0; out[N + n] = 0; out[2 * N + n] = 0; out[3 * N + n] = 0;
+    out.put(n, O(0), O(0), O(0), O(0));
     return;
   }
   C ref[2][9];
@@ -555,17 +573,10 @@ __global__ void __launch_bounds__(128) k_collide(const T* __restrict__ f, const 
   const C inv = C(1) / (rho[0] + rho[1]);
   const C ux = ((jxA + jxB) + C(0.5) * (F[0][0] + F[1][0])) * inv;
   const C uy = ((jyA + jyB) + C(0.5) * (F[0][1] + F[1][1])) * inv;
-  if (MODE == 1) {
-    out[n] = O(rho[0]);
-    out[N + n] = O(rho[1]);
-    out[2 * N + n] = O(ux);
-    out[3 * N + n] = O(uy);
-  } else {
-    out[n] = O(F[0][0]);
-    out[N + n] = O(F[0][1]);
-    out[2 * N + n] = O(F[1][0]);
-    out[3 * N + n] = O(F[1][1]);
-  }
+  if (MODE == 1)
+    out.put(n, O(rho[0]), O(rho[1]), O(ux), O(uy));
+  else
+    out.put(n, O(F[0][0]), O(F[0][1]), O(F[1][0]), O(F[1][1]));
 }
 
 // Widen n floats to doubles (separate arrays).

@@ -168,6 +168,23 @@ __device__ __forceinline__ void collide2(float2 f[9], float2 rho, float ux, floa
   f[0] = sub2(f[0], acc);
 }
 
+// rho, force and velocity u of Eq. 3 of one fluid node; arguments as for
+// update_pair.
+template <bool GENERAL>
+__device__ __forceinline__ float2 moments_pair(const float2 fp[9], const float2 q[9], uint16_t fl,
+                                               const PhysK<float>& ph, float2& Fx, float2& Fy, float& ux, float& uy) {
+  const float2 rho = density_pair(fp);
+  interaction_force2<GENERAL>(ph, fl, rho, q, Fx, Fy);
+  // momentum of each component as paired differences, then u of Eq. 3
+  const float2 d57 = sub2(fp[5], fp[7]), d86 = sub2(fp[8], fp[6]);
+  const float2 jx = add2(sub2(fp[1], fp[3]), add2(d57, d86));
+  const float2 jy = add2(sub2(fp[2], fp[4]), sub2(d57, d86));
+  const float inv = 1.0f / (rho.x + rho.y);
+  ux = ((jx.x + jx.y) + 0.5f * (Fx.x + Fx.y)) * inv;
+  uy = ((jy.x + jy.y) + 0.5f * (Fy.x + Fy.y)) * inv;
+  return rho;
+}
+
 // Force, velocity and collision of one fluid node (Eqs. 1-5, 7): fp holds
 // the pulled populations f_i of both components on entry and f*_i on exit;
 // q[i] the density plane at x + c_i. GENERAL: the node may have solid
@@ -177,19 +194,9 @@ __device__ __forceinline__ void collide2(float2 f[9], float2 rho, float ux, floa
 template <bool GENERAL>
 __device__ __forceinline__ float2 update_pair(float2 fp[9], const float2 q[9], uint16_t fl,
                                               const PhysK<float>& ph, float& ux_out, float& uy_out) {
-  const float2 rho = density_pair(fp);
   float2 Fx, Fy;
-  interaction_force2<GENERAL>(ph, fl, rho, q, Fx, Fy);
-  // momentum of each component as paired differences, then u of Eq. 3
-  const float2 d57 = sub2(fp[5], fp[7]), d86 = sub2(fp[8], fp[6]);
-  const float2 jx = add2(sub2(fp[1], fp[3]), add2(d57, d86));
-  const float2 jy = add2(sub2(fp[2], fp[4]), sub2(d57, d86));
-  const float inv = 1.0f / (rho.x + rho.y);
-  const float ux = ((jx.x + jx.y) + 0.5f * (Fx.x + Fx.y)) * inv;
-  const float uy = ((jy.x + jy.y) + 0.5f * (Fy.x + Fy.y)) * inv;
-  collide2(fp, rho, ux, uy, Fx, Fy, ph);
-  ux_out = ux;
-  uy_out = uy;
+  const float2 rho = moments_pair<GENERAL>(fp, q, fl, ph, Fx, Fy, ux_out, uy_out);
+  collide2(fp, rho, ux_out, uy_out, Fx, Fy, ph);
   return rho;
 }
 

@@ -162,3 +162,58 @@ def test_batch_of_mixed_members_matches_members_alone(storage, graph):
     for a, b in pairs:  # and alone again
         assert torch.equal(a.step(2).populations(), b.step(2).populations())
     batch.close()
+
+
+@pytest.mark.parametrize("storage,vref", [("fp32", False), ("fp16", False), ("bf16", True)])
+@pytest.mark.parametrize("scheme", ["improved", "llkc"])
+def test_moments_of_halo_contexts_match_the_general_evaluation(storage, vref, scheme):
+    """The halo kernel's moments against the density, Eq. 8 and evaluation
+    passes of a two-pass context, on a ragged grid; each array may be left
+    out or lie on any byte."""
+    nx, ny = 75, 43
+    wet = IMPROVED if scheme == "improved" else SCHEMES[scheme]
+    mask = inputs.random_solid_mask(nx, ny, seed=4, fraction=0.15, periodic_x=True, periodic_y=False)
+    rA, rB, ux, uy = inputs.random_fields(nx, ny, 6, umax=0.05)
+    sims = []
+    for kernel in ("auto", "two_pass"):
+        sim = lbm.Simulation(nx, ny, storage=storage, velocity_refs=vref, kernel=kernel, periodic_x=True)
+        sim.set_geometry(mask).set_wetting(wet[0], **wet[1]).init_fields(rA, rB, ux, uy)
+        sims.append(sim.step(3))
+    a, b = (torch.cat([m.reshape(-1) for m in s.moments()]) for s in sims)
+    assert torch.equal(a, b)
+    n = nx * ny * 8
+    raw = torch.full((n + 16,), 7, dtype=torch.uint8, device="cuda")
+    for off, field in ((0, 2), (3, 1)):
+        ptr = [None] * 4
+        ptr[field] = raw.data_ptr() + off
+        assert sims[0].lib.lbm_moments(sims[0].h, *ptr) == lbm.OK
+        got = raw[off:off + n].clone().view(torch.float64)
+        assert torch.equal(got, a[field * nx * ny:(field + 1) * nx * ny])
+        assert torch.all(raw[off + n:] == 7)
+
+
+@pytest.mark.parametrize("nx,ny", [(8, 8), (300, 200), (512, 300)])
+def test_diagnostics_at_block_edges(nx, ny):
+    """Fewer blocks than the reduction's 256, about one node per thread, and
+    several, with a bridge longer than the 32 rows of one scan: against the
+    same sums of the moments."""
+    mask = np.zeros((ny, nx), np.uint8)
+    rA = np.full((ny, nx), 0.05)
+    rA[: ny * 2 // 3, : nx * 2 // 3] = 1.0
+    sim = lbm.Simulation(nx, ny, storage="fp64", kernel="two_pass", periodic_x=True, periodic_y=True)
+    sim.set_geometry(mask).set_wetting("martys_chen").init_fields(rA, 1.05 - rA, np.full((ny, nx), 0.01),
+                                                                 np.zeros((ny, nx)))
+    r, _, u = (m.cpu().numpy() for m in sim.moments())
+    d = sim.diagnostics(level=0.5, rho_out=0.055, bridge=(1, 1), wall_point=(0.0, -100.0))
+    w = np.maximum(r - 0.055, 0.0)
+    yy, xx = np.mgrid[0:ny, 0:nx]
+    assert abs(d["weight"] - w.sum()) < 1e-9 * w.sum()
+    assert abs(d["com"][0] - (w * xx).sum() / w.sum()) < 1e-9 * nx
+    assert abs(d["com"][1] - (w * yy).sum() / w.sum()) < 1e-9 * ny
+    assert abs(d["max_u"] - np.sqrt((u ** 2).sum(0).max())) < 1e-12
+    above = r >= 0.5
+    cross = (above[:, :-1] != above[:, 1:]).sum() + (above[:-1] != above[1:]).sum()
+    assert d["contour_points"] == cross and d["nonfinite_nodes"] == 0
+    y1 = ny * 2 // 3  # the first row below the level
+    t = (r[y1 - 1, 1] - 0.5) / (r[y1 - 1, 1] - r[y1, 1])
+    assert abs(d["bridge_radius"] - (y1 - 1 + t - 0.5)) < 1e-9
