@@ -477,20 +477,48 @@ bool wants_halo(const lbm_ctx* c) {
          (c->prm.kernel == LBM_KERNEL_AUTO && c->prm.storage != LBM_STORE_FP64);
 }
 
-// The halo schedule's lists for the installed geometry, in the unused parts
-// of the workspace: behind the interface cells (their arrays have room for
-// every node) and in the area halo contexts keep. Leaves halo_ready false,
-// and the two-pass schedule runs instead, if they do not fit. Synchronises.
-lbm_status build_halo_lists(lbm_ctx* c) {
+// The halo schedule's lists for the installed geometry go to the unused parts
+// of the workspace: the area halo contexts keep, and behind the interface
+// cells (their arrays have room for every node). Where they do not fit,
+// halo_ready stays false and the two-pass schedule runs.
+//
+// First half, enqueued before lbm_set_geometry reads its counts back: the
+// tiles' sizes, scanned to offsets (totals at small[6 ... 8]), in arrays at
+// the start of the area or at the end of the interface arrays.
+lbm_status count_halo_lists(lbm_ctx* c) {
   const Geo& g = c->g;
-  c->halo_ready = false;
-  if (!c->hmaps_ok || c->n_fluid == 0) return LBM_OK;
-  const int ntx = (g.nx + HALO_W - 1) / HALO_W;
   const int H = halo_rows((int)elem_size(c->prm.storage));
   const int64_t nt = halo_tile_count(g, H);
-  if (nt * HALO_RW * (H + 6) > 0x7fffffff) return LBM_OK;  // 32-bit places in the lists
-  char* from[2] = {(char*)align_up((size_t)(c->iface_mask + c->n_iface), 256), c->halo_area[0]};
-  char* const end[2] = {c->iface_end, c->halo_area[1]};
+  c->halo_off = nullptr;
+  if (!wants_halo(c) || !c->hmaps_ok || nt * HALO_RW * (H + 6) > 0x7fffffff) return LBM_OK;  // 32-bit places in the lists
+  const size_t each = align_up((size_t)nt * 4, 256);
+  if ((size_t)(c->halo_area[1] - c->halo_area[0]) >= 3 * each)
+    c->halo_off = c->halo_area[0];
+  else if ((size_t)c->if_capacity * 4 >= 3 * each)  // inside the second interface array
+    c->halo_off = c->iface_end - 3 * each;
+  else
+    return LBM_OK;
+  int* off = (int*)c->halo_off;
+  k_halo_lists<false><<<(unsigned)nt, HALO_LIST_THREADS, 0, c->stream>>>(
+      c->flags, g, (g.nx + HALO_W - 1) / HALO_W, H, off, off + each / 4, off + each / 2, nullptr, nullptr, nullptr);
+  lbm_status s = after_launch(c, "k_halo_lists(count)");
+  if (s) return s;
+  k_scan3<<<3, 1024, 0, c->stream>>>(off, off + each / 4, off + each / 2, (int)nt, c->small + 6);
+  return after_launch(c, "k_scan3");
+}
+
+// Second half, with the totals at hand: n_entries, n_cells, n_work.
+lbm_status write_halo_lists(lbm_ctx* c, const int* totals) {
+  if (!c->halo_off || c->n_fluid == 0) return LBM_OK;
+  const Geo& g = c->g;
+  const int H = halo_rows((int)elem_size(c->prm.storage));
+  const int64_t nt = halo_tile_count(g, H);
+  const size_t each = align_up((size_t)nt * 4, 256);
+  const bool in_area = c->halo_off == c->halo_area[0];
+  char* from[2] = {(char*)align_up((size_t)(c->iface_mask + c->n_iface), 256),
+                   in_area ? c->halo_area[0] + 3 * each : c->halo_area[0]};
+  char* const end[2] = {in_area ? c->iface_end : c->halo_off, c->halo_area[1]};
+  if ((char*)(c->iface_mask + c->n_iface) > end[0]) return LBM_OK;  // the offsets would be overwritten
   auto take = [&](size_t bytes) -> char* {
     for (int r = 1; r >= 0; --r)
       if (from[r] < end[r] && (size_t)(end[r] - from[r]) >= bytes) {
@@ -500,30 +528,16 @@ lbm_status build_halo_lists(lbm_ctx* c) {
       }
     return nullptr;
   };
-  HaloTile* work = (HaloTile*)take((size_t)nt * sizeof(HaloTile));
-  int* off[3];  // entries, cells, work list
-  for (int i = 0; i < 3; ++i)
-    if (!(off[i] = (int*)take((size_t)nt * 4))) return LBM_OK;
-  if (!work) return LBM_OK;
-  lbm_status s;
-  k_halo_lists<<<(unsigned)nt, HALO_LIST_THREADS, 0, c->stream>>>(c->flags, g, ntx, H, off[0], off[1], off[2], nullptr,
-                                                                  nullptr, nullptr);
-  if ((s = after_launch(c, "k_halo_lists(count)"))) return s;
-  for (int i = 0; i < 3; ++i) {
-    k_iface_scan<<<1, 1024, 0, c->stream>>>(off[i], (int)nt, c->small + 6 + i);
-    if ((s = after_launch(c, "k_iface_scan(halo)"))) return s;
-  }
-  int h[3];
-  s = check_cuda(c, cudaMemcpyAsync(h, c->small + 6, sizeof(h), cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync");
-  if (!s) s = check_cuda(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+  HaloTile* work = (HaloTile*)take((size_t)totals[2] * sizeof(HaloTile));
+  uint32_t* entries = (uint32_t*)take((size_t)totals[0] * 4);
+  uint2* cells = (uint2*)take((size_t)(totals[1] > 0 ? totals[1] : 1) * 8);
+  if (!work || !entries || !cells) return LBM_OK;
+  int* off = (int*)c->halo_off;
+  k_halo_lists<true><<<(unsigned)nt, HALO_LIST_THREADS, 0, c->stream>>>(
+      c->flags, g, (g.nx + HALO_W - 1) / HALO_W, H, off, off + each / 4, off + each / 2, work, entries, cells);
+  lbm_status s = after_launch(c, "k_halo_lists(write)");
   if (s) return s;
-  uint32_t* entries = (uint32_t*)take((size_t)h[0] * 4);
-  uint2* cells = (uint2*)take((size_t)(h[1] > 0 ? h[1] : 1) * 8);
-  if (!entries || !cells) return LBM_OK;
-  k_halo_lists<<<(unsigned)nt, HALO_LIST_THREADS, 0, c->stream>>>(c->flags, g, ntx, H, off[0], off[1], off[2], work,
-                                                                  entries, cells);
-  if ((s = after_launch(c, "k_halo_lists(write)"))) return s;
-  c->halo = HaloLists{work, h[2], entries, cells};
+  c->halo = HaloLists{work, totals[2], entries, cells};
   c->halo_ready = true;
   return LBM_OK;
 }
@@ -845,7 +859,9 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const uint8_t* d_mask) {
   s = check_cuda(c, cudaMemsetAsync(c->Pbase, 0, (c->Pbuf[2] ? 6 : 4) * (size_t)g.plane * compute_size(c->prm.storage),
                                     c->stream), "cudaMemsetAsync");
   if (s) return s;
-  int h[3];
+  c->halo_ready = false;
+  if ((s = count_halo_lists(c))) return s;
+  int h[9];
   s = check_cuda(c, cudaMemcpyAsync(h, c->small, sizeof(h), cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync");
   if (!s) s = check_cuda(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
   if (s) return s;
@@ -861,8 +877,7 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const uint8_t* d_mask) {
   }
   c->tiles_built = false;
   if (c->n_tiles > 0 && c->prm.kernel != LBM_KERNEL_AUTO && (s = build_tile_lists(c, c->stream))) return s;
-  c->halo_ready = false;
-  if (wants_halo(c) && (s = build_halo_lists(c))) return s;
+  if ((s = write_halo_lists(c, h + 6))) return s;
   c->has_geometry = true;
   return LBM_OK;
 }

@@ -100,18 +100,23 @@ static __global__ void __launch_bounds__(SCAN_BLOCK) k_class_count(const uint16_
   if (threadIdx.x == 0) counts[blockIdx.x] = c;
 }
 
-// Pass 2: exclusive scan of the per-block counts in one block (fixed order).
-static __global__ void __launch_bounds__(1024) k_iface_scan(int* __restrict__ counts, int nblocks,
-                                                     int* __restrict__ total) {
-  __shared__ int carry;
+// Exclusive scan of v[0 ... n) in place by one block of 1024 threads (fixed
+// order), four consecutive values a thread and round; returns the total.
+__device__ __forceinline__ int scan_block(int* __restrict__ v, int n) {
   __shared__ int warp_sums[32];
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < nblocks; base += 1024) {
-    const int i = base + threadIdx.x;
-    const int v = i < nblocks ? counts[i] : 0;
-    int x = v;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int carry = 0;
+  for (int base = 0; base < n; base += 4096) {
+    const int i = base + 4 * threadIdx.x;
+    int a[4], sum = 0;
+    if (i + 4 <= n) {
+      const int4 q = *reinterpret_cast<const int4*>(v + i);
+      a[0] = q.x; a[1] = q.y; a[2] = q.z; a[3] = q.w;
+    } else {
+      for (int j = 0; j < 4; ++j) a[j] = i + j < n ? v[i + j] : 0;
+    }
+    for (int j = 0; j < 4; ++j) sum += a[j];
+    int x = sum;
     for (int o = 1; o < 32; o <<= 1) {
       const int t = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += t;
@@ -127,13 +132,35 @@ static __global__ void __launch_bounds__(1024) k_iface_scan(int* __restrict__ co
       warp_sums[lane] = s;
     }
     __syncthreads();
-    const int incl = x + (wid ? warp_sums[wid - 1] : 0);
-    if (i < nblocks) counts[i] = carry + incl - v;
-    __syncthreads();
-    if (threadIdx.x == 1023) carry += incl;
+    int before = carry + x - sum + (wid ? warp_sums[wid - 1] : 0);
+    for (int j = 0; j < 4; ++j) {
+      const int t = a[j];
+      a[j] = before;
+      before += t;
+    }
+    if (i + 4 <= n)
+      *reinterpret_cast<int4*>(v + i) = make_int4(a[0], a[1], a[2], a[3]);
+    else
+      for (int j = 0; j < 4; ++j)
+        if (i + j < n) v[i + j] = a[j];
+    carry += warp_sums[31];
     __syncthreads();
   }
-  if (threadIdx.x == 0) *total = carry;
+  return carry;
+}
+
+// Pass 2: exclusive scan of the per-block counts (a 16-byte aligned array).
+static __global__ void __launch_bounds__(1024) k_iface_scan(int* __restrict__ counts, int nblocks,
+                                                     int* __restrict__ total) {
+  const int t = scan_block(counts, nblocks);
+  if (threadIdx.x == 0) *total = t;
+}
+
+// Three arrays of n values, one block each; totals to total[0 ... 2].
+static __global__ void __launch_bounds__(1024) k_scan3(int* __restrict__ a, int* __restrict__ b, int* __restrict__ c,
+                                                       int n, int* __restrict__ total) {
+  const int t = scan_block(blockIdx.x == 0 ? a : blockIdx.x == 1 ? b : c, n);
+  if (threadIdx.x == 0) total[blockIdx.x] = t;
 }
 
 // Pass 3: write the padded indices of the nodes of class cls in node order,

@@ -117,67 +117,87 @@ __device__ __forceinline__ uint32_t fluid_mask25(const uint16_t* __restrict__ fl
   return m;
 }
 
-// One CTA per tile, two passes over the same fixed order. Count pass
-// (entries == nullptr): the tile's sizes and whether it owns nodes, which the
-// scans turn into offsets and places in the work list. Write pass: work list,
-// entries and cells.
-static __global__ void __launch_bounds__(HALO_LIST_THREADS)
-    k_halo_lists(const uint16_t* __restrict__ flags, Geo g, int ntx, int H, int* __restrict__ eoff, int* __restrict__ ioff,
-                 int* __restrict__ woff, HaloTile* __restrict__ work, uint32_t* __restrict__ entries,
-                 uint2* __restrict__ cells) {
-  __shared__ int warp_cnt[HALO_LIST_THREADS / 32];
+// One CTA per tile, two passes over the same fixed order (a slot per thread and
+// chunk, its place by a scan over chunks and warps for each of the four lists:
+// own nodes, ring 1, rings 2 and 3, interface-solid cells). Count pass: the
+// tile's sizes and whether it owns nodes, which the scans turn into offsets
+// and places in the work list. Write pass: work list, entries and cells.
+template <bool WRITE>
+__global__ void __launch_bounds__(HALO_LIST_THREADS)
+    k_halo_lists(const uint16_t* __restrict__ flags, Geo g, int ntx, int H, int* __restrict__ eoff,
+                 int* __restrict__ ioff, int* __restrict__ woff, HaloTile* __restrict__ work,
+                 uint32_t* __restrict__ entries, uint2* __restrict__ cells) {
+  constexpr int CHUNKS = 4, WARPS = HALO_LIST_THREADS / 32;
+  static_assert(CHUNKS * HALO_LIST_THREADS >= HALO_RW * (HALO_H + 6) &&
+                    CHUNKS * HALO_LIST_THREADS >= HALO_RW * (HALO_H16 + 6) && CHUNKS * WARPS == 32,
+                "a region's slots, and one warp's scan over chunks and warps");
+  __shared__ int place[4][32];
+  __shared__ int total[4];
   const int tile = blockIdx.x;
   const int x0 = (tile % ntx) * HALO_W, y0 = (tile / ntx) * H;
   const int tw = min(HALO_W, g.nx - x0), th = min(H, g.ny - y0), RS = HALO_RW * (H + 6);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int base = 0;
-  int cum[4];
-  for (int round = 0; round < 4; ++round) {  // own nodes, ring 1, rings 2 and 3, interface-solid cells
-    if (round == 3) base = 0;
-    for (int c0 = 0; c0 < RS; c0 += HALO_LIST_THREADS) {
-      const int slot = c0 + threadIdx.x;
-      const int row = slot / HALO_RW, col = slot - row * HALO_RW;
-      // distance (max norm) from the owned rectangle
-      const int dc = col < 3 ? 3 - col : (col >= 3 + tw ? col - (2 + tw) : 0);
-      const int dr = row < 3 ? 3 - row : (row >= 3 + th ? row - (2 + th) : 0);
-      const int ring = slot < RS ? max(dc, dr) : 99;
-      const int x = x0 - 3 + col, y = y0 - 3 + row;
-      const uint16_t fl = ring <= 3 ? flags[g.idx(x, y)] : F_SOLID;
-      const int cls = ring >= 2 ? 2 : ring;
-      const bool hit = round == 3 ? ring <= 1 && (fl & F_IFACE) : !(fl & F_SOLID) && cls == round;
-      const unsigned ball = __ballot_sync(0xffffffffu, hit);
-      if (lane == 0) warp_cnt[wid] = __popc(ball);
-      __syncthreads();
-      int before = 0, all = 0;
-      for (int w = 0; w < HALO_LIST_THREADS / 32; ++w) {
-        const int v = warp_cnt[w];
-        before += w < wid ? v : 0;
-        all += v;
-      }
-      if (entries && hit && (round == 0 || cum[0] > 0)) {
-        const int pos = base + before + __popc(ball & ((1u << lane) - 1u));
-        uint32_t e = (uint32_t)(col + 1) | (uint32_t)(row + 1) << 6;
-        if (round == 3) {
-          cells[ioff[tile] + pos] = make_uint2(e, fluid_mask25(flags, g, g.idx(x, y)));
-        } else {
-          e |= (uint32_t)(fl & NB_ANY) << HE_NB_SHIFT;
-          if (ring == 0 && near_border(g, x, y)) e |= HE_BORDER;
-          entries[eoff[tile] + pos] = e;
-        }
-      }
-      base += all;
-      __syncthreads();
+  uint16_t fl[CHUNKS];
+  int list[CHUNKS];  // 0 ... 3, or -1
+#pragma unroll
+  for (int c = 0; c < CHUNKS; ++c) {
+    const int slot = c * HALO_LIST_THREADS + threadIdx.x;
+    const int row = slot / HALO_RW, col = slot - row * HALO_RW;
+    // distance (max norm) from the owned rectangle
+    const int dc = col < 3 ? 3 - col : (col >= 3 + tw ? col - (2 + tw) : 0);
+    const int dr = row < 3 ? 3 - row : (row >= 3 + th ? row - (2 + th) : 0);
+    const int ring = slot < RS ? max(dc, dr) : 99;
+    fl[c] = ring <= 3 ? flags[g.idx(x0 - 3 + col, y0 - 3 + row)] : F_SOLID;
+    list[c] = !(fl[c] & F_SOLID) ? min(ring, 2) : ring <= 1 && (fl[c] & F_IFACE) ? 3 : -1;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const unsigned ball = __ballot_sync(0xffffffffu, list[c] == l);
+      if (lane == 0) place[l][c * WARPS + wid] = __popc(ball);
     }
-    cum[round] = base;
   }
-  if (threadIdx.x == 0) {
-    if (!entries) {
-      eoff[tile] = cum[0] > 0 ? (cum[2] + 3) & ~3 : 0;
-      ioff[tile] = cum[0] > 0 ? cum[3] : 0;
-      woff[tile] = cum[0] > 0;
-    } else if (cum[0] > 0) {
-      work[woff[tile]] = HaloTile{make_int4(cum[0], cum[1], cum[2], cum[3]), eoff[tile], ioff[tile], tile, 0};
+  __syncthreads();
+  if (wid < 4) {
+    const int v = place[wid][lane];
+    int x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += t;
     }
+    place[wid][lane] = x - v;
+    if (lane == 31) total[wid] = x;
+  }
+  __syncthreads();
+  const int n0 = total[0], n1 = n0 + total[1], n3 = n1 + total[2];
+  if (!WRITE) {
+    if (threadIdx.x == 0) {
+      eoff[tile] = n0 > 0 ? (n3 + 3) & ~3 : 0;
+      ioff[tile] = n0 > 0 ? total[3] : 0;
+      woff[tile] = n0 > 0;
+    }
+    return;
+  }
+  if (n0 == 0) return;
+  const int e0 = eoff[tile], i0 = ioff[tile];
+  if (threadIdx.x == 0) work[woff[tile]] = HaloTile{make_int4(n0, n1, n3, total[3]), e0, i0, tile, 0};
+#pragma unroll
+  for (int c = 0; c < CHUNKS; ++c) {
+    const int slot = c * HALO_LIST_THREADS + threadIdx.x;
+    const int row = slot / HALO_RW, col = slot - row * HALO_RW;
+    const uint32_t at = (uint32_t)(col + 1) | (uint32_t)(row + 1) << 6;
+    int pos = 0;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const unsigned ball = __ballot_sync(0xffffffffu, list[c] == l);
+      if (list[c] == l)
+        pos = place[l][c * WARPS + wid] + __popc(ball & ((1u << lane) - 1u)) + (l == 1 ? n0 : l == 2 ? n1 : 0);
+    }
+    if (list[c] < 0) continue;
+    const int x = x0 - 3 + col, y = y0 - 3 + row;
+    if (list[c] == 3)
+      cells[i0 + pos] = make_uint2(at, fluid_mask25(flags, g, g.idx(x, y)));
+    else
+      entries[e0 + pos] = at | (uint32_t)(fl[c] & NB_ANY) << HE_NB_SHIFT |
+                          (list[c] == 0 && near_border(g, x, y) ? HE_BORDER : 0u);
   }
 }
 

@@ -68,6 +68,7 @@ struct lbm_ctx {
   bool halo_smem_set[2];  // k_halo's dynamic shared memory limit raised (one ring, three rings)
   uint32_t tma_extra_tx;  // test hook of the TMA schedule's bounded wait (lbm_debug_tma_expect_extra); 0
   lbm::HaloLists halo;  // halo schedule: per-tile lists, placed by lbm_set_geometry
+  char* halo_off;      // the tiles' offsets while the lists are built (null: no lists)
   char* halo_area[2];  // an area of the workspace for these lists (may be empty)
   char* iface_end;     // end of the interface arrays, whose unused part also holds them
   int* scan_counts;    // per-block interface counts / offsets
