@@ -267,8 +267,8 @@ lbm_status launch_virtual(lbm_ctx* c, C* P) {
   if (c->ph.bc != BC_VAVG || c->n_iface == 0) return LBM_OK;
   c->virt_written = true;
   return launch(c, LBM_KC_VIRTUAL, "k_virtual_density", [&] {
-    k_virtual_density<C><<<(c->n_iface + 127) / 128, 128, 0, c->stream>>>(P, c->iface_mask, c->iface_list, c->n_iface,
-                                                                           c->g, kphys<C>(c->ph));
+    launch_pdl(k_virtual_density<C>, (c->n_iface + 127) / 128, 128, 0, c->stream, P, c->iface_mask, c->iface_list,
+               c->n_iface, c->g, kphys<C>(c->ph));
   });
 }
 
@@ -307,15 +307,15 @@ lbm_status step_two_pass(lbm_ctx* c, int nsteps) {
     const bool vr = kDev<T> && c->prm.velocity_refs;
     lbm_status s = launch(c, LBM_KC_DENSITY, "k_density_list", [&] {
       auto kd = vr ? k_density_list<T, kDev<T>> : k_density_list<T, false>;
-      kd<<<nb, 256, 0, c->stream>>>(fin, P, Pref, c->Ubuf[c->cur], c->flags, c->fluid_list, c->n_fluid, c->g,
-                                    kphys<C>(c->ph));
+      launch_pdl(kd, nb, 256, 0, c->stream, fin, P, Pref, c->Ubuf[c->cur], c->flags, c->fluid_list, c->n_fluid, c->g,
+                 kphys<C>(c->ph));
     });
     if (s) return s;
     if ((s = launch_virtual<C>(c, P))) return s;
     s = launch(c, LBM_KC_COLLIDE, "k_collide_list", [&] {
       auto kc = vr ? k_collide_list<T, kDev<T>> : k_collide_list<T, false>;
-      kc<<<nbc, ntc, 0, c->stream>>>(fin, fout, P, Pref, c->Ubuf[c->cur], c->Ubuf[c->cur ^ 1], c->flags,
-                                                 c->fluid_list, c->n_fluid, c->g, kphys<C>(c->ph));
+      launch_pdl(kc, nbc, ntc, 0, c->stream, fin, fout, P, Pref, c->Ubuf[c->cur], c->Ubuf[c->cur ^ 1], c->flags,
+                 c->fluid_list, c->n_fluid, c->g, kphys<C>(c->ph));
     });
     if (s) return s;
     c->cur ^= 1;
@@ -449,7 +449,8 @@ bool encode_halo_map(CUtensorMap* map, const Geo& g, void* base, int node_bytes,
   const cuuint32_t m = node_bytes > 8 ? node_bytes / 8 : 1;  // elements per node
   const cuuint64_t dim[3] = {(cuuint64_t)m * g.px, (cuuint64_t)g.py, (cuuint64_t)planes};
   const cuuint64_t str[2] = {(cuuint64_t)node_bytes * g.px, (cuuint64_t)node_bytes * g.plane};
-  const cuuint32_t box[3] = {(cuuint32_t)(m * (HALO_W + 2 * O)), (cuuint32_t)(H + 2 * (R + 1)), 1};
+  const int rows = H + 2 * R + (planes == 1 ? 2 : 0);  // references: a row more on each side
+  const cuuint32_t box[3] = {(cuuint32_t)(m * (HALO_W + 2 * O)), (cuuint32_t)rows, 1};
   const cuuint32_t ones[3] = {1, 1, 1};
   return enc(map, node_bytes >= 8 ? CU_TENSOR_MAP_DATA_TYPE_UINT64 : CU_TENSOR_MAP_DATA_TYPE_UINT32, planes > 1 ? 3 : 2,
              base, dim, str, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -557,7 +558,7 @@ lbm_status launch_halo(lbm_ctx* c) {
   const CUtensorMap* mr = kDev<T> ? &c->hmap_ref[R == 3][c->Ubuf[0] ? c->cur : c->pcur] : mf;
   const HaloArgs<T> a = halo_args<T>(c, c->cur, c->pcur);
   return launch(c, LBM_KC_FUSED, "k_halo", [&] {
-    kern<<<c->halo.n_work, HALO_THREADS, S::BYTES, c->stream>>>(*mf, *mr, a, c->halo.work, c->tma_extra_tx);
+    launch_pdl(kern, c->halo.n_work, halo_threads<R>, S::BYTES, c->stream, *mf, *mr, a, c->halo.work, c->tma_extra_tx);
   });
 }
 
@@ -622,7 +623,7 @@ lbm_status launch_halo_moments(lbm_ctx* c, const EvalOut<O>& out) {
   const CUtensorMap* mr = kDev<T> ? &c->hmap_ref[R == 3][c->Ubuf[0] ? c->cur : c->pcur] : mf;
   k_zero_solid<O><<<node_grid(c->g, 128), 128, 0, c->stream>>>(c->flags, c->g, out);
   if ((s = after_launch(c, "k_zero_solid"))) return s;
-  kern<<<c->halo.n_work, HALO_THREADS, S::BYTES, c->stream>>>(*mf, *mr, halo_args<T>(c, c->cur, c->pcur), c->halo.work,
+  kern<<<c->halo.n_work, halo_threads<R>, S::BYTES, c->stream>>>(*mf, *mr, halo_args<T>(c, c->cur, c->pcur), c->halo.work,
                                                               c->tma_extra_tx, out);
   c->halo_used = true;
   return after_launch(c, "k_halo_moments");

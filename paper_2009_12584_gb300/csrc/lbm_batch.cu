@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(256) k_density_batch(const BatchDesc<typename 
   if (t < D.n_fluid)
     density_node<T>((const T*)D.f[cur], (C*)D.Pbuf[pcur ^ into], (const C*)D.Pbuf[pcur], VR ? D.Ubuf[cur] : nullptr,
                     D.flags,
-                    D.fluid_list, t, D.g);
+                    (unsigned)__ldg(D.fluid_list + t), D.g);
 }
 
 // Eq. 8 into the plane the next pass reads: Pbuf[pcur ^ into] (into as
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(128) k_virtual_batch(const BatchDesc<C>* __res
   const BatchDesc<C>& D = d[b.x];
   const int pcur = D.pcur ^ parity;
   const int t = b.y + threadIdx.x;
-  if (t < D.n_iface) virtual_density_node<C>((C*)D.Pbuf[pcur ^ into], D.iface_mask, D.iface_list, t, D.g, D.ph);
+  if (t < D.n_iface) virtual_density_node<C>((C*)D.Pbuf[pcur ^ into], D.iface_mask[t], D.iface_list[t], D.g, D.ph);
 }
 
 // Tiled single-pass step of every member: CTA -> (member, tile).
@@ -94,9 +94,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_collide_batch(c
   const int2 b = blk[blockIdx.x];
   const BatchDesc<C>& D = d[b.x];
   const int cur = D.cur ^ parity, pcur = D.pcur ^ parity;
+  const int t = b.y + threadIdx.x;
+  const bool valid = t < D.n_fluid;
   collide_node<T>((const T*)D.f[cur], (T*)D.f[cur ^ 1], (const C*)D.Pbuf[pcur ^ 1], (const C*)D.Pbuf[pcur],
-                  VR ? D.Ubuf[cur] : nullptr, VR ? D.Ubuf[cur ^ 1] : nullptr, D.flags, D.fluid_list, b.y + threadIdx.x,
-                  D.n_fluid, D.g, D.ph);
+                  VR ? D.Ubuf[cur] : nullptr, VR ? D.Ubuf[cur ^ 1] : nullptr, D.flags,
+                  valid ? (unsigned)__ldg(D.fluid_list + t) : 0u, valid, D.g, D.ph);
 }
 
 // The halo step of every member with R rings; 45 simulations of 400 x 200 in
@@ -107,16 +109,17 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_collide_batch(c
 // (populations of buffers 0 and 1, references of buffers 0 and 1), in global
 // memory, hence the fence. cur: two indices per member, into its maps.
 template <typename T, int R, bool VR>
-__global__ void __launch_bounds__(HALO_THREADS, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
+__global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
     k_halo_batch(const HaloArgs<T>* __restrict__ args, const CUtensorMap* __restrict__ maps,
                  const HaloTile* __restrict__ work, const int2* __restrict__ cur, const int* __restrict__ stop,
                  int parity) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ HaloArgs<T> a;
-  static_assert(sizeof(a) % 4 == 0 && sizeof(a) / 4 <= HALO_THREADS, "one thread per word");
+  static_assert(sizeof(a) % 4 == 0 && sizeof(a) / 4 <= halo_threads<R>, "one thread per word");
   HaloTile h;
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
+  pdl_wait();  // the launch before; what is read above it does not write
   if (*(const volatile int*)stop) return;
   if (threadIdx.x == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(work + blockIdx.x + HALO_AHEAD));
@@ -149,6 +152,7 @@ __global__ void __launch_bounds__(256) k_halo_gather(const HaloTile* __restrict_
 
 // Members of a halo launch: rings of the step and velocity references.
 constexpr int HALO_CLASSES = 4;
+int halo_block(int cls) { return cls < 2 ? halo_threads<1> : halo_threads<3>; }
 int halo_class(const lbm_ctx* c) { return (halo_reach(c->ph) == 3 ? 2 : 0) + (c->Ubuf[0] ? 1 : 0); }
 template <typename T>
 const void* halo_kernel(int cls) {
@@ -417,8 +421,17 @@ lbm_status launch_step(lbm_batch* b, int p) {
     for (int k = 0; k < HALO_CLASSES; ++k) {
       if (b->n_hwork[k] == 0) continue;
       HaloLaunch<T> L(b, k, p);
-      lbm_status st = bcuda(b, cudaLaunchKernel(halo_kernel<T>(k), dim3(b->n_hwork[k]), dim3(HALO_THREADS), L.args,
-                                                halo_smem<T>(k), b->stream), "batched halo launch");
+      cudaLaunchAttribute at;
+      at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      at.val.programmaticStreamSerializationAllowed = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(b->n_hwork[k]);
+      cfg.blockDim = dim3(halo_block(k));
+      cfg.dynamicSmemBytes = halo_smem<T>(k);
+      cfg.stream = b->stream;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      lbm_status st = bcuda(b, cudaLaunchKernelExC(&cfg, halo_kernel<T>(k), L.args), "batched halo launch");
       if (st) return st;
       b->launches++;
     }
@@ -490,7 +503,7 @@ lbm_status build_graph(lbm_batch* b, int steps) {
         memset(&kp, 0, sizeof(kp));
         kp.func = (void*)halo_kernel<T>(q);
         kp.gridDim = dim3(b->n_hwork[q]);
-        kp.blockDim = dim3(HALO_THREADS);
+        kp.blockDim = dim3(halo_block(q));
         kp.sharedMemBytes = (unsigned)halo_smem<T>(q);
         kp.kernelParams = L.args;
         cudaGraphNode_t node;

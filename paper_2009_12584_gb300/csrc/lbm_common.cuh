@@ -27,6 +27,32 @@ __host__ __device__ constexpr C w_of(int i) {
   return i == 0 ? C(4) / C(9) : (i <= 4 ? C(1) / C(9) : C(1) / C(36));
 }
 
+// Programmatic dependent launch: a kernel of a step may start (and load what no
+// kernel of a step writes: lists, flags, tables) while the one before it in
+// the stream drains. pdl_wait returns when all work before the launch is
+// complete and visible; only then may the next kernel start (so that its
+// first part can rely on everything before this one). Both do nothing in a
+// launch without the attribute.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Ghost layer width around the owned nx * ny nodes. Periodic axes hold
 // copies of the opposite border there; walled axes hold solid cells. Four
 // layers cover the widest stencil of the step (Eq. 8's D2Q25 reach of 2 plus

@@ -43,24 +43,27 @@
 namespace lbm {
 
 constexpr int HALO_W = 32;  // owned columns of a tile
-// Owned rows and threads: three windows of three rings, or four of one ring,
-// fill an SM's shared memory, and the threads take the tile's own nodes of a
-// porous medium (60% fluid) in about one round at 72 to 80 registers each.
-// 4096^2 porous, us per step, improved scheme / LLKC: FP32 with 14 rows and
-// 224 threads 406 / 363 (256 threads 411 / 363, 12 rows 429 / 371, 16 rows
-// 480 / 383); FP16 with 20 rows and 224 threads 387 / 330 (192 threads 388 /
-// 338, 256 threads 384 / 343, 16 rows and 256 threads 400 / 346, 24 rows 356 /
-// 352, but with velocity references 515 against 464).
-constexpr int HALO_H = 14, HALO_H16 = 20;
+// Owned rows: three windows of three rings, or four of one ring, fill an SM's
+// shared memory. Threads: the tile's own nodes of a porous medium (60% fluid)
+// take one round or two at 72 to 80 registers each, R = 1 with four CTAs per
+// SM, R = 3 with three. 4096^2 porous, us per step, improved scheme / LLKC:
+// FP32 with 224 threads 400 / 357, with 256 395 / 367; FP16 375 / 315 and 367 /
+// 335, with velocity references 449 and 433 (improved scheme). With 14 (20)
+// rows and the window rows of all directions copied for each: FP32 406 / 363,
+// FP16 387 / 330. Tiles of 28 x 18 (24) nodes, whose window rows take fewer
+// 128-byte lines: FP32 404 / 374, FP16 387 / 338.
+constexpr int HALO_H = 16, HALO_H16 = 20;
 template <typename T>
 constexpr int halo_h = sizeof(T) == 2 ? HALO_H16 : HALO_H;
 __host__ __device__ inline int halo_rows(int elem_size) { return elem_size == 2 ? HALO_H16 : HALO_H; }
 constexpr int HALO_O = 4;                        // entries count columns and rows from (x0 - 4, y0 - 4)
-constexpr int HALO_THREADS = 224;
+template <int R>
+constexpr int halo_threads = R == 1 ? 224 : 256;
 constexpr int HALO_AHEAD = 512;  // CTAs between one and that whose record it asks L2 for
 constexpr int HALO_LIST_THREADS = 256;
 constexpr int HALO_RW = HALO_W + 6;              // region of the lists: the tile and three rings
-static_assert(HALO_H + 2 * HALO_O <= 32 && HALO_H16 + 2 * HALO_O <= 32, "entries: 6 column bits, 5 row bits");
+static_assert(HALO_W + 2 * HALO_O <= 64 && HALO_H + 2 * HALO_O <= 32 && HALO_H16 + 2 * HALO_O <= 32,
+              "entries: 6 column bits, 5 row bits");
 
 // List entry: column (bits 0-5) and row (6-10) from (x0 - 4, y0 - 4),
 // solid-neighbour bits 1 ... 8 of the flags (11-18), border tag.
@@ -205,13 +208,15 @@ __global__ void __launch_bounds__(HALO_LIST_THREADS)
 template <typename T, int R, bool VR>
 struct HaloSmem {
   using C = typename Pop<T>::C;
-  // the window: R + 1 more nodes on each side, with 16-bit storage four more
-  // columns whatever R (copies start on 16 bytes)
+  // The window: the tile and R rings, R + 1 columns more on each side (four
+  // with 16-bit storage, whose copies could not start on 16 bytes otherwise).
+  // A plane's rows are those its direction pulls from, y - c_i.y; the
+  // references, which every direction reads, have a row more on each side.
   static constexpr int H = halo_h<T>, O = kDev<T> ? 4 : R + 1, P = HALO_W + 2 * O;
-  static constexpr int ROWS = H + 2 * (R + 1), CELLS = P * ROWS;
+  static constexpr int ROWS = H + 2 * R, CELLS = P * ROWS;
   static constexpr int pad(int n) { return (n + 127) / 128 * 128; }
   static constexpr int FBYTES = CELLS * 2 * (int)sizeof(T), FSLOT = pad(FBYTES);
-  static constexpr int RBYTES = kDev<T> ? CELLS * (VR ? (int)sizeof(UPair) : 2 * (int)sizeof(C)) : 0;
+  static constexpr int RBYTES = kDev<T> ? (CELLS + 2 * P) * (VR ? (int)sizeof(UPair) : 2 * (int)sizeof(C)) : 0;
   static constexpr int REF = 9 * FSLOT, RHO = REF + pad(RBYTES), ENT = RHO + pad(CELLS * 2 * (int)sizeof(C));
   static constexpr int BYTES = ENT + pad((HALO_W + 2 * R) * (H + 2 * R) * 4 + 16) + 128;
 };
@@ -234,7 +239,7 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
   using C = typename Pop<T>::C;
   using V = typename CPair<C>::V;
   using S = HaloSmem<T, R, VR>;
-  constexpr int NT = HALO_THREADS;
+  constexpr int NT = halo_threads<R>;
   constexpr uint32_t FB = 2 * sizeof(T);
   __shared__ __align__(8) uint64_t bar;
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
@@ -247,13 +252,13 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // the window's first node: column x0 - O + LP (a multiple of 4 nodes with
-    // 16-bit storage, of 2 otherwise: 16-byte aligned), row y0 - (R + 1) + GH
-    const int xw = x0 - S::O + LP, yw = y0 - (R + 1) + GH;
+    // 16-bit storage, of 2 otherwise: 16-byte aligned), row y0 - R - c_i.y + GH
+    const int xw = x0 - S::O + LP, yw = y0 - R + GH;
     const uint32_t ebytes = (uint32_t)((n_a + 3) & ~3) * 4;
     mbar_expect_tx(&bar, 9u * S::FBYTES + S::RBYTES + ebytes + extra_tx);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) tma_load_3d(sm + i * S::FSLOT, mapf, sizeof(T) == 8 ? 2 * xw : xw, yw, i, &bar);
-    if (kDev<T>) tma_load_2d(sm + S::REF, mapref, VR ? 2 * xw : xw, yw, &bar);
+    for (int i = 0; i < 9; ++i) tma_load_3d(sm + i * S::FSLOT, mapf, sizeof(T) == 8 ? 2 * xw : xw, yw - cy_of(i), i, &bar);
+    if (kDev<T>) tma_load_2d(sm + S::REF, mapref, VR ? 2 * xw : xw, yw - 1, &bar);
     bulk_load(sm + S::ENT, entries + h.e0, ebytes, &bar);
   }
   ready();
@@ -266,7 +271,7 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
   // An entry's node in the window held in shared memory, and in cells of
   // the padded grid from the entries' node (0, 0).
   auto place = [](uint32_t e) {
-    return (int)(e >> 6 & 31u) * S::P + (int)(e & 63u) - ((3 - R) * S::P + HALO_O - S::O);
+    return (int)(e >> 6 & 31u) * S::P + (int)(e & 63u) - ((HALO_O - R) * S::P + HALO_O - S::O);
   };
   auto cells = [&](uint32_t e) { return (e >> 6 & 31u) * (uint32_t)g.px + (e & 63u); };
   // Post-streaming populations of the node at window place w.
@@ -274,14 +279,13 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
     const typename Pop<T>::V* win = (const typename Pop<T>::V*)sm;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-      const int up = -(cx_of(i) + cy_of(i) * S::P);  // to x - c_i
-      const auto v = win[i * (S::FSLOT / (int)FB) + w + up];
+      const auto v = win[i * (S::FSLOT / (int)FB) + w - cx_of(i)];  // f*_i(x - c_i)
       C ra = C(0), rb = C(0);
       if constexpr (kDev<T>) {
         // the writer: x - c_i, or the node itself where that is solid (its
         // bounced value, sent along -c_i)
         const bool back = i != 0 && (fl & nb_bit(opp_of(i)));
-        const int m = back ? w : w + up;
+        const int m = w + S::P - (back ? 0 : cx_of(i) + cy_of(i) * S::P);
         if constexpr (VR) {
           const UVal u = u_unpack(((const UPair*)(sm + S::REF))[m]);
           const float ca = cdot(i, u.v[0]), cb = cdot(i, u.v[1]);
@@ -300,14 +304,23 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
   bool ok = mbar_wait(&bar, 0);
   if (!ok) ok = mbar_wait(&bar, 0);  // the copies in flight, once more
 
-  // phase A
+  // phase A; the populations of a thread's first node, which is one of the
+  // tile's own or a ring node, stay in registers for phase B (4096^2 porous
+  // FP16 387 -> 375 us per step, FP32 402 -> 400)
+  V fp[9];
   if (ok) {
-    for (int t = tid; t < n_a; t += NT) {
-      const uint32_t e = ent[t];
+    if (tid < n_a) {
+      const uint32_t e = ent[tid];
       const int w = place(e);
-      V fp[9];
       gather_node(w, (e >> HE_NB_SHIFT) & NB_ANY, fp);
       rho[w] = density_pair(fp);
+    }
+    for (int t = tid + NT; t < n_a; t += NT) {
+      const uint32_t e = ent[t];
+      const int w = place(e);
+      V fr[9];
+      gather_node(w, (e >> HE_NB_SHIFT) & NB_ANY, fr);
+      rho[w] = density_pair(fr);
     }
     if (R == 1)
       for (int t = tid; t < n_if; t += NT) {
@@ -355,8 +368,8 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
     if (!valid) continue;
     const int w = place(e);
     const uint32_t kp = (uint32_t)korg + cells(e);  // padded index
-    V fp[9], q[9];
-    gather_node(w, fl, fp);
+    V q[9];
+    if (b > 0) gather_node(w, fl, fp);
     q[0].x = q[0].y = C(0);
 #pragma unroll
     for (int i = 1; i < 9; ++i) q[i] = rho[w + cx_of(i) + cy_of(i) * S::P];
@@ -425,13 +438,14 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
 // it). FP64 is bound by its arithmetic, not by the one CTA per SM that its
 // windows allow.
 template <typename T, int R, bool VR>
-__global__ void __launch_bounds__(HALO_THREADS, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
+__global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
     k_halo(const __grid_constant__ CUtensorMap mapf, const __grid_constant__ CUtensorMap mapref,
            const __grid_constant__ HaloArgs<T> a, const HaloTile* __restrict__ work, uint32_t extra_tx) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   HaloTile h;
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
+  pdl_wait();  // the step before; what is read above, a geometry's lists, it does not write
   if (*(volatile int*)a.stop) return;
   if (threadIdx.x == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(work + blockIdx.x + HALO_AHEAD));
@@ -443,7 +457,7 @@ __global__ void __launch_bounds__(HALO_THREADS, sizeof(T) == 8 ? 1 : R == 1 ? 4 
 // 1000, eight steps, the diagnostics and the moments: 481 -> 410 us; 512
 // members read one by one: 16.5 -> 7 ms).
 template <typename T, int R, bool VR, typename O>
-__global__ void __launch_bounds__(HALO_THREADS, R == 1 ? 4 : 3)
+__global__ void __launch_bounds__(halo_threads<R>, R == 1 ? 4 : 3)
     k_halo_moments(const __grid_constant__ CUtensorMap mapf, const __grid_constant__ CUtensorMap mapref,
                    const __grid_constant__ HaloArgs<T> a, const HaloTile* __restrict__ work, uint32_t extra_tx,
                    const __grid_constant__ EvalOut<O> out) {

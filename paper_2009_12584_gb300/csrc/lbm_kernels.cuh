@@ -199,10 +199,8 @@ template <typename T>
 __device__ __forceinline__ void density_node(const T* __restrict__ f, typename Pop<T>::C* __restrict__ P,
                                              const typename Pop<T>::C* __restrict__ Pref,
                                              const UPair* __restrict__ Uref,
-                                             const uint16_t* __restrict__ flags, const int* __restrict__ list, int t,
-                                             const Geo& g) {
+                                             const uint16_t* __restrict__ flags, unsigned e, const Geo& g) {
   using C = typename Pop<T>::C;
-  const unsigned e = (unsigned)__ldg(list + t);
   const int k = (int)(e & ~LIST_TAGS);
   C ref[2][9];
   if constexpr (kDev<T>) {
@@ -235,7 +233,9 @@ __global__ void __launch_bounds__(256, VR ? 1 : 8) k_density_list(const T* __res
                                                       const int* __restrict__ list, int nfluid, Geo g,
                                                       PhysK<typename Pop<T>::C> ph) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < nfluid) density_node<T>(f, P, Pref, VR ? Uref : nullptr, flags, list, t, g);
+  const unsigned e = t < nfluid ? (unsigned)__ldg(list + t) : 0u;
+  pdl_wait();
+  if (t < nfluid) density_node<T>(f, P, Pref, VR ? Uref : nullptr, flags, e, g);
 }
 
 // The update of collide_node for the FP32 compute type, with the two
@@ -333,19 +333,16 @@ inline int collide_threads(int n, int num_sms) {
 // periodic borders) loads no flags and has no adhesion and no bounce-back;
 // a warp with wall nodes but none near a periodic border stores bounced
 // slots at k - c_i; any other warp takes the general path with periodic
-// images. All lanes of the warp must call this (t >= nfluid marks an idle
-// lane).
+// images. All lanes of the warp must call this (an idle one with !valid and
+// entry 0).
 template <typename T>
 __device__ __forceinline__ void collide_node(const T* __restrict__ f, T* __restrict__ fo,
                                              const typename Pop<T>::C* __restrict__ P,
                                              const typename Pop<T>::C* __restrict__ Pref,
                                              const UPair* __restrict__ Uref, UPair* __restrict__ Uo,
-                                             const uint16_t* __restrict__ flags, const int* __restrict__ list,
-                                             int t, int nfluid, const Geo& g,
+                                             const uint16_t* __restrict__ flags, unsigned e, bool valid, const Geo& g,
                                              const PhysK<typename Pop<T>::C>& ph) {
   using C = typename Pop<T>::C;
-  const bool valid = t < nfluid;
-  const unsigned e = valid ? (unsigned)__ldg(list + t) : 0u;
   const bool warp_edge = __any_sync(0xffffffffu, (e & EDGE_TAG) != 0u);
   const bool warp_border = __any_sync(0xffffffffu, (e & BORDER_TAG) != 0u);
   if (!valid) return;
@@ -390,8 +387,10 @@ __global__ void __launch_bounds__(COLLIDE_THREADS, sizeof(T) == 8 ? 4 : 8) k_col
                                                          const int* __restrict__ list, int nfluid, Geo g,
                                                          PhysK<typename Pop<T>::C> ph) {
   prefetch_list_ahead(list, nfluid);
-  collide_node<T>(f, fo, P, Pref, VR ? Uref : nullptr, VR ? Uo : nullptr, flags, list,
-                  blockIdx.x * blockDim.x + threadIdx.x, nfluid, g, ph);
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned e = t < nfluid ? (unsigned)__ldg(list + t) : 0u;
+  pdl_wait();
+  collide_node<T>(f, fo, P, Pref, VR ? Uref : nullptr, VR ? Uo : nullptr, flags, e, t < nfluid, g, ph);
 }
 
 // ---- K2: virtual solid density of Eq. 8 over the interface-solid list -----
@@ -469,11 +468,8 @@ __device__ __forceinline__ void virtual_density(const C* __restrict__ P, uint32_
 }
 
 template <typename C>
-__device__ __forceinline__ void virtual_density_node(C* __restrict__ P, const uint32_t* __restrict__ mask,
-                                                     const int* __restrict__ list, int t, const Geo& g,
+__device__ __forceinline__ void virtual_density_node(C* __restrict__ P, uint32_t msk, int k, const Geo& g,
                                                      const PhysK<C>& ph) {
-  const int k = list[t];
-  const uint32_t msk = mask[t];
   C v0, v1;
   if (ph.avg9)
     virtual_density<C, true>(P, msk, g, k, ph, v0, v1);
@@ -503,7 +499,10 @@ __global__ void __launch_bounds__(128) k_virtual_density(C* __restrict__ P, cons
                                                          const int* __restrict__ list, int n, Geo g,
                                                          PhysK<C> ph) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) virtual_density_node<C>(P, mask, list, t, g, ph);
+  const int k = t < n ? __ldg(list + t) : 0;
+  const uint32_t m = t < n ? __ldg(mask + t) : 0u;
+  pdl_wait();
+  if (t < n) virtual_density_node<C>(P, m, k, g, ph);
 }
 
 
