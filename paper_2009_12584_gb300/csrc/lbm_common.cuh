@@ -311,6 +311,7 @@ struct PhysK {
   C kF[2];   // 1 - 1 / (2 tau)
   C k3[2];   // kF / 3
   C h[2];    // (1 - omega) / 2
+  C G36;     // -G_AB / 36
   C G_AB, G_s[2], chi[2], rho_s[2];
   int bc, pairing, avg9, uniform;
 };
@@ -328,6 +329,7 @@ inline PhysK<C> kphys(const Phys& p) {
     k.rho_s[s] = C(p.rho_s[s]);
   }
   k.G_AB = C(p.G_AB);
+  k.G36 = C(p.G_AB / -36.0);
   k.bc = p.bc;
   k.pairing = p.pairing;
   k.avg9 = p.avg9;
@@ -381,16 +383,14 @@ __device__ __forceinline__ void weighted_sum36(const C q[9], C& sx, C& sy) {
 template <typename C>
 __device__ __forceinline__ void interaction_force(const PhysK<C>& ph, uint16_t fl, bool walls, const C rho[2],
                                                   const C nbP[2][9], C F[2][2]) {
-  C ax[2], ay[2], r36[2];
-#pragma unroll
-  for (int s = 0; s < 2; ++s) r36[s] = rho[s] * C(-1.0 / 36.0);
+  C ax[2], ay[2];
   if (ph.bc != BC_VAVG || ph.uniform || !walls) {
 #pragma unroll
     for (int s = 0; s < 2; ++s) weighted_sum36(nbP[s], ax[s], ay[s]);
     if (ph.bc == BC_VAVG || !walls) {
 #pragma unroll
       for (int s = 0; s < 2; ++s) {
-        const C rg = r36[s] * ph.G_AB;
+        const C rg = rho[s] * ph.G36;
         F[s][0] = rg * ax[1 - s];
         F[s][1] = rg * ay[1 - s];
       }
@@ -404,7 +404,7 @@ __device__ __forceinline__ void interaction_force(const PhysK<C>& ph, uint16_t f
       const C rho_c = ph.pairing != 0 ? rho[s] : rho[1 - s];
       const C rs_c = ph.pairing != 0 ? ph.rho_s[s] : ph.rho_s[1 - s];
       const C gs = ph.bc == BC_MC ? ph.G_s[s] : ph.G_s[s] * (ph.bc == BC_LLKC ? rho_c : rs_c);
-      const C rg = r36[s] * ph.G_AB, rs = r36[s] * gs;
+      const C rg = rho[s] * ph.G36, rs = rho[s] * (C(-1.0 / 36.0) * gs);
       F[s][0] = fma(rg, ax[1 - s], rs * vx);
       F[s][1] = fma(rg, ay[1 - s], rs * vy);
     }
@@ -429,7 +429,7 @@ __device__ __forceinline__ void interaction_force(const PhysK<C>& ph, uint16_t f
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     const C bx = self ? sx[s] : sx[1 - s], by = self ? sy[s] : sy[1 - s];
-    const C rg = r36[s] * ph.G_AB, rs = r36[s] * ph.G_s[s];
+    const C rg = rho[s] * ph.G36, rs = rho[s] * (C(-1.0 / 36.0) * ph.G_s[s]);
     F[s][0] = fma(rg, ax[1 - s], rs * bx);
     F[s][1] = fma(rg, ay[1 - s], rs * by);
   }
@@ -450,20 +450,9 @@ __device__ __forceinline__ C density(const C f[9]) {
   return ((f[0] + (f[1] + f[3])) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8]));
 }
 
-// rho / 9 with one rounding: the product with the two-term split of 1/9.
-// Multiplying by the rounded 1/9 alone makes every weight w_i too large by
-// the same 7.5e-9 (FP32), so sum_i f^eq_i = rho (1 + 7.5e-9) and each
-// collision would add that much mass at every node.
-template <typename C>
-__device__ __forceinline__ C rho_over_9(C rho);
-template <>
-__device__ __forceinline__ float rho_over_9<float>(float rho) {
-  constexpr float HI = (float)(1.0 / 9.0);               // fl(1/9)
-  constexpr float LO = (float)(1.0 / 9.0 - (double)HI);  // 1/9 - fl(1/9)
-  return fmaf(rho, HI, rho * LO);
-}
-template <>
-__device__ __forceinline__ double rho_over_9<double>(double rho) {
+// rho / 9 with one rounding: the product with the two-term split of 1/9. The
+// rounded 1/9 alone makes every weight w_i too large by the same 2^-54.
+__device__ __forceinline__ double rho_over_9(double rho) {
   constexpr double HI = 1.0 / 9.0;
   constexpr double LO = HI * 0x1p-54;  // 9 HI = 1 - 2^-54
   return fma(rho, HI, rho * LO);
@@ -481,10 +470,10 @@ __device__ __forceinline__ double rho_over_9<double>(double rho) {
 // r = w_i rho, e = 4.5 (c.u)^2 - 1.5 u^2, g = 3 w_i (1 - 1/(2 tau)) c.F,
 // E = 3 c.u g - 3 w_i (1 - 1/(2 tau)) u.F; the rest population takes minus
 // what the pairs gained (sum_i Delta_i = 0 by Eqs. 2 and 4), so that each
-// component's mass changes only by rounding. About 180 FP64 instructions
-// per node where one direction at a time took 366; with the two-pass
-// schedule, 800 x 600 went from 207 to 178 us per step (128 registers, no
-// spills).
+// component's mass changes only by rounding (rho minus the pairs, and
+// omega / 9 as one constant, are 12 instructions less and twice the rounding
+// error after 300 steps). About 180 FP64 instructions per node where one
+// direction at a time took 366 (128 registers, no spills).
 template <typename C>
 __device__ __forceinline__ void update_node(C f[2][9], const C nbP[2][9], uint16_t fl, bool walls,
                                             const PhysK<C>& ph, C rho[2], C u[2]) {
@@ -506,25 +495,26 @@ __device__ __forceinline__ void update_node(C f[2][9], const C nbP[2][9], uint16
   const C inv = C(1) / (rho[0] + rho[1]);
   const C ux = fma(C(0.5), F[0][0] + F[1][0], jx[0] + jx[1]) * inv;
   const C uy = fma(C(0.5), F[0][1] + F[1][1], jy[0] + jy[1]) * inv;
-  const C c3[4] = {C(3) * ux, C(3) * uy, C(3) * (ux + uy), C(3) * (uy - ux)};
-  const C base = fma(C(-1.5), fma(ux, ux, uy * uy), C(1));
-  C e1[4];  // 1 + e
+  const C cx3 = C(3) * ux, cy3 = C(3) * uy;
+  const C c3[4] = {cx3, cy3, cx3 + cy3, cy3 - cx3};
+  const C base = fma(C(-3), fma(ux, ux, uy * uy), C(2));
+  C e2[4];  // 2 (1 + e)
 #pragma unroll
-  for (int a = 0; a < 4; ++a) e1[a] = fma(C(0.5) * c3[a], c3[a], base);
+  for (int a = 0; a < 4; ++a) e2[a] = fma(c3[a], c3[a], base);
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
-    const C w9 = ph.omega[s] * rho_over_9(rho[s]), w36 = C(0.25) * w9;
+    const C w9 = ph.omega[s] * rho_over_9(rho[s]), w36 = C(0.25) * w9, w18 = C(0.5) * w9, w72 = C(0.125) * w9;
     const C gx = ph.k3[s] * F[s][0], gy = ph.k3[s] * F[s][1];
     const C uF = fma(ux, gx, uy * gy), gx4 = C(0.25) * gx, gy4 = C(0.25) * gy;
     const C g[4] = {gx, gy, gx4 + gy4, gy4 - gx4};
+    const C uF4 = C(0.25) * uF;
     C acc = C(0);
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
       const int i = a < 2 ? a + 1 : a + 3;
-      const C r = a < 2 ? w9 : w36;
-      const C E = fma(c3[a], g[a], a < 2 ? -uF : C(-0.25) * uF);
-      const C P = fma(ph.h[s], S[s][a], fma(r, e1[a], E));
-      const C M = fma(ph.h[s], D[s][a], fma(r, c3[a], g[a]));
+      const C E = fma(c3[a], g[a], a < 2 ? -uF : -uF4);
+      const C P = fma(ph.h[s], S[s][a], fma(a < 2 ? w18 : w72, e2[a], E));
+      const C M = fma(ph.h[s], D[s][a], fma(a < 2 ? w9 : w36, c3[a], g[a]));
       acc += fma(C(2), P, -S[s][a]);
       f[s][i] = P + M;
       f[s][opp_of(i)] = P - M;

@@ -112,7 +112,10 @@ __device__ __forceinline__ void interaction_force2(const PhysK<float>& ph, uint1
   Fy = mul2(nrho, fma2(G, swap2(ay), mul2(Gs, by)));
 }
 
-// rho / 9 with one rounding per component (the two-term split of 1/9).
+// rho / 9 with one rounding per component: the product with the two-term
+// split of 1/9. Multiplying by the rounded 1/9 alone makes every weight w_i
+// too large by the same 7.5e-9, so sum_i f^eq_i = rho (1 + 7.5e-9) and each
+// collision would add that much mass at every node.
 __device__ __forceinline__ float2 rho_over_9_2(float2 rho) {
   return fma2(rho, KC.hi9, mul2(rho, KC.lo9));
 }
