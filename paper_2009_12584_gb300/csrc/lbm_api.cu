@@ -43,9 +43,8 @@ struct Layout {
       smask, stage, dpart, total;
 };
 
-// Whether a context keeps the per-tile lists of the tiled schedule (the
-// schedule AUTO picks for 4- and 8-byte storage; 16-bit storage runs it
-// only when asked for).
+// Whether a context keeps the per-tile lists of the tiled schedule (AUTO
+// has room for them with 4- and 8-byte storage: batches may run it).
 bool uses_tiles(const lbm_params* p) {
   const bool wide = p->storage == LBM_STORE_FP32 || p->storage == LBM_STORE_FP64;
   return p->kernel == LBM_KERNEL_TILED || p->kernel == LBM_KERNEL_TMA || (p->kernel == LBM_KERNEL_AUTO && wide);
@@ -597,7 +596,8 @@ lbm_status do_step(lbm_ctx* c, int nsteps) {
   // AUTO with FP64 storage: bound by the FP64 pipe, so the schedule that
   // sums and updates every node once. Before the update's operations were
   // halved too, 100 x 50 took 20.5 us per step against 61 for the single
-  // passes, 800 x 600 207 against 298 us, 1400 x 1000 553 against 701 us.
+  // passes, 800 x 600 207 against 298 us, 1400 x 1000 553 against 701 us
+  // (with the operations halved 15.5 us and, at 800 x 600, 132 us).
   const bool halo = k == LBM_KERNEL_HALO || (k == LBM_KERNEL_AUTO && sizeof(T) != 8);
   if (halo && c->halo_ready) return step_halo<T>(c, nsteps);
   if constexpr (sizeof(T) >= 4) {  // the marching kernel stores 4- and 8-byte populations only
@@ -612,7 +612,7 @@ lbm_status do_step(lbm_ctx* c, int nsteps) {
 
 // Moments by the halo schedule's kernel (contexts with its lists).
 template <typename T, int R, bool VR, typename O>
-lbm_status launch_halo_moments(lbm_ctx* c, const EvalOut<O>& out) {
+lbm_status launch_halo_moments(lbm_ctx* c, const EvalOut<O>& out, bool solid) {
   using S = HaloSmem<T, R, VR>;
   auto kern = k_halo_moments<T, R, VR, O>;
   // (per call: an evaluation is one of several kernels)
@@ -621,23 +621,26 @@ lbm_status launch_halo_moments(lbm_ctx* c, const EvalOut<O>& out) {
   if (s) return s;
   const CUtensorMap* mf = &c->hmap_f[R == 3][c->cur];
   const CUtensorMap* mr = kDev<T> ? &c->hmap_ref[R == 3][c->Ubuf[0] ? c->cur : c->pcur] : mf;
-  k_zero_solid<O><<<node_grid(c->g, 128), 128, 0, c->stream>>>(c->flags, c->g, out);
-  if ((s = after_launch(c, "k_zero_solid"))) return s;
-  kern<<<c->halo.n_work, halo_threads<R>, S::BYTES, c->stream>>>(*mf, *mr, halo_args<T>(c, c->cur, c->pcur), c->halo.work,
-                                                              c->tma_extra_tx, out);
+  launch_pdl(kern, c->halo.n_work, halo_threads<R>, S::BYTES, c->stream, *mf, *mr, halo_args<T>(c, c->cur, c->pcur),
+             c->halo.work, c->tma_extra_tx, out);
   c->halo_used = true;
-  return after_launch(c, "k_halo_moments");
+  if ((s = after_launch(c, "k_halo_moments")) || !solid) return s;
+  const dim3 grid((c->g.nx + 127) / 128, (c->g.ny + ZERO_ROWS - 1) / ZERO_ROWS);
+  launch_pdl(k_zero_solid<O>, grid, 128, 0, c->stream, c->flags, c->g, out);
+  return after_launch(c, "k_zero_solid");
 }
 
+// solid: whether the zeros at solid nodes are wanted.
 template <typename T, int MODE, typename O>
-lbm_status do_eval(lbm_ctx* c, const EvalOut<O>& out) {
+lbm_status do_eval(lbm_ctx* c, const EvalOut<O>& out, bool solid = true) {
   using C = typename Pop<T>::C;
   if constexpr (MODE == 1 && sizeof(T) <= 4) {
     if (c->halo_ready) {
       const bool three = halo_reach(c->ph) == 3;
       if (kDev<T> && c->prm.velocity_refs)
-        return three ? launch_halo_moments<T, 3, kDev<T>>(c, out) : launch_halo_moments<T, 1, kDev<T>>(c, out);
-      return three ? launch_halo_moments<T, 3, false>(c, out) : launch_halo_moments<T, 1, false>(c, out);
+        return three ? launch_halo_moments<T, 3, kDev<T>>(c, out, solid)
+                     : launch_halo_moments<T, 1, kDev<T>>(c, out, solid);
+      return three ? launch_halo_moments<T, 3, false>(c, out, solid) : launch_halo_moments<T, 1, false>(c, out, solid);
     }
   }
   const T* fin = (const T*)c->f[c->cur];
@@ -1069,13 +1072,14 @@ lbm_status lbm_diagnostics(lbm_ctx* c, const lbm_diag_params* p, lbm_diag* h_out
   a.bridge_y0 = p->bridge_y0;
   lbm_status s;
   const EvalOut<double> ev = fields(c->stage, (int64_t)c->g.nx * c->g.ny);
-  LBM_DISPATCH(c, s = (do_eval<T, 1>(c, ev)); break);
+  LBM_DISPATCH(c, s = (do_eval<T, 1>(c, ev, false)); break);
   if (s) return s;
   double* out_d = c->dpart + (size_t)DIAG_BLOCKS * DIAG_NRED;
-  const int nb = diag_blocks(c->g);
-  k_diag_partial<<<nb, DIAG_THREADS, 0, c->stream>>>(c->stage, c->flags, c->g, a, c->dpart);
+  int threads;
+  const int nb = diag_blocks(c->g, c->num_sms, &threads);
+  launch_pdl(k_diag_partial, nb, threads, 0, c->stream, c->stage, c->flags, c->g, a, c->dpart);
   if ((s = after_launch(c, "k_diag_partial"))) return s;
-  k_diag_final<<<1, 32 * DIAG_NQ, 0, c->stream>>>(c->dpart, nb, c->stage, c->g, a, out_d);
+  launch_pdl(k_diag_final, 1, 32 * DIAG_NQ, 0, c->stream, c->dpart, nb, c->stage, c->flags, c->g, a, out_d);
   if ((s = after_launch(c, "k_diag_final"))) return s;
   double q[DIAG_NQ];
   s = check_cuda(c, cudaMemcpyAsync(q, out_d, sizeof(q), cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync");

@@ -8,12 +8,15 @@
 
 namespace lbm {
 
-constexpr int DIAG_BLOCKS = 256;
-constexpr int DIAG_THREADS = 256;
-// A node per thread until all blocks are in use.
-inline int diag_blocks(const Geo& g) {
-  const int64_t nb = ((int64_t)g.nx * g.ny + DIAG_THREADS - 1) / DIAG_THREADS;
-  return nb < DIAG_BLOCKS ? (int)nb : DIAG_BLOCKS;
+constexpr int DIAG_BLOCKS = 256;  // at most
+constexpr int DIAG_THREADS = 512; // at most
+// Blocks of 256 threads with a node each while one per SM is enough (a block's
+// reduction costs as much FP64 time as a few nodes per thread), then one of
+// 512 threads on each SM.
+inline int diag_blocks(const Geo& g, int num_sms, int* threads) {
+  const int64_t nb = ((int64_t)g.nx * g.ny + 255) / 256, most = num_sms < DIAG_BLOCKS ? num_sms : DIAG_BLOCKS;
+  *threads = nb <= most ? 256 : DIAG_THREADS;
+  return (int)(nb <= most ? nb : most);
 }
 // reduced quantities: 0 sum w, 1 sum w x, 2 sum w y, 3 sum w u_x,
 // 4 sum w u_y, 5 crossings kept, 6..13 the Kasa sums over kept crossings
@@ -64,9 +67,9 @@ __device__ __forceinline__ void diag_point(const DiagArgs& a, double px, double 
 
 // Per-block partial sums (and max) over a fixed grid-stride assignment of
 // the owned nodes; st = [rho^A | rho^B | u_x | u_y], each nx * ny. Bound by the
-// FP64 pipe (2 lanes per clock and SM): signs and tests go by the bits, a node
-// without weight adds nothing to the weighted sums, and a warp without a
-// crossing reduces no fit sums.
+// FP64 pipe (2 lanes per clock and SM): signs and tests go by the bits, and a
+// node without weight adds nothing to the weighted sums. 4096^2 porous, with
+// the moments: 1.23 ms; 1.56 with 256 blocks and a tree per quantity.
 static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(const double* __restrict__ st,
                                                                       const uint16_t* __restrict__ flags, Geo g,
                                                                       DiagArgs a, double* __restrict__ partial) {
@@ -74,8 +77,10 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(const doub
   double acc[DIAG_NRED];
 #pragma unroll
   for (int q = 0; q < DIAG_NRED; ++q) acc[q] = 0.0;
+  long long umax = 0;  // max |u|^2: non-negative values order like their bits
   const int64_t N = (int64_t)g.nx * g.ny;
-  for (int64_t n = (int64_t)blockIdx.x * DIAG_THREADS + threadIdx.x; n < N; n += (int64_t)gridDim.x * DIAG_THREADS) {
+  pdl_wait();
+  for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N; n += (int64_t)gridDim.x * blockDim.x) {
     const int y = (int)((unsigned)n / (unsigned)g.nx), x = (int)((unsigned)n - (unsigned)y * (unsigned)g.nx);
     const int k = g.idx(x, y);
     if (flags[k] & F_SOLID) continue;
@@ -92,7 +97,7 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(const doub
       acc[3] += w * ux;
       acc[4] += w * uy;
     }
-    acc[14] = fmax(acc[14], ux * ux + uy * uy);
+    umax = max(umax, __double_as_longlong(ux * ux + uy * uy));
     const double d = rA - a.level;
     if (x + 1 < g.nx && !(flags[k + 1] & F_SOLID)) {  // edge to (x + 1, y)
       const double e = st[n + 1] - a.level;
@@ -104,26 +109,27 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(const doub
     }
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const bool fit = __any_sync(0xffffffffu, __double_as_longlong(acc[5]) != 0);
-  const bool bad = __any_sync(0xffffffffu, __double_as_longlong(acc[15]) != 0);
+  for (int o = 16; o > 0; o >>= 1) umax = max(umax, __shfl_xor_sync(0xffffffffu, umax, o));
+  // The sums by halving: at each step a lane hands over one half of its
+  // quantities and keeps the sums of the other; 16 FP64 additions in all,
+  // where a tree per quantity takes 5 each.
 #pragma unroll
-  for (int q = 0; q < DIAG_NRED; ++q) {
-    double v = acc[q];
-    if ((q >= 5 && q <= 13 && !fit) || (q == 15 && !bad)) {  // zero in every lane
-      if (lane == 0) red[wid][q] = 0.0;
-      continue;
+  for (int w = 8; w >= 1; w >>= 1) {
+    const bool hi = lane & (2 * w);
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const double keep = hi ? acc[i + w] : acc[i], give = hi ? acc[i] : acc[i + w];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * w);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      const double t = __shfl_down_sync(0xffffffffu, v, o);
-      v = q == 14 ? fmax(v, t) : v + t;
-    }
-    if (lane == 0) red[wid][q] = v;
   }
+  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+  const int mine = lane >> 1;  // the quantity this lane holds now
+  if ((lane & 1) == 0) red[wid][mine] = mine == 14 ? __longlong_as_double(umax) : acc[0];
   __syncthreads();
   if (threadIdx.x < DIAG_NRED) {
     const int q = threadIdx.x;
     double v = red[0][q];
-    for (int w = 1; w < DIAG_THREADS / 32; ++w) v = q == 14 ? fmax(v, red[w][q]) : v + red[w][q];
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) v = q == 14 ? fmax(v, red[w][q]) : v + red[w][q];
     partial[(size_t)blockIdx.x * DIAG_NRED + q] = v;
   }
 }
@@ -132,9 +138,11 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(const doub
 // then a tree), and the bridge radius by a scan of one column, 32 rows at a
 // time (one thread's dependent loads and FP64 additions took 27 us).
 static __global__ void __launch_bounds__(32 * DIAG_NQ) k_diag_final(const double* __restrict__ partial, int nblocks,
-                                                                    const double* __restrict__ st, Geo g, DiagArgs a,
-                                                                    double* __restrict__ out) {
+                                                                    const double* __restrict__ st,
+                                                                    const uint16_t* __restrict__ flags, Geo g,
+                                                                    DiagArgs a, double* __restrict__ out) {
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait();
   if (q < DIAG_NRED) {
     double v = 0.0;  // also the identity of the maximum of |u|^2
     for (int b = lane; b < nblocks; b += 32) {
@@ -150,11 +158,14 @@ static __global__ void __launch_bounds__(32 * DIAG_NQ) k_diag_final(const double
   }
   double br = 0.0;
   if (a.bridge_x >= 0) {
-    const double* col = st + a.bridge_x;  // rho^A, stride nx
+    // rho^A on the column, 0 at solid nodes
+    auto col = [&](int y) {
+      return (flags[g.idx(a.bridge_x, y)] & F_SOLID) ? 0.0 : st[(int64_t)y * g.nx + a.bridge_x];
+    };
     // first row from bridge_y0 on below the level (or ny)
     int y1 = g.ny;
     for (int y = a.bridge_y0; y < g.ny; y += 32) {
-      const bool below = y + lane < g.ny && !(col[(int64_t)(y + lane) * g.nx] >= a.level);
+      const bool below = y + lane < g.ny && !(col(y + lane) >= a.level);
       const unsigned m = __ballot_sync(0xffffffffu, below);
       if (m) {
         y1 = y + __ffs(m) - 1;
@@ -165,7 +176,7 @@ static __global__ void __launch_bounds__(32 * DIAG_NQ) k_diag_final(const double
       br = g.ny - (a.bridge_y0 - 0.5);
     } else if (y1 > a.bridge_y0) {
       const int y = y1 - 1;
-      const double c0 = col[(int64_t)y * g.nx], c1 = col[(int64_t)y1 * g.nx];
+      const double c0 = col(y), c1 = col(y1);
       br = y + (c0 - a.level) / (c0 - c1) - (a.bridge_y0 - 0.5);
     }
   }

@@ -465,6 +465,7 @@ __global__ void __launch_bounds__(halo_threads<R>, R == 1 ? 4 : 3)
   HaloTile h;
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
+  pdl_wait();
   if (*(volatile int*)a.stop) return;
   halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, a.ntx, smem_raw, extra_tx, [] {}, out);
 }

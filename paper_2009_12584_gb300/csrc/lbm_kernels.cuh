@@ -518,11 +518,23 @@ struct EvalOut {
   }
 };
 
-// The zeros of an evaluation at solid nodes.
+// The zeros of an evaluation at solid nodes; after the halo moments kernel,
+// whose last tiles it overlaps: they write the other nodes, and have started
+// only when all earlier work was done. A column of eight nodes per thread: with
+// one, 4096^2 took 131,072 blocks and the moments 412 us for 359.
+constexpr int ZERO_ROWS = 8;
 template <typename O>
 __global__ void __launch_bounds__(128) k_zero_solid(const uint16_t* __restrict__ flags, Geo g, EvalOut<O> out) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-  if (x < g.nx && (__ldg(flags + g.idx(x, y)) & F_SOLID)) out.put((int64_t)y * g.nx + x, O(0), O(0), O(0), O(0));
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y0 = blockIdx.y * ZERO_ROWS;
+  if (x < g.nx) {
+    bool solid[ZERO_ROWS];
+#pragma unroll
+    for (int r = 0; r < ZERO_ROWS; ++r) solid[r] = y0 + r < g.ny && (__ldg(flags + g.idx(x, y0 + r)) & F_SOLID);
+#pragma unroll
+    for (int r = 0; r < ZERO_ROWS; ++r)
+      if (solid[r]) out.put((int64_t)(y0 + r) * g.nx + x, O(0), O(0), O(0), O(0));
+  }
+  pdl_wait();
 }
 
 // ---- Evaluation of the current state: moments or forces -----------------
