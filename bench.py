@@ -79,14 +79,24 @@ def source_hash():
 
 
 def effective_schedule(kernel, storage):
-    """The schedule lbm_step runs on the benchmark workload (improved scheme):
-    AUTO takes the tiled one for 4- and 8-byte storage (the halo one only
-    under the one-node-reach schemes) and the two-pass one for 16-bit
-    storage; 16-bit storage runs a FUSED choice as two-pass too (the
-    marching kernel has no 16-bit path)."""
+    """The schedule whose workspace a choice takes and whose L2 fetch
+    granularity it runs with: tiled for AUTO with 4- and 8-byte storage,
+    two-pass for 16-bit storage under every choice but TILED. What lbm_step
+    runs is step_schedule."""
     if storage in ("fp16", "bf16"):
         return "tiled" if kernel == "tiled" else "two_pass"
     return "tiled" if kernel == "auto" else kernel
+
+
+def step_schedule(kernel, storage):
+    """The schedule lbm_step runs on the benchmark workload: AUTO takes the
+    halo one, with FP64 storage the two-pass one; 16-bit storage has the halo,
+    tiled and two-pass ones and runs every other choice as two-pass."""
+    if kernel == "auto":
+        return "two_pass" if storage == "fp64" else "halo"
+    if storage in ("fp16", "bf16"):
+        return kernel if kernel in ("halo", "tiled") else "two_pass"
+    return kernel
 
 
 def l2_fetch_for(kernel, storage, requested):
@@ -532,9 +542,9 @@ def main():
     alg_bytes = bpu * nf
     achieved = alg_bytes / (per_launch_ms / 1e3) / 1e9
     pk, pk_kind = peaks()
-    # the single-pass class is k_tile under AUTO and TILED (4- and 8-byte
-    # storage), k_march under FUSED, k_halo under HALO, k_tile_tma under TMA
-    sched = effective_schedule(args.kernel, args.storage)
+    # the single-pass class is k_halo under AUTO and HALO, k_tile under TILED,
+    # k_march under FUSED, k_tile_tma under TMA
+    sched = step_schedule(args.kernel, args.storage)
     tkey = dom if dom != "fused" else {"tiled": "tile", "fused": "march"}.get(sched, sched)
     traffic = measured_traffic(tkey, args.storage, l2_fetch)
     kernel_name = {"tile": "k_tile", "march": "k_march", "halo": "k_halo", "tma": "k_tile_tma",
@@ -603,7 +613,7 @@ def main():
                            "nx": n, "ny": n, "fluid_nodes": nf, "solid_fraction": round(1 - nf / n / n, 4),
                            "bc": "virtual_avg", "xi": XI, "chi": chi, "tau": 1.0, "G_AB": 3.0,
                            "storage": args.storage, "kernel": args.kernel,
-                           "schedule": effective_schedule(args.kernel, args.storage),
+                           "schedule": step_schedule(args.kernel, args.storage),
                            "l2": "inputs larger than L2 (populations %.1f GB per buffer)"
                                  % (18 * n * n * BYTES_PER_UPDATE[args.storage] / 144 * 4 / 1e9),
                            "all_node_mlups": round(world * n * n * args.steps / (t_ms / 1e3) / 1e6, 1),

@@ -97,7 +97,7 @@ typedef enum {
  *   16-bit storage by a third density plane (8 bytes per padded node), since
  *   a 16-bit step decodes with the densities of the step before.
  * HALO: one kernel per step, and for 4- and 8-byte storage no density plane:
- *   each CTA takes a tile of 32 x 14 nodes (32 x 20 with 16-bit storage), whose
+ *   each CTA takes a tile of 32 x 16 nodes (32 x 20 with 16-bit storage), whose
  *   populations the Tensor Memory Accelerator copies into shared memory with
  *   the 2 or 4 nodes around it, computes rho(t) of the tile and of the rings
  *   its force and Eq. 8 reach (3 under the improved scheme, 1 under the
@@ -120,8 +120,8 @@ typedef enum {
  * AUTO picks the schedule measured fastest on GB300: TWO_PASS for FP64 storage
  * (bound by the FP64 pipe: the single passes compute densities around a tile
  * again) and HALO for the others (porous 4096^2, us per step under the
- * improved scheme / LLKC: FP32 406 / 363 against 449 / 427 for TILED and 514 /
- * 488 for TWO_PASS; FP16 376 / 337 against 434 / 412 for TWO_PASS); the
+ * improved scheme / LLKC: FP32 398 / 357 against 449 / 427 for TILED and 514 /
+ * 488 for TWO_PASS; FP16 367 / 315 against 434 / 412 for TWO_PASS); the
  * workspace of 4- and 8-byte storage also keeps room for the tiled lists,
  * which batches use. */
 typedef enum {

@@ -164,8 +164,8 @@ def set_l2_fetch_granularity(nbytes: int) -> int:
     (32, 64 or 128 bytes; lbm_set_l2_fetch_granularity) and return the
     previous value. It applies to every kernel of this process on that
     device; the library never sets it by itself. On porous geometries 128
-    bytes is fastest for the tiled schedule (the default for FP32/FP64) and
-    the batched one, 32 bytes for the two-pass schedule."""
+    bytes is fastest for the tiled schedule and batches of it, 32 bytes for
+    the two-pass schedule."""
     lib = load()
     prev = ctypes.c_int32()
     st = lib.lbm_set_l2_fetch_granularity(int(nbytes), ctypes.byref(prev))
@@ -177,9 +177,9 @@ def set_l2_fetch_granularity(nbytes: int) -> int:
 def make_params(nx, ny, *, tau=(1.0, 1.0), G_AB=3.0, periodic_x=False, periodic_y=False,
                 storage="fp32", kernel="auto", rho_ref=(1.0, 1.0), max_interface=0,
                 velocity_refs=False) -> LbmParams:
-    """lbm_params of the C ABI. kernel: "auto" (tiled for fp32/fp64, two-pass
-    for fp16/bf16), "two_pass", "fused" (marching single pass, fp32/fp64) or
-    "tiled"; every schedule gives the same results bit for bit."""
+    """lbm_params of the C ABI. kernel: "auto" (halo, two-pass for fp64),
+    "two_pass", "fused" (marching single pass, fp32/fp64), "tiled", "halo" or
+    "tma"; every schedule gives the same results bit for bit."""
     p = LbmParams()
     p.nx, p.ny = int(nx), int(ny)
     p.periodic_x, p.periodic_y = int(bool(periodic_x)), int(bool(periodic_y))
@@ -436,7 +436,8 @@ class Batch:
         return int(ch[0]), int(ch[1])
 
     def set_schedule(self, kernel):
-        """"two_pass" (default) or "tiled" (4-/8-byte storage)."""
+        """"two_pass" (default: members with halo lists step by the halo kernel)
+        or "tiled" (4-/8-byte storage)."""
         self._check(self.lib.lbm_batch_set_schedule(self.h, KERNEL[kernel] if isinstance(kernel, str) else int(kernel)),
                     "lbm_batch_set_schedule")
         return self
