@@ -120,7 +120,6 @@ __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ?
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
   pdl_wait();  // the launch before; what is read above it does not write
-  if (*(const volatile int*)stop) return;
   if (threadIdx.x == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(work + blockIdx.x + HALO_AHEAD));
   const HaloArgs<T>* src = args + 2 * h.member + parity;
@@ -133,7 +132,7 @@ __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ?
     if (kDev<T>) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(mr) : "memory");
   }
   const uint32_t* entries = (const uint32_t*)__ldg((const unsigned long long*)&src->entries);
-  halo_tile<T, R, VR>(h, mf, mr, entries, a, __ldg(&src->ntx), smem_raw, 0u,
+  halo_tile<T, R, VR>(h, mf, mr, entries, a, stop, __ldg(&src->ntx), smem_raw, 0u,
                       [&] {
                         if (threadIdx.x < sizeof(a) / 4)
                           ((uint32_t*)&a)[threadIdx.x] = __ldg((const uint32_t*)src + threadIdx.x);

@@ -225,15 +225,19 @@ struct HaloSmem {
 // populations (pairs; x in units of Pop<T>::V, FP64 of 8 bytes), with a box of
 // one tile's window; mapref: of the references. a: the simulation's arguments,
 // and entries its list, which the thread that issues the copies has at hand.
-// stage: shared memory of HaloSmem::BYTES. The error word is set to 1 when
+// smem_raw: shared memory of HaloSmem::BYTES. The error word is set to 1 when
 // the copies were not seen to complete within the bound; extra_tx: see
 // tma_issue. ready(): called once by every thread before the first use of a.
+// stop: a CTA that finds it set does nothing (it would wait like the one that
+// set it). Another CTA of the same launch may be setting it, so one thread reads
+// it, and the CTA's first barrier carries the answer: all of its threads go on
+// or none does.
 // eval: an EvalOut that takes the moments (rho^A, rho^B, u of Eq. 3) of the
 // tile's nodes instead of a step, or NoEval.
 struct NoEval {};
 template <typename T, int R, bool VR, typename Ready, typename Eval = NoEval>
 __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* mapf, const CUtensorMap* mapref,
-                                          const uint32_t* entries, const HaloArgs<T>& a, int ntx,
+                                          const uint32_t* entries, const HaloArgs<T>& a, const int* stop, int ntx,
                                           unsigned char* smem_raw, uint32_t extra_tx, Ready&& ready,
                                           const Eval& eval = Eval{}) {
   using C = typename Pop<T>::C;
@@ -242,13 +246,14 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
   constexpr int NT = halo_threads<R>;
   constexpr uint32_t FB = 2 * sizeof(T);
   __shared__ __align__(8) uint64_t bar;
+  __shared__ int stopped;
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
   V* rho = (V*)(sm + S::RHO);
   const uint32_t* ent = (const uint32_t*)(sm + S::ENT);
   const int tid = threadIdx.x;
   const int n_own = h.n.x, n_a = R == 1 ? h.n.y : h.n.z, n_if = h.n.w, i0 = h.i0;
   const int x0 = (h.tile % ntx) * HALO_W, y0 = (h.tile / ntx) * S::H;
-  if (tid == 0) {
+  if (tid == 0 && (stopped = *(const volatile int*)stop) == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     // the window's first node: column x0 - O + LP (a multiple of 4 nodes with
@@ -262,7 +267,8 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
     bulk_load(sm + S::ENT, entries + h.e0, ebytes, &bar);
   }
   ready();
-  __syncthreads();  // the barrier is initialised
+  __syncthreads();  // the barrier is initialised, or the CTA stops
+  if (stopped) return;
   const Geo& g = a.g;
   const PhysK<C>& ph = a.ph;
   // this thread's interface-solid cell, needed after phase A
@@ -433,9 +439,7 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
   }
 }
 
-// A step of one simulation, a CTA per tile that owns fluid nodes. A CTA that
-// finds the error word set does nothing (it would wait like the one that set
-// it). FP64 is bound by its arithmetic, not by the one CTA per SM that its
+// A step of one simulation, a CTA per tile that owns fluid nodes. FP64 is bound by its arithmetic, not by the one CTA per SM that its
 // windows allow.
 template <typename T, int R, bool VR>
 __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
@@ -446,10 +450,9 @@ __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ?
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
   pdl_wait();  // the step before; what is read above, a geometry's lists, it does not write
-  if (*(volatile int*)a.stop) return;
   if (threadIdx.x == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(work + blockIdx.x + HALO_AHEAD));
-  halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, a.ntx, smem_raw, extra_tx, [] {});
+  halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, a.stop, a.ntx, smem_raw, extra_tx, [] {});
 }
 
 // The moments of the current state at fluid nodes, one launch where the
@@ -466,8 +469,7 @@ __global__ void __launch_bounds__(halo_threads<R>, R == 1 ? 4 : 3)
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
   pdl_wait();
-  if (*(volatile int*)a.stop) return;
-  halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, a.ntx, smem_raw, extra_tx, [] {}, out);
+  halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, a.stop, a.ntx, smem_raw, extra_tx, [] {}, out);
 }
 
 }  // namespace lbm

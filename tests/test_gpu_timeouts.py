@@ -1,0 +1,52 @@
+"""The bounded wait of the halo step's copies, made to run out on the host's
+word (the barriers expect more bytes than the copies deliver, so no wait can
+complete; nothing faults): what each caller hears, and what the CTAs that had
+not started yet do."""
+import time
+
+import pytest
+
+from paper_2009_12584_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+from paper_2009_12584_gb300 import lbm  # noqa: E402
+
+WET = dict(G_s=(3.0, 3.0), chi=(1.2, 0.8))
+
+
+def _sim(nx, ny, storage="fp32", kernel="auto", vref=False):
+    mask = inputs.inclined_wall_mask(nx, ny, 20.0, 9)
+    sim = lbm.Simulation(nx, ny, storage=storage, kernel=kernel, velocity_refs=vref)
+    sim.set_geometry(mask).set_wetting("virtual_avg", **WET)
+    return sim.init_fields(*inputs.sharp_droplet(nx, ny, nx / 2, ny / 2, 9))
+
+
+def _times_out(call):
+    with pytest.raises(lbm.LbmError) as e:
+        call()
+    assert e.value.status == lbm.ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+def test_wait_runs_out_in_a_grid_of_several_waves(storage):
+    """More tiles than the chip holds at once: the CTAs of the later waves find
+    the error word set by the first, while others of their wave may still be
+    setting it, and end as a whole; so do the moments of that state. The
+    waits run out once, not once per wave, and the context steps on."""
+    nx, ny = 1504, 1000
+    sim = _sim(nx, ny, storage).step(1)
+    sim.sync()
+    sim.debug_tma_expect_extra(16)
+    t0 = time.time()
+    sim.step(2).moments()
+    _times_out(sim.sync)
+    assert 0.5 < time.time() - t0 < 10.0
+    sim.debug_tma_expect_extra(0).sync()
+    rA, rB = inputs.sharp_droplet(nx, ny, nx / 2, ny / 2, 9)
+    ref = _sim(nx, ny, storage, "two_pass")
+    assert torch.equal(sim.init_fields(rA, rB).step(3).populations(), ref.step(3).populations())
+    sim.sync()
