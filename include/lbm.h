@@ -104,7 +104,11 @@ typedef enum {
  *   others), evaluates Eq. 8 there and updates its own nodes. Its lists take
  *   the parts of the workspace that the geometry leaves unused (4- and 8-byte
  *   storage: the workspace grows by about 4 bytes per node); where they do
- *   not fit, TWO_PASS runs. The copies' wait is bounded as for TMA.
+ *   not fit, TWO_PASS runs. A copy not seen to complete within about a second
+ *   ends the step, and further halo steps do nothing until the next call that
+ *   synchronises (lbm_sync, lbm_mass, lbm_diagnostics, lbm_set_geometry,
+ *   lbm_run_host, lbm_run_host_f32 or lbm_step_profiled) has returned
+ *   LBM_ERR_TIMEOUT; lbm_moments of such a state are NaN at fluid nodes.
  * TMA: the TILED schedule (same lists, same results bit for bit) with two
  *   persistent CTAs per SM walking a list of the tiles that own fluid
  *   nodes; each tile's inputs, the nine population planes and the density
@@ -113,9 +117,7 @@ typedef enum {
  *   two-stage ring, one tile ahead of the update. FP32 storage (other
  *   storage runs TILED); the workspace grows by 16 bytes per tile. A copy
  *   not seen to complete within about a second stops the kernel and is
- *   reported as LBM_ERR_TIMEOUT by the next lbm_sync, lbm_mass or
- *   lbm_step_profiled (until then further halo steps do nothing). Slower than
- *   TILED on GB300 (the windows also carry
+ *   reported as for HALO. Slower than TILED on GB300 (the windows also carry
  *   the solid slots that the tiled kernel's lists skip).
  * AUTO picks the schedule measured fastest on GB300: TWO_PASS for FP64 storage
  * (bound by the FP64 pipe: the single passes compute densities around a tile
@@ -259,9 +261,8 @@ lbm_status lbm_set_l2_fetch_granularity(int32_t bytes, int32_t* previous);
  * production use): from the next step on, the barrier of every tile's copies expects `bytes`
  * (0 ... 4096) more than the copies deliver, so that its wait runs out
  * after about a second, each CTA stops after waiting (bounded) for the
- * copies it has in flight, and the next lbm_sync, lbm_mass or
- * lbm_step_profiled returns LBM_ERR_TIMEOUT; the populations of that step
- * are then incomplete (re-initialise or restore them). 0, the default,
+ * copies it has in flight, and the next call that synchronises returns
+ * LBM_ERR_TIMEOUT; the populations of that step are then incomplete (re-initialise or restore them). 0, the default,
  * restores normal operation. No effect on other schedules. LBM_ERR_ARG for
  * a null context or a size out of range. */
 lbm_status lbm_debug_tma_expect_extra(lbm_ctx* ctx, int32_t bytes);

@@ -107,7 +107,7 @@ bool layout(const lbm_params* p, const Geo& g, Layout* L) {
   L->mass = off;     off = align_up(off + 16, A);
   L->smask = off;    off = align_up(off + (size_t)N, A);
   L->stage = off;    off = align_up(off + 4 * (size_t)N * 8, A);
-  L->dpart = off;    off = align_up(off + ((size_t)DIAG_BLOCKS * DIAG_NRED + DIAG_NQ) * 8, A);
+  L->dpart = off;    off = align_up(off + ((size_t)DIAG_BLOCKS * DIAG_NRED + DIAG_OUT) * 8, A);
   L->total = off;
   return true;
 }
@@ -172,20 +172,22 @@ lbm_status check_cuda(lbm_ctx* c, cudaError_t e, const char* where) {
 }
 
 // The bounded waits of the TMA and halo schedules set small[4] when a copy was
-// not seen to complete; synchronising calls report it (and clear it).
+// not seen to complete; every call that synchronises reports it and clears it.
+// v: the word, read after the work.
+lbm_status report_timeout(lbm_ctx* c, int v) {
+  c->halo_used = false;
+  if (!v) return LBM_OK;
+  lbm_status s = check_cuda(c, cudaMemsetAsync(c->small + 4, 0, sizeof(int), c->stream), "cudaMemsetAsync");
+  return s ? s : fail(c, LBM_ERR_TIMEOUT, "a TMA copy of a step did not complete within its bounded wait");
+}
+
 lbm_status check_timeout(lbm_ctx* c) {
   if (!c->tma && !c->halo_used) return LBM_OK;
-  c->halo_used = false;
   int v = 0;
   lbm_status s = check_cuda(c, cudaMemcpyAsync(&v, c->small + 4, sizeof(int), cudaMemcpyDeviceToHost, c->stream),
                             "cudaMemcpyAsync");
   if (!s) s = check_cuda(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-  if (s) return s;
-  if (v) {
-    s = check_cuda(c, cudaMemsetAsync(c->small + 4, 0, sizeof(int), c->stream), "cudaMemsetAsync");
-    return s ? s : fail(c, LBM_ERR_TIMEOUT, "a TMA copy of a step did not complete within its bounded wait");
-  }
-  return LBM_OK;
+  return s ? s : report_timeout(c, v);
 }
 
 lbm_status after_launch(lbm_ctx* c, const char* where) {
@@ -838,7 +840,8 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const uint8_t* d_mask) {
   const Geo& g = c->g;
   c->has_fields = false;
   c->has_geometry = false;
-  lbm_status s = check_cuda(c, cudaMemsetAsync(c->small, 0, 64, c->stream), "cudaMemsetAsync");
+  // the counts; not the error word, which the read-back below reports
+  lbm_status s = check_cuda(c, cudaMemsetAsync(c->small, 0, 4 * sizeof(int), c->stream), "cudaMemsetAsync");
   if (s) return s;
   k_flags<<<dim3((g.px + 127) / 128, g.py), 128, 0, c->stream>>>(d_mask, c->flags, g, c->small);
   if ((s = after_launch(c, "k_flags"))) return s;
@@ -869,6 +872,7 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const uint8_t* d_mask) {
   s = check_cuda(c, cudaMemcpyAsync(h, c->small, sizeof(h), cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync");
   if (!s) s = check_cuda(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
   if (s) return s;
+  if ((s = report_timeout(c, h[4]))) return s;
   if (h[0] > 0) return fail(c, LBM_ERR_ARG, "fluid node on a non-periodic border");
   if (h[1] > c->if_capacity) return fail(c, LBM_ERR_SPACE, "interface-solid list exceeds max_interface");
   c->n_iface = h[1];
@@ -1079,11 +1083,13 @@ lbm_status lbm_diagnostics(lbm_ctx* c, const lbm_diag_params* p, lbm_diag* h_out
   const int nb = diag_blocks(c->g, c->num_sms, &threads);
   launch_pdl(k_diag_partial, nb, threads, 0, c->stream, c->stage, c->flags, c->g, a, c->dpart);
   if ((s = after_launch(c, "k_diag_partial"))) return s;
-  launch_pdl(k_diag_final, 1, 32 * DIAG_NQ, 0, c->stream, c->dpart, nb, c->stage, c->flags, c->g, a, out_d);
+  launch_pdl(k_diag_final, 1, 32 * DIAG_NQ, 0, c->stream, c->dpart, nb, c->stage, c->flags, c->g, a, c->small + 4,
+             out_d);
   if ((s = after_launch(c, "k_diag_final"))) return s;
-  double q[DIAG_NQ];
+  double q[DIAG_OUT];
   s = check_cuda(c, cudaMemcpyAsync(q, out_d, sizeof(q), cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync");
   if (!s) s = check_cuda(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+  if (!s) s = report_timeout(c, q[DIAG_NQ] != 0);
   if (s) return s;
   const double nan = NAN;
   lbm_diag& o = *h_out;
@@ -1181,7 +1187,7 @@ lbm_status lbm_run_host(lbm_ctx* c, const lbm_wetting_params* w, const uint8_t* 
       s = check_cuda(c, cudaMemcpyAsync(outs[a], c->stage + a * N, N * 8, cudaMemcpyDeviceToHost, c->stream),
                      "cudaMemcpyAsync");
   if (!s) s = check_cuda(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-  return s;
+  return s ? s : check_timeout(c);
 }
 
 lbm_status lbm_run_host_f32(lbm_ctx* c, const lbm_wetting_params* w, const uint8_t* h_mask, const float* h_rhoA,
@@ -1214,7 +1220,7 @@ lbm_status lbm_run_host_f32(lbm_ctx* c, const lbm_wetting_params* w, const uint8
       s = check_cuda(c, cudaMemcpyAsync(outs[a], out + a * N, N * 4, cudaMemcpyDeviceToHost, c->stream),
                      "cudaMemcpyAsync");
   if (!s) s = check_cuda(c, cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-  return s;
+  return s ? s : check_timeout(c);
 }
 
 lbm_status lbm_destroy(lbm_ctx* c) {

@@ -24,6 +24,7 @@ inline int diag_blocks(const Geo& g, int num_sms, int* threads) {
 // the grid centre), 14 max |u|^2 over finite nodes, 15 fluid nodes whose
 // rho^A, rho^B or u is not finite, 16 bridge radius (final kernel only)
 constexpr int DIAG_NQ = 17;
+constexpr int DIAG_OUT = DIAG_NQ + 1;  // what is read back: these and the error word
 constexpr int DIAG_NRED = 16;  // quantities reduced over nodes (0..15)
 
 struct DiagArgs {
@@ -140,7 +141,8 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(const doub
 static __global__ void __launch_bounds__(32 * DIAG_NQ) k_diag_final(const double* __restrict__ partial, int nblocks,
                                                                     const double* __restrict__ st,
                                                                     const uint16_t* __restrict__ flags, Geo g,
-                                                                    DiagArgs a, double* __restrict__ out) {
+                                                                    DiagArgs a, const volatile int* err,
+                                                                    double* __restrict__ out) {
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_wait();
   if (q < DIAG_NRED) {
@@ -180,7 +182,10 @@ static __global__ void __launch_bounds__(32 * DIAG_NQ) k_diag_final(const double
       br = y + (c0 - a.level) / (c0 - c1) - (a.bridge_y0 - 0.5);
     }
   }
-  if (lane == 0) out[16] = br;
+  if (lane == 0) {
+    out[16] = br;
+    out[DIAG_NQ] = *err;
+  }
 }
 
 }  // namespace lbm

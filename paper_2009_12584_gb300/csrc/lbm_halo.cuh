@@ -233,7 +233,8 @@ struct HaloSmem {
 // it, and the CTA's first barrier carries the answer: all of its threads go on
 // or none does.
 // eval: an EvalOut that takes the moments (rho^A, rho^B, u of Eq. 3) of the
-// tile's nodes instead of a step, or NoEval.
+// tile's nodes instead of a step, or NoEval; NaN where the wait ran out or the
+// CTA stops, so that nothing older is taken for them.
 struct NoEval {};
 template <typename T, int R, bool VR, typename Ready, typename Eval = NoEval>
 __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* mapf, const CUtensorMap* mapref,
@@ -253,6 +254,16 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
   const int tid = threadIdx.x;
   const int n_own = h.n.x, n_a = R == 1 ? h.n.y : h.n.z, n_if = h.n.w, i0 = h.i0;
   const int x0 = (h.tile % ntx) * HALO_W, y0 = (h.tile / ntx) * S::H;
+  auto give_up = [&] {
+    if constexpr (!std::is_same<Eval, NoEval>::value) {
+      const float nan = __int_as_float(0x7fffffff);
+      for (int t = tid; t < n_own; t += NT) {
+        const uint32_t e = __ldg(entries + h.e0 + t);
+        const int x = x0 - HALO_O + (int)(e & 63u), y = y0 - HALO_O + (int)(e >> 6 & 31u);
+        eval.put((int64_t)y * a.g.nx + x, nan, nan, nan, nan);
+      }
+    }
+  };
   if (tid == 0 && (stopped = *(const volatile int*)stop) == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -268,7 +279,10 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
   }
   ready();
   __syncthreads();  // the barrier is initialised, or the CTA stops
-  if (stopped) return;
+  if (stopped) {
+    give_up();
+    return;
+  }
   const Geo& g = a.g;
   const PhysK<C>& ph = a.ph;
   // this thread's interface-solid cell, needed after phase A
@@ -340,6 +354,7 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
       atomicExch(a.err, 1);
       atomicExch(a.stop, 1);
     }
+    give_up();
     return;
   }
 

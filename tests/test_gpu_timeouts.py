@@ -50,3 +50,40 @@ def test_wait_runs_out_in_a_grid_of_several_waves(storage):
     ref = _sim(nx, ny, storage, "two_pass")
     assert torch.equal(sim.init_fields(rA, rB).step(3).populations(), ref.step(3).populations())
     sim.sync()
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+@pytest.mark.parametrize("call", ["diagnostics", "mass", "set_geometry", "run_host", "run_host_f32", "step_profiled"])
+def test_every_synchronising_call_reports_the_timeout(call, storage):
+    """What waits for a step's results says that there are none, once, and the
+    next use of the context is sound again."""
+    nx, ny = 70, 50
+    sim = _sim(nx, ny, storage).step(2)
+    before = sim.diagnostics()
+    mask = sim.mask.cpu().numpy()
+    rA, rB = inputs.sharp_droplet(nx, ny, nx / 2, ny / 2, 9)
+    wet = lbm.make_wetting("virtual_avg", **WET)
+
+    def run_host():
+        import numpy as np
+        t = np.float64 if call == "run_host" else np.float32
+        out = [np.empty((ny, nx), t) for _ in range(4)]
+        getattr(sim, call)(wet, mask, rA.astype(t), rB.astype(t), 2, out)
+        return out
+
+    calls = dict(diagnostics=sim.diagnostics, mass=sim.mass, set_geometry=lambda: sim.set_geometry(mask),
+                 step_profiled=lambda: sim.step_profiled(1), run_host=run_host, run_host_f32=run_host)
+    sim.debug_tma_expect_extra(16)
+    if not call.startswith("run_host"):
+        sim.step(1)
+        moments = sim.moments()
+        _fluid = torch.from_numpy(mask == 0).cuda()
+        for m in (moments[0], moments[1], moments[2][0], moments[2][1]):
+            assert torch.all(torch.isnan(m[_fluid])) and torch.all(m[~_fluid] == 0)
+    _times_out(calls[call])
+    sim.debug_tma_expect_extra(0).sync()
+    sim.set_geometry(mask).init_fields(rA, rB).step(2)
+    assert sim.diagnostics() == before
+    if call.startswith("run_host"):
+        assert torch.equal(torch.from_numpy(run_host()[0]).cuda(), sim.moments()[0].to(
+            torch.float64 if call == "run_host" else torch.float32))
