@@ -107,11 +107,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_collide_batch(c
 // member. args: two per member (buffer parity of the step), copied to shared
 // memory while the copies are under way; maps: four tensor maps per member
 // (populations of buffers 0 and 1, references of buffers 0 and 1), in global
-// memory, hence the fence. cur: two indices per member, into its maps.
+// memory, hence the fence. cur: per member two indices into its maps, and its
+// extra_tx.
 template <typename T, int R, bool VR>
 __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
     k_halo_batch(const HaloArgs<T>* __restrict__ args, const CUtensorMap* __restrict__ maps,
-                 const HaloTile* __restrict__ work, const int2* __restrict__ cur, const int* __restrict__ stop,
+                 const HaloTile* __restrict__ work, const int4* __restrict__ cur, const int* __restrict__ stop,
                  int parity) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ HaloArgs<T> a;
@@ -124,19 +125,31 @@ __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ?
     asm volatile("prefetch.global.L2 [%0];" ::"l"(work + blockIdx.x + HALO_AHEAD));
   const HaloArgs<T>* src = args + 2 * h.member + parity;
   const CUtensorMap *mf = maps, *mr = maps;
+  uint32_t extra_tx = 0;
   if (threadIdx.x == 0) {
-    const int2 b = __ldg(cur + h.member);
+    const int4 b = __ldg(cur + h.member);
+    extra_tx = (uint32_t)b.z;
     mf = maps + 4 * h.member + (b.x ^ parity);
     mr = maps + 4 * h.member + 2 + (b.y ^ parity);
     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(mf) : "memory");
     if (kDev<T>) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(mr) : "memory");
   }
   const uint32_t* entries = (const uint32_t*)__ldg((const unsigned long long*)&src->entries);
-  halo_tile<T, R, VR>(h, mf, mr, entries, a, stop, __ldg(&src->ntx), smem_raw, 0u,
+  halo_tile<T, R, VR>(h, mf, mr, entries, a, stop, __ldg(&src->ntx), smem_raw, extra_tx,
                       [&] {
                         if (threadIdx.x < sizeof(a) / 4)
                           ((uint32_t*)&a)[threadIdx.x] = __ldg((const uint32_t*)src + threadIdx.x);
                       });
+}
+
+// stop = whether some member's error word is set: a step that it missed has not
+// been reported yet.
+template <typename T>
+__global__ void __launch_bounds__(256) k_halo_stop(const HaloArgs<T>* __restrict__ args, int n, int* stop) {
+  int any = 0;
+  for (int s = threadIdx.x; s < n; s += 256) any |= *(const volatile int*)args[2 * s].err;
+  any = __syncthreads_or(any);
+  if (threadIdx.x == 0) *stop = any != 0;
 }
 
 // A member's tile records into the batch's list.
@@ -206,11 +219,11 @@ struct lbm_batch {
   void* d_hargs;        // HaloArgs[2 n], and their host staging
   void* h_hargs;
   CUtensorMap* d_hmaps; // [4 n]
-  int2* d_hcur;         // [n], and host staging
-  int2* h_hcur;
+  int4* d_hcur;         // [n], and host staging
+  int4* h_hcur;
   HaloTile* d_hwork[HALO_CLASSES];
   int n_hwork[HALO_CLASSES];
-  int* d_stop;
+  int* d_stop;          // set by a CTA whose wait ran out: no further halo step of this call
   int bs;               // threads per block of the density and collide kernels
   void* h_desc;         // host staging of the descriptors
   int2* h_tab;          // host staging of the block tables
@@ -276,7 +289,7 @@ BLayout blayout(int n, lbm_ctx* const* ctxs) {
   L.tblk = off;  off = align_up(off + (size_t)nt * sizeof(int2), 256);
   L.hargs = off; off = align_up(off + 2 * (size_t)n * hargs_bytes(ctxs[0]->prm.storage), 256);
   L.hmaps = off; off = align_up(off + 4 * (size_t)n * sizeof(CUtensorMap), 256);
-  L.hcur = off;  off = align_up(off + (size_t)n * sizeof(int2), 256);
+  L.hcur = off;  off = align_up(off + (size_t)n * sizeof(int4), 256);
   for (int k = 0; k < HALO_CLASSES; ++k) L.n_hwork[k] = 0;
   for (int s = 0; s < n; ++s)
     if (batch_halo(ctxs[s])) L.n_hwork[halo_class(ctxs[s])] += ctxs[s]->halo.n_work;
@@ -327,7 +340,7 @@ void fill_halo(lbm_batch* b) {
   for (int s = 0; s < b->n; ++s) {
     const lbm_ctx* c = b->ctx[s];
     for (int p = 0; p < 2; ++p) h[2 * s + p] = halo_args<T>(c, c->cur ^ p, c->pcur ^ p, b->d_stop);
-    b->h_hcur[s] = make_int2(c->cur, c->Ubuf[0] ? c->cur : c->pcur);
+    b->h_hcur[s] = make_int4(c->cur, c->Ubuf[0] ? c->cur : c->pcur, (int)c->tma_extra_tx, 0);
   }
 }
 
@@ -373,7 +386,7 @@ struct HaloLaunch {
   const HaloArgs<T>* hargs;
   const CUtensorMap* maps;
   const HaloTile* work;
-  const int2* cur;
+  const int4* cur;
   const int* stop;
   int parity;
   void* args[6];
@@ -535,19 +548,27 @@ lbm_status batch_step(lbm_batch* b, int nsteps) {
   }
   lbm_status st = bcuda(b, cudaMemcpyAsync(b->d_desc, b->h_desc, (size_t)b->n * sizeof(BatchDesc<C>),
                                            cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
-  const bool halo = !tiled && any_halo(b);
+  const bool halo = !tiled && any_halo(b) && nsteps > 0;
+  int stop = 0;
   if constexpr (sizeof(T) <= 4) {
     if (halo && !st) {
       fill_halo<T>(b);
       st = bcuda(b, cudaMemcpyAsync(b->d_hargs, b->h_hargs, 2 * (size_t)b->n * sizeof(HaloArgs<T>),
                                     cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
-      if (!st) st = bcuda(b, cudaMemcpyAsync(b->d_hcur, b->h_hcur, (size_t)b->n * sizeof(int2),
+      if (!st) st = bcuda(b, cudaMemcpyAsync(b->d_hcur, b->h_hcur, (size_t)b->n * sizeof(int4),
                                              cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
-      if (!st) st = bcuda(b, cudaMemsetAsync(b->d_stop, 0, 4, b->stream), "cudaMemsetAsync");
+      if (!st) {
+        k_halo_stop<T><<<1, 256, 0, b->stream>>>((const HaloArgs<T>*)b->d_hargs, b->n, b->d_stop);
+        st = bcuda(b, cudaGetLastError(), "k_halo_stop");
+      }
+      if (!st) st = bcuda(b, cudaMemcpyAsync(&stop, b->d_stop, sizeof(int), cudaMemcpyDeviceToHost, b->stream),
+                          "cudaMemcpyAsync");
     }
   }
   // the staging buffers are rewritten by the next call: wait for the copies
   if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
+  if (!st && stop)  // not from a state that misses a step; lbm_sync of the members reports and clears it
+    return bfail(b, LBM_ERR_TIMEOUT, "a TMA copy of a member's step did not complete within its bounded wait");
   if (!st && tiled && nsteps > 0) {
     // the tiled step reads rho(t) from Pbuf[pcur]: compute it for every
     // member once (a member whose plane already holds it gets the same bits)
@@ -574,7 +595,7 @@ lbm_status batch_step(lbm_batch* b, int nsteps) {
       c->pcur ^= 1;
       c->P = c->Pbuf[c->pcur];
     }
-    if (halo && b->halo[s] && nsteps > 0) c->halo_used = true;
+    if (halo && b->halo[s]) c->halo_used = true;
     // after tiled steps Pbuf[pcur] holds rho of the current state
     c->p_valid = tiled && (nsteps > 0 || c->p_valid);
   }
@@ -705,10 +726,10 @@ lbm_status lbm_batch_create(int32_t n, lbm_ctx* const* ctxs, void* d_workspace, 
   b->h_tab = (int2*)malloc((size_t)tab_cap * sizeof(int2));
   b->halo = (bool*)malloc((size_t)n);
   b->h_hargs = malloc(2 * (size_t)n * hargs_bytes(b->storage));
-  b->h_hcur = (int2*)malloc((size_t)n * sizeof(int2));
+  b->h_hcur = (int4*)malloc((size_t)n * sizeof(int4));
   b->d_hargs = b->ws + L.hargs;
   b->d_hmaps = (CUtensorMap*)(b->ws + L.hmaps);
-  b->d_hcur = (int2*)(b->ws + L.hcur);
+  b->d_hcur = (int4*)(b->ws + L.hcur);
   b->d_stop = (int*)(b->ws + L.stop);
   for (int k = 0; k < HALO_CLASSES; ++k) {
     b->d_hwork[k] = (HaloTile*)(b->ws + L.hwork[k]);

@@ -229,9 +229,10 @@ struct HaloSmem {
 // the copies were not seen to complete within the bound; extra_tx: see
 // tma_issue. ready(): called once by every thread before the first use of a.
 // stop: a CTA that finds it set does nothing (it would wait like the one that
-// set it). Another CTA of the same launch may be setting it, so one thread reads
-// it, and the CTA's first barrier carries the answer: all of its threads go on
-// or none does.
+// set it) and sets its own simulation's error word, whose step is missing then
+// (in a batch the words are apart). Another CTA of the same launch may be
+// setting stop, so one thread reads it, and the CTA's first barrier carries the
+// answer: all of its threads go on or none does.
 // eval: an EvalOut that takes the moments (rho^A, rho^B, u of Eq. 3) of the
 // tile's nodes instead of a step, or NoEval; NaN where the wait ran out or the
 // CTA stops, so that nothing older is taken for them.
@@ -280,6 +281,7 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
   ready();
   __syncthreads();  // the barrier is initialised, or the CTA stops
   if (stopped) {
+    if (tid == 0) atomicExch(a.err, 1);
     give_up();
     return;
   }

@@ -87,3 +87,40 @@ def test_every_synchronising_call_reports_the_timeout(call, storage):
     if call.startswith("run_host"):
         assert torch.equal(torch.from_numpy(run_host()[0]).cuda(), sim.moments()[0].to(
             torch.float64 if call == "run_host" else torch.float32))
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+@pytest.mark.parametrize("graph", [0, 2])
+def test_batch_tells_every_member_that_missed_a_step(storage, graph):
+    """One member's wait runs out: the halo members, of both launches, miss the
+    steps that follow and all say so, the one of the two passes does not; the
+    batch refuses to step on from there until they have said it."""
+    sizes = [(70, 50, "auto", "virtual_avg"), (96, 61, "auto", "virtual_avg"), (130, 70, "halo", "llkc"),
+             (64, 40, "two_pass", "virtual_avg")]
+
+    def member(nx, ny, kernel, scheme):
+        sim = _sim(nx, ny, storage, kernel)
+        return sim.set_wetting(scheme, **(WET if scheme == "virtual_avg" else dict(G_s=(-0.5, 0.3))))
+
+    sims = [member(*z) for z in sizes]
+    batch = lbm.Batch(sims)
+    if graph:
+        batch.set_graph_steps(graph)
+    batch.step(1)
+    sims[1].debug_tma_expect_extra(16)
+    batch.step(4)
+    sims[1].debug_tma_expect_extra(0)
+    _times_out(lambda: batch.step(1))
+    for sim in sims[:2]:
+        _times_out(sim.sync)
+    _times_out(lambda: batch.step(1))
+    _times_out(sims[2].sync)
+    for sim in sims:
+        sim.sync()
+    for sim, z in zip(sims, sizes):
+        sim.init_fields(*inputs.sharp_droplet(z[0], z[1], z[0] / 2, z[1] / 2, 9))
+    batch.step(5)
+    for sim, z in zip(sims, sizes):
+        sim.sync()
+        assert torch.equal(sim.populations(), member(*z).step(5).populations())
+    batch.close()
