@@ -396,13 +396,13 @@ lbm_status lbm_field_mass_noalloc(const double* d_rhoA, const double* d_rhoB,
  * (the Eq. 8 launch and one tiled single-pass launch over all members'
  * 32 x 14 tiles; 4- and 8-byte storage, members created with
  * LBM_KERNEL_AUTO or LBM_KERNEL_TILED so that they keep tile lists). The batch keeps pointers to the contexts; they
- * must outlive it, keep their geometry and wetting, and may still be
- * queried individually (lbm_moments, lbm_mass, ...) between batch steps.
+ * must outlive it, and may still be queried (lbm_moments, lbm_mass, ...) or
+ * take another geometry or wetting between batch steps: the next one builds
+ * its tables again.
  * When the copies of a member's halo step do not complete (see HALO), every
  * member whose steps are missing after that reports LBM_ERR_TIMEOUT at its next
  * synchronising call, and lbm_batch_step returns it, without a step, until they
- * all have.
- * The batch snapshots which members use the improved scheme at creation. */
+ * all have. */
 typedef struct lbm_batch lbm_batch;
 
 /* Device workspace bytes of a batch over ctxs[0..n). Every member must have

@@ -840,6 +840,7 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const uint8_t* d_mask) {
   const Geo& g = c->g;
   c->has_fields = false;
   c->has_geometry = false;
+  ++c->geometry;
   // the counts; not the error word, which the read-back below reports
   lbm_status s = check_cuda(c, cudaMemsetAsync(c->small, 0, 4 * sizeof(int), c->stream), "cudaMemsetAsync");
   if (s) return s;

@@ -190,14 +190,18 @@ size_t desc_bytes(int storage) {
   return storage == LBM_STORE_FP64 ? sizeof(BatchDesc<double>) : sizeof(BatchDesc<float>);
 }
 
-// block-table entries for lists of the given lengths and block size
-int64_t table_entries(const int* lens, int n, int bs) {
-  int64_t e = 0;
-  for (int s = 0; s < n; ++s) e += (lens[s] + bs - 1) / bs;
-  return e;
-}
-
 }  // namespace
+
+// What the block tables and the halo launches depend on, of one member.
+struct Member {
+  int cls;           // its halo launch, or -1: it steps by the two passes
+  int n_fluid;
+  int n_virtual;     // interface-solid cells that take Eq. 8 (none under the other schemes)
+  int64_t geometry;  // lbm_ctx::geometry
+  bool operator==(const Member& o) const {
+    return cls == o.cls && n_fluid == o.n_fluid && n_virtual == o.n_virtual && geometry == o.geometry;
+  }
+};
 
 struct lbm_batch {
   int n;
@@ -214,14 +218,15 @@ struct lbm_batch {
   int schedule;         // LBM_KERNEL_TWO_PASS or LBM_KERNEL_TILED
   bool tiled_ok;        // 4- or 8-byte storage and every member keeps tile lists
   bool vr;              // 16-bit storage and some member keeps velocity references
+  Member* m;            // per member: what the tables were built for
   // halo steps of the list schedule
-  bool* halo;           // per member: it steps by the halo kernel
   void* d_hargs;        // HaloArgs[2 n], and their host staging
   void* h_hargs;
   CUtensorMap* d_hmaps; // [4 n]
   int4* d_hcur;         // [n], and host staging
   int4* h_hcur;
-  HaloTile* d_hwork[HALO_CLASSES];
+  HaloTile* d_hwork;    // tile records, class by class
+  HaloTile* d_class[HALO_CLASSES];
   int n_hwork[HALO_CLASSES];
   int* d_stop;          // set by a CTA whose wait ran out: no further halo step of this call
   int bs;               // threads per block of the density and collide kernels
@@ -248,10 +253,11 @@ lbm_status bcuda(lbm_batch* b, cudaError_t e, const char* where) {
 }
 
 // Device layout of a batch workspace: descriptors, fluid block table (sized
-// for the smallest block size), interface block table, tile block table.
+// for the smallest block size), interface block table, tile block table. The
+// tables have room for whatever geometry and wetting the members may take.
 struct BLayout {
-  size_t desc, fblk, iblk, tblk, hargs, hmaps, hcur, hwork[HALO_CLASSES], stop, total;
-  int n_hwork[HALO_CLASSES];
+  size_t desc, fblk, iblk, tblk, hargs, hmaps, hcur, hwork, stop, total;
+  int64_t table;  // entries of the longest block table
 };
 size_t hargs_bytes(int storage) {
   return storage == LBM_STORE_FP64 ? sizeof(HaloArgs<double>)
@@ -271,36 +277,33 @@ bool batch_tiled_ok(int n, lbm_ctx* const* ctxs) {
 // keep the two passes (bound by the FP64 pipe).
 bool batch_halo(const lbm_ctx* c) { return c->halo_ready && c->prm.storage != LBM_STORE_FP64; }
 
+Member member_now(const lbm_ctx* c) {
+  return Member{batch_halo(c) ? halo_class(c) : -1, c->n_fluid, c->ph.bc == BC_VAVG ? c->n_iface : 0, c->geometry};
+}
+
 BLayout blayout(int n, lbm_ctx* const* ctxs) {
-  int* lf = (int*)malloc(sizeof(int) * n);
-  int* li = (int*)malloc(sizeof(int) * n);
+  const bool tiled = batch_tiled_ok(n, ctxs);
+  int64_t nf = 0, ni = 0, nt = 0, nw = 0;
   for (int s = 0; s < n; ++s) {
-    lf[s] = ctxs[s]->n_fluid;
-    li[s] = ctxs[s]->ph.bc == BC_VAVG ? ctxs[s]->n_iface : 0;
+    const lbm_ctx* c = ctxs[s];
+    nf += ((int64_t)c->g.nx * c->g.ny + 127) / 128;
+    ni += (c->if_capacity + 127) / 128;
+    nt += tiled ? c->n_tiles : 0;
+    nw += c->prm.storage != LBM_STORE_FP64 ? halo_tile_count(c->g, halo_rows(c->prm.storage == LBM_STORE_FP32 ? 4 : 2)) : 0;
   }
   BLayout L;
   size_t off = 0;
   L.desc = off;  off = align_up(off + (size_t)n * desc_bytes(ctxs[0]->prm.storage), 256);
-  L.fblk = off;  off = align_up(off + (size_t)table_entries(lf, n, 128) * sizeof(int2), 256);
-  L.iblk = off;  off = align_up(off + (size_t)table_entries(li, n, 128) * sizeof(int2), 256);
-  int64_t nt = 0;
-  if (batch_tiled_ok(n, ctxs))
-    for (int s = 0; s < n; ++s) nt += ctxs[s]->n_tiles;
+  L.fblk = off;  off = align_up(off + (size_t)nf * sizeof(int2), 256);
+  L.iblk = off;  off = align_up(off + (size_t)ni * sizeof(int2), 256);
   L.tblk = off;  off = align_up(off + (size_t)nt * sizeof(int2), 256);
   L.hargs = off; off = align_up(off + 2 * (size_t)n * hargs_bytes(ctxs[0]->prm.storage), 256);
   L.hmaps = off; off = align_up(off + 4 * (size_t)n * sizeof(CUtensorMap), 256);
   L.hcur = off;  off = align_up(off + (size_t)n * sizeof(int4), 256);
-  for (int k = 0; k < HALO_CLASSES; ++k) L.n_hwork[k] = 0;
-  for (int s = 0; s < n; ++s)
-    if (batch_halo(ctxs[s])) L.n_hwork[halo_class(ctxs[s])] += ctxs[s]->halo.n_work;
-  for (int k = 0; k < HALO_CLASSES; ++k) {
-    L.hwork[k] = off;
-    off = align_up(off + (size_t)L.n_hwork[k] * sizeof(HaloTile), 256);
-  }
+  L.hwork = off; off = align_up(off + (size_t)nw * sizeof(HaloTile), 256);
   L.stop = off;  off = align_up(off + 4, 256);
   L.total = off;
-  free(lf);
-  free(li);
+  L.table = nf > ni ? (nf > nt ? nf : nt) : (ni > nt ? ni : nt);
   return L;
 }
 
@@ -319,15 +322,13 @@ int build_table(int2* h_tab, int n, int bs, LenFn len) {
 lbm_status upload_tables(lbm_batch* b, int bs) {
   const bool all = b->schedule == LBM_KERNEL_TILED;
   b->bs = bs;
-  b->n_fblk = build_table(b->h_tab, b->n, bs, [&](int s) { return all || !b->halo[s] ? b->ctx[s]->n_fluid : 0; });
+  b->n_fblk = build_table(b->h_tab, b->n, bs, [&](int s) { return all || b->m[s].cls < 0 ? b->m[s].n_fluid : 0; });
   lbm_status st = bcuda(b, cudaMemcpyAsync(b->d_fblk, b->h_tab, (size_t)b->n_fblk * sizeof(int2),
                                            cudaMemcpyHostToDevice, b->stream), "cudaMemcpyAsync");
   if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
   if (st) return st;
   // interface blocks (128 threads), only for simulations with the improved scheme
-  b->n_iblk = build_table(b->h_tab, b->n, 128, [&](int s) {
-    return b->ctx[s]->ph.bc == BC_VAVG && (all || !b->halo[s]) ? b->ctx[s]->n_iface : 0;
-  });
+  b->n_iblk = build_table(b->h_tab, b->n, 128, [&](int s) { return all || b->m[s].cls < 0 ? b->m[s].n_virtual : 0; });
   st = bcuda(b, cudaMemcpyAsync(b->d_iblk, b->h_tab, (size_t)b->n_iblk * sizeof(int2), cudaMemcpyHostToDevice,
                                 b->stream), "cudaMemcpyAsync");
   if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
@@ -391,7 +392,7 @@ struct HaloLaunch {
   int parity;
   void* args[6];
   HaloLaunch(const lbm_batch* b, int k, int p)
-      : hargs((const HaloArgs<T>*)b->d_hargs), maps(b->d_hmaps), work(b->d_hwork[k]), cur(b->d_hcur), stop(b->d_stop),
+      : hargs((const HaloArgs<T>*)b->d_hargs), maps(b->d_hmaps), work(b->d_class[k]), cur(b->d_hcur), stop(b->d_stop),
         parity(p), args{&hargs, &maps, &work, &cur, &stop, &parity} {}
   HaloLaunch(const HaloLaunch&) = delete;
 };
@@ -534,11 +535,81 @@ lbm_status build_graph(lbm_batch* b, int steps) {
   return LBM_OK;
 }
 
+// Tensor maps and tile records of the members that step by the halo kernel.
+// Synchronises.
+lbm_status gather_halo(lbm_batch* b) {
+  CUtensorMap* h = (CUtensorMap*)malloc(4 * (size_t)b->n * sizeof(CUtensorMap));
+  if (!h) return LBM_ERR_SPACE;
+  HaloTile* to[HALO_CLASSES];
+  for (int k = 0; k < HALO_CLASSES; ++k) to[k] = b->d_class[k];
+  lbm_status st = LBM_OK;
+  for (int s = 0; s < b->n && !st; ++s) {
+    const lbm_ctx* c = b->ctx[s];
+    const int k = b->m[s].cls, r = halo_reach(c->ph) == 3;
+    if (k < 0) continue;
+    for (int i = 0; i < 2; ++i) {
+      h[4 * s + i] = c->hmap_f[r][i];
+      h[4 * s + 2 + i] = c->hmap_ref[r][i];
+    }
+    k_halo_gather<<<(c->halo.n_work + 255) / 256, 256, 0, b->stream>>>(c->halo.work, c->halo.n_work, s, to[k]);
+    to[k] += c->halo.n_work;
+    st = bcuda(b, cudaGetLastError(), "k_halo_gather");
+  }
+  if (!st) st = bcuda(b, cudaMemcpyAsync(b->d_hmaps, h, 4 * (size_t)b->n * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
+                                         b->stream), "cudaMemcpyAsync");
+  if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
+  for (int k = 0; k < HALO_CLASSES && !st; ++k) {
+    if (b->n_hwork[k] == 0) continue;
+    switch (b->storage) {
+      case LBM_STORE_FP32:
+        st = bcuda(b, cudaFuncSetAttribute(halo_kernel<float>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           halo_smem<float>(k)), "cudaFuncSetAttribute");
+        break;
+      case LBM_STORE_FP16:
+        st = bcuda(b, cudaFuncSetAttribute(halo_kernel<__half>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           halo_smem<__half>(k)), "cudaFuncSetAttribute");
+        break;
+      default:
+        st = bcuda(b, cudaFuncSetAttribute(halo_kernel<__nv_bfloat16>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           halo_smem<__nv_bfloat16>(k)), "cudaFuncSetAttribute");
+    }
+  }
+  free(h);
+  return st;
+}
+
+// Build the tables and the halo launches for the members as they are now.
+// Synchronises.
+lbm_status take_members(lbm_batch* b) {
+  for (int k = 0; k < HALO_CLASSES; ++k) b->n_hwork[k] = 0;
+  for (int s = 0; s < b->n; ++s) {
+    b->m[s] = member_now(b->ctx[s]);
+    if (b->m[s].cls >= 0) b->n_hwork[b->m[s].cls] += b->ctx[s]->halo.n_work;
+  }
+  HaloTile* at = b->d_hwork;
+  for (int k = 0; k < HALO_CLASSES; ++k) {
+    b->d_class[k] = at;
+    at += b->n_hwork[k];
+  }
+  lbm_status st = upload_tables(b, b->bs);
+  return !st && any_halo(b) ? gather_halo(b) : st;
+}
+
 template <typename T>
 lbm_status batch_step(lbm_batch* b, int nsteps) {
   using C = typename Pop<T>::C;
-  fill_descs<C>(b);
   const bool tiled = b->schedule == LBM_KERNEL_TILED;
+  bool same = true;
+  for (int s = 0; s < b->n; ++s) same = same && b->m[s] == member_now(b->ctx[s]);
+  if (!same && nsteps > 0) {
+    lbm_status ms = take_members(b);
+    if (!ms && b->graph_steps > 0) ms = build_graph<T>(b, b->graph_steps);
+    if (ms) {
+      b->m[0].geometry = -1;  // again at the next step
+      return ms;
+    }
+  }
+  fill_descs<C>(b);
   for (int s = 0; s < b->n && nsteps > 0; ++s) {
     lbm_ctx* c = b->ctx[s];
     lbm_status cs = clear_virtual(c, b->stream);
@@ -595,7 +666,7 @@ lbm_status batch_step(lbm_batch* b, int nsteps) {
       c->pcur ^= 1;
       c->P = c->Pbuf[c->pcur];
     }
-    if (halo && b->halo[s]) c->halo_used = true;
+    if (halo && b->m[s].cls >= 0) c->halo_used = true;
     // after tiled steps Pbuf[pcur] holds rho of the current state
     c->p_valid = tiled && (nsteps > 0 || c->p_valid);
   }
@@ -614,53 +685,10 @@ void free_batch(lbm_batch* b) {
   free(b->ctx);
   free(b->h_desc);
   free(b->h_tab);
-  free(b->halo);
+  free(b->m);
   free(b->h_hargs);
   free(b->h_hcur);
   delete b;
-}
-
-// Tensor maps and tile records of the members that step by the halo kernel.
-// Synchronises.
-lbm_status create_halo(lbm_batch* b) {
-  CUtensorMap* h = (CUtensorMap*)malloc(4 * (size_t)b->n * sizeof(CUtensorMap));
-  if (!h) return LBM_ERR_SPACE;
-  size_t off[HALO_CLASSES] = {};
-  lbm_status st = LBM_OK;
-  for (int s = 0; s < b->n && !st; ++s) {
-    const lbm_ctx* c = b->ctx[s];
-    if (!b->halo[s]) continue;
-    const int k = halo_class(c), r = halo_reach(c->ph) == 3;
-    for (int i = 0; i < 2; ++i) {
-      h[4 * s + i] = c->hmap_f[r][i];
-      h[4 * s + 2 + i] = c->hmap_ref[r][i];
-    }
-    k_halo_gather<<<(c->halo.n_work + 255) / 256, 256, 0, b->stream>>>(c->halo.work, c->halo.n_work, s,
-                                                                       b->d_hwork[k] + off[k]);
-    off[k] += c->halo.n_work;
-    st = bcuda(b, cudaGetLastError(), "k_halo_gather");
-  }
-  if (!st) st = bcuda(b, cudaMemcpyAsync(b->d_hmaps, h, 4 * (size_t)b->n * sizeof(CUtensorMap), cudaMemcpyHostToDevice,
-                                         b->stream), "cudaMemcpyAsync");
-  if (!st) st = bcuda(b, cudaStreamSynchronize(b->stream), "cudaStreamSynchronize");
-  for (int k = 0; k < HALO_CLASSES && !st; ++k) {
-    if (b->n_hwork[k] == 0) continue;
-    switch (b->storage) {
-      case LBM_STORE_FP32:
-        st = bcuda(b, cudaFuncSetAttribute(halo_kernel<float>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           halo_smem<float>(k)), "cudaFuncSetAttribute");
-        break;
-      case LBM_STORE_FP16:
-        st = bcuda(b, cudaFuncSetAttribute(halo_kernel<__half>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           halo_smem<__half>(k)), "cudaFuncSetAttribute");
-        break;
-      default:
-        st = bcuda(b, cudaFuncSetAttribute(halo_kernel<__nv_bfloat16>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           halo_smem<__nv_bfloat16>(k)), "cudaFuncSetAttribute");
-    }
-  }
-  free(h);
-  return st;
 }
 
 lbm_status check_members(int32_t n, lbm_ctx* const* ctxs) {
@@ -711,40 +739,22 @@ lbm_status lbm_batch_create(int32_t n, lbm_ctx* const* ctxs, void* d_workspace, 
   b->schedule = LBM_KERNEL_TWO_PASS;
   b->ctx = (lbm_ctx**)malloc(sizeof(lbm_ctx*) * n);
   b->h_desc = malloc((size_t)n * desc_bytes(b->storage));
-  // host staging large enough for any table (fluid and interface tables at
-  // 128 threads per block, the tile table)
-  int64_t tab_cap = 1;
-  {
-    int64_t ef = 0, ei = 0, et = 0;
-    for (int s = 0; s < n; ++s) {
-      ef += (ctxs[s]->n_fluid + 127) / 128;
-      ei += ctxs[s]->ph.bc == BC_VAVG ? (ctxs[s]->n_iface + 127) / 128 : 0;
-      et += b->tiled_ok ? ctxs[s]->n_tiles : 0;
-    }
-    tab_cap += ef > ei ? (ef > et ? ef : et) : (ei > et ? ei : et);
-  }
-  b->h_tab = (int2*)malloc((size_t)tab_cap * sizeof(int2));
-  b->halo = (bool*)malloc((size_t)n);
+  b->h_tab = (int2*)malloc((size_t)(L.table + 1) * sizeof(int2));
+  b->m = (Member*)malloc((size_t)n * sizeof(Member));
   b->h_hargs = malloc(2 * (size_t)n * hargs_bytes(b->storage));
   b->h_hcur = (int4*)malloc((size_t)n * sizeof(int4));
   b->d_hargs = b->ws + L.hargs;
   b->d_hmaps = (CUtensorMap*)(b->ws + L.hmaps);
   b->d_hcur = (int4*)(b->ws + L.hcur);
   b->d_stop = (int*)(b->ws + L.stop);
-  for (int k = 0; k < HALO_CLASSES; ++k) {
-    b->d_hwork[k] = (HaloTile*)(b->ws + L.hwork[k]);
-    b->n_hwork[k] = L.n_hwork[k];
-  }
-  if (!b->ctx || !b->h_desc || !b->h_tab || !b->halo || !b->h_hargs || !b->h_hcur) {
+  b->d_hwork = (HaloTile*)(b->ws + L.hwork);
+  if (!b->ctx || !b->h_desc || !b->h_tab || !b->m || !b->h_hargs || !b->h_hcur) {
     free_batch(b);
     return LBM_ERR_SPACE;
   }
-  for (int s = 0; s < n; ++s) {
-    b->ctx[s] = ctxs[s];
-    b->halo[s] = batch_halo(ctxs[s]);
-  }
-  st = upload_tables(b, 256);
-  if (!st && any_halo(b)) st = create_halo(b);
+  for (int s = 0; s < n; ++s) b->ctx[s] = ctxs[s];
+  b->bs = 256;
+  st = take_members(b);
   if (!st && b->tiled_ok) {
     // tile blocks: every tile of every member, member by member
     int e = 0;

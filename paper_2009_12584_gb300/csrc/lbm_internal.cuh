@@ -85,6 +85,7 @@ struct lbm_ctx {
   int n_fluid;
   int cur;             // index of the buffer holding the current state
   bool has_geometry, has_fields, has_wetting;
+  int64_t geometry;    // calls of lbm_set_geometry so far
   int64_t launches;
   // lbm_step_profiled: when prof_on, every launch is bracketed by a pair of
   // events from this pool and tagged with its kernel class
