@@ -102,13 +102,15 @@ typedef enum {
  *   the 2 or 4 nodes around it, computes rho(t) of the tile and of the rings
  *   its force and Eq. 8 reach (3 under the improved scheme, 1 under the
  *   others), evaluates Eq. 8 there and updates its own nodes. Its lists take
- *   the parts of the workspace that the geometry leaves unused (4- and 8-byte
- *   storage: the workspace grows by about 4 bytes per node); where they do
- *   not fit, TWO_PASS runs. A copy not seen to complete within about a second
- *   ends the step, and further halo steps do nothing until the next call that
- *   synchronises (lbm_sync, lbm_mass, lbm_diagnostics, lbm_set_geometry,
- *   lbm_run_host, lbm_run_host_f32 or lbm_step_profiled) has returned
- *   LBM_ERR_TIMEOUT; lbm_moments of such a state are NaN at fluid nodes.
+ *   the parts of the workspace that the geometry and the schedule leave unused
+ *   (4- and 8-byte storage: the workspace grows by about 4 bytes per node);
+ *   where they do not fit (16-bit storage with many solid nodes or a small
+ *   max_interface), TWO_PASS runs, under AUTO with FP32 storage TILED. A copy
+ *   not seen to complete within about a second ends the step, and further halo
+ *   steps do nothing until the next call that synchronises (lbm_sync, lbm_mass,
+ *   lbm_diagnostics, lbm_set_geometry, lbm_run_host, lbm_run_host_f32 or
+ *   lbm_step_profiled) has returned LBM_ERR_TIMEOUT; lbm_moments of such a state
+ *   are NaN at fluid nodes.
  * TMA: the TILED schedule (same lists, same results bit for bit) with two
  *   persistent CTAs per SM walking a list of the tiles that own fluid
  *   nodes; each tile's inputs, the nine population planes and the density

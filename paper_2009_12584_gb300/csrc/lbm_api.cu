@@ -57,7 +57,7 @@ bool uses_tma(const lbm_params* p) {
 
 // Whether the workspace has an area of its own for the lists of the halo
 // schedule (4- and 8-byte storage). The lists themselves go wherever they
-// fit (place_halo_lists): the part of the interface arrays that the geometry
+// fit (write_halo_lists): the part of the interface arrays that the geometry
 // leaves unused usually holds them all, with any storage.
 bool uses_halo(const lbm_params* p) {
   const bool wide = p->storage == LBM_STORE_FP32 || p->storage == LBM_STORE_FP64;
@@ -241,20 +241,66 @@ lbm_status build_tile_lists(lbm_ctx* c, cudaStream_t stream) {
   return LBM_OK;
 }
 
+namespace {
+
+// Second density plane while it holds the halo schedule's lists: not to be
+// written.
+bool plane_taken(const lbm_ctx* c) { return c->halo_in_plane && c->halo_ready; }
+// Planes of the current state's encoding references and of its densities.
+void* ref_plane(const lbm_ctx* c) { return plane_taken(c) ? c->Pbuf[0] : c->Pbuf[c->pcur]; }
+void* spare_plane(const lbm_ctx* c) { return plane_taken(c) ? c->Pbuf[0] : c->Pbuf[c->pcur ^ 1]; }
+
+}  // namespace
+
 // Before work that reads the density planes under a scheme without virtual
 // densities: zero the rho~ an earlier scheme of this context left in them.
 lbm_status clear_virtual(lbm_ctx* c, cudaStream_t stream) {
   if (!c->virt_written || c->ph.bc == BC_VAVG) return LBM_OK;
   const int nb = (c->n_iface + 127) / 128;
+  void* P1 = plane_taken(c) ? c->Pbuf[0] : c->Pbuf[1];
   if (c->prm.storage == LBM_STORE_FP64)
-    k_clear_virtual<double><<<nb, 128, 0, stream>>>((double*)c->Pbuf[0], (double*)c->Pbuf[1], (double*)c->Pbuf[2],
+    k_clear_virtual<double><<<nb, 128, 0, stream>>>((double*)c->Pbuf[0], (double*)P1, (double*)c->Pbuf[2],
                                                     c->iface_list, c->n_iface, c->g);
   else
-    k_clear_virtual<float><<<nb, 128, 0, stream>>>((float*)c->Pbuf[0], (float*)c->Pbuf[1], (float*)c->Pbuf[2],
+    k_clear_virtual<float><<<nb, 128, 0, stream>>>((float*)c->Pbuf[0], (float*)P1, (float*)c->Pbuf[2],
                                                    c->iface_list, c->n_iface, c->g);
   lbm_status s = after_launch(c, "k_clear_virtual");
   if (!s) c->virt_written = false;
   return s;
+}
+
+namespace {
+
+// The write pass over the placed lists, whose offsets are at halo_off.
+lbm_status launch_halo_lists(lbm_ctx* c, cudaStream_t stream) {
+  const Geo& g = c->g;
+  const int H = halo_rows((int)elem_size(c->prm.storage));
+  const int64_t nt = halo_tile_count(g, H);
+  const size_t each = align_up((size_t)nt * 4, 256);
+  int* off = (int*)c->halo_off;
+  k_halo_lists<true><<<(unsigned)nt, HALO_LIST_THREADS, 0, stream>>>(
+      c->flags, g, (g.nx + HALO_W - 1) / HALO_W, H, off, off + each / 4, off + each / 2, (HaloTile*)c->halo.work,
+      (uint32_t*)c->halo.entries, (uint2*)c->halo.cells);
+  return after_launch(c, "k_halo_lists(write)");
+}
+
+}  // namespace
+
+// Lists in the second density plane give way to a batch's tiled or two-pass
+// steps, which need it (use false), and are written again for the next halo
+// step: one pass over the flags, their places and offsets stay.
+lbm_status use_halo_lists(lbm_ctx* c, bool use, cudaStream_t stream) {
+  if (!c->halo_in_plane || c->halo_ready == use) return LBM_OK;
+  const size_t bytes = 2 * (size_t)c->g.plane * compute_size(c->prm.storage);
+  lbm_status s = use ? launch_halo_lists(c, stream)
+                     : check_cuda(c, cudaMemsetAsync(c->Pbuf[1], 0, bytes, stream), "cudaMemsetAsync");
+  // k_halo reads its tile record before pdl_wait, which the kernel right before
+  // it must not have written: something else comes between
+  if (!s && use) s = check_cuda(c, cudaMemsetAsync(c->small + 9, 0, sizeof(int), stream), "cudaMemsetAsync");
+  if (s) return s;
+  c->halo_ready = use;
+  c->p_valid = false;
+  return LBM_OK;
 }
 
 namespace {
@@ -274,13 +320,13 @@ lbm_status launch_virtual(lbm_ctx* c, C* P) {
 }
 
 // Densities of the current state (and rho~ at interface-solid nodes) into
-// the spare density plane Pbuf[pcur ^ 1]; Pbuf[pcur] keeps the references
-// the current populations were encoded with.
+// the spare density plane; the other one keeps the references the current
+// populations were encoded with.
 template <typename T>
 lbm_status launch_density_and_virtual(lbm_ctx* c, const T* f) {
   using C = typename Pop<T>::C;
-  C* P = (C*)c->Pbuf[c->pcur ^ 1];
-  const C* Pref = (const C*)c->Pbuf[c->pcur];
+  C* P = (C*)spare_plane(c);
+  const C* Pref = (const C*)ref_plane(c);
   lbm_status s = launch(c, LBM_KC_DENSITY, "k_density", [&] {
     k_density<T><<<node_grid(c->g, 128), 128, 0, c->stream>>>(f, P, Pref, c->Ubuf[c->cur], c->flags, c->g,
                                                                 kphys<C>(c->ph));
@@ -480,9 +526,15 @@ bool wants_halo(const lbm_ctx* c) {
 }
 
 // The halo schedule's lists for the installed geometry go to the unused parts
-// of the workspace: the area halo contexts keep, and behind the interface
-// cells (their arrays have room for every node). Where they do not fit,
-// halo_ready stays false and the two-pass schedule runs.
+// of the workspace: the area halo contexts keep, behind the interface cells
+// (their arrays have room for every node, unless max_interface says otherwise),
+// and, with 4- and 8-byte storage, the second density plane, which this
+// schedule has no use for (use_halo_lists gives it back). 32 bits an entry and
+// 64 a cell, the tiles' rings included, make at most 6.5 bytes per fluid node
+// and 9.6 per interface cell in FP32; the area has 3.6 per node and the plane
+// 8, so with 4- and 8-byte storage they fit until five nodes in six are
+// interface cells. Where they do not fit, halo_ready stays false and do_step
+// falls back.
 //
 // First half, enqueued before lbm_set_geometry reads its counts back: the
 // tiles' sizes, scanned to offsets (totals at small[6 ... 8]), in arrays at
@@ -512,20 +564,23 @@ lbm_status count_halo_lists(lbm_ctx* c) {
 // Second half, with the totals at hand: n_entries, n_cells, n_work.
 lbm_status write_halo_lists(lbm_ctx* c, const int* totals) {
   if (!c->halo_off || c->n_fluid == 0) return LBM_OK;
-  const Geo& g = c->g;
   const int H = halo_rows((int)elem_size(c->prm.storage));
-  const int64_t nt = halo_tile_count(g, H);
-  const size_t each = align_up((size_t)nt * 4, 256);
-  const bool in_area = c->halo_off == c->halo_area[0];
-  char* from[2] = {(char*)align_up((size_t)(c->iface_mask + c->n_iface), 256),
-                   in_area ? c->halo_area[0] + 3 * each : c->halo_area[0]};
-  char* const end[2] = {in_area ? c->iface_end : c->halo_off, c->halo_area[1]};
-  if ((char*)(c->iface_mask + c->n_iface) > end[0]) return LBM_OK;  // the offsets would be overwritten
+  const size_t each = align_up((size_t)halo_tile_count(c->g, H) * 4, 256);
+  const bool in_area = c->halo_off == c->halo_area[0], wide = elem_size(c->prm.storage) >= 4;
+  char* const plane = (char*)c->Pbuf[1];
+  // in the order they are taken: area, interface arrays, density plane
+  char* from[3] = {in_area ? c->halo_area[0] + 3 * each : c->halo_area[0],
+                   (char*)align_up((size_t)(c->iface_mask + c->n_iface), 256), plane};
+  char* const end[3] = {c->halo_area[1], in_area ? c->iface_end : c->halo_off,
+                        wide ? plane + 2 * (size_t)c->g.plane * compute_size(c->prm.storage) : plane};
+  if ((char*)(c->iface_mask + c->n_iface) > end[1]) return LBM_OK;  // the offsets would be overwritten
+  bool in_plane = false;
   auto take = [&](size_t bytes) -> char* {
-    for (int r = 1; r >= 0; --r)
+    for (int r = 0; r < 3; ++r)
       if (from[r] < end[r] && (size_t)(end[r] - from[r]) >= bytes) {
         char* p = from[r];
         from[r] = (char*)align_up((size_t)(p + bytes), 256);
+        in_plane = in_plane || r == 2;
         return p;
       }
     return nullptr;
@@ -534,13 +589,11 @@ lbm_status write_halo_lists(lbm_ctx* c, const int* totals) {
   uint32_t* entries = (uint32_t*)take((size_t)totals[0] * 4);
   uint2* cells = (uint2*)take((size_t)(totals[1] > 0 ? totals[1] : 1) * 8);
   if (!work || !entries || !cells) return LBM_OK;
-  int* off = (int*)c->halo_off;
-  k_halo_lists<true><<<(unsigned)nt, HALO_LIST_THREADS, 0, c->stream>>>(
-      c->flags, g, (g.nx + HALO_W - 1) / HALO_W, H, off, off + each / 4, off + each / 2, work, entries, cells);
-  lbm_status s = after_launch(c, "k_halo_lists(write)");
-  if (s) return s;
   c->halo = HaloLists{work, totals[2], entries, cells};
+  lbm_status s = launch_halo_lists(c, c->stream);
+  if (s) return s;
   c->halo_ready = true;
+  c->halo_in_plane = in_plane;
   return LBM_OK;
 }
 
@@ -601,11 +654,23 @@ lbm_status do_step(lbm_ctx* c, int nsteps) {
   // passes, 800 x 600 207 against 298 us, 1400 x 1000 553 against 701 us
   // (with the operations halved 15.5 us and, at 800 x 600, 132 us).
   const bool halo = k == LBM_KERNEL_HALO || (k == LBM_KERNEL_AUTO && sizeof(T) != 8);
-  if (halo && c->halo_ready) return step_halo<T>(c, nsteps);
+  if (halo) {
+    lbm_status s = use_halo_lists(c, true, c->stream);
+    if (s) return s;
+    if (c->halo_ready) return step_halo<T>(c, nsteps);
+  }
   if constexpr (sizeof(T) >= 4) {  // the marching kernel stores 4- and 8-byte populations only
     if (k == LBM_KERNEL_FUSED && fused_supported<T>(c->g, c->ph)) return step_fused<T>(c, nsteps);
-    if ((k == LBM_KERNEL_TILED || k == LBM_KERNEL_TMA) && c->n_tiles > 0)
+    // FP32 without room for the halo lists: tiles (449 and 427 us at 4096^2
+    // porous, improved scheme and LLKC, against 514 and 488 by two passes)
+    const bool tiles = halo && k == LBM_KERNEL_AUTO && c->n_fluid > 0;
+    if ((k == LBM_KERNEL_TILED || k == LBM_KERNEL_TMA || tiles) && c->n_tiles > 0) {
+      if (!c->tiles_built && nsteps > 0) {
+        lbm_status s = build_tile_lists(c, c->stream);
+        if (s) return s;
+      }
       return step_fused<T>(c, nsteps);
+    }
   } else {
     if (c->Pbuf[2] && c->n_tiles > 0) return step_tiled16<T>(c, nsteps);
   }
@@ -650,7 +715,7 @@ lbm_status do_eval(lbm_ctx* c, const EvalOut<O>& out, bool solid = true) {
   if (!s) s = launch_density_and_virtual<T>(c, fin);
   if (s) return s;
   k_collide<T, MODE, O><<<node_grid(c->g, 128), 128, 0, c->stream>>>(
-      fin, (const C*)c->Pbuf[c->pcur ^ 1], (const C*)c->Pbuf[c->pcur], c->Ubuf[c->cur], c->flags, c->g,
+      fin, (const C*)spare_plane(c), (const C*)ref_plane(c), c->Ubuf[c->cur], c->flags, c->g,
       kphys<C>(c->ph), out);
   return after_launch(c, "k_collide(eval)");
 }
@@ -674,7 +739,7 @@ template <typename T, int SRC>
 lbm_status do_set_state(lbm_ctx* c, const double* fin, const double* rA, const double* rB, const double* ux,
                         const double* uy) {
   using C = typename Pop<T>::C;
-  k_set_state<T, SRC><<<node_grid(c->g, 128), 128, 0, c->stream>>>((T*)c->f[c->cur], (C*)c->P, c->Ubuf[c->cur],
+  k_set_state<T, SRC><<<node_grid(c->g, 128), 128, 0, c->stream>>>((T*)c->f[c->cur], (C*)ref_plane(c), c->Ubuf[c->cur],
                                                                      c->flags, c->g,
                                                                      kphys<C>(c->ph), fin, rA, rB, ux, uy);
   return after_launch(c, "k_set_state");
@@ -867,7 +932,7 @@ lbm_status lbm_set_geometry(lbm_ctx* c, const uint8_t* d_mask) {
   s = check_cuda(c, cudaMemsetAsync(c->Pbase, 0, (c->Pbuf[2] ? 6 : 4) * (size_t)g.plane * compute_size(c->prm.storage),
                                     c->stream), "cudaMemsetAsync");
   if (s) return s;
-  c->halo_ready = false;
+  c->halo_ready = c->halo_in_plane = false;
   if ((s = count_halo_lists(c))) return s;
   int h[9];
   s = check_cuda(c, cudaMemcpyAsync(h, c->small, sizeof(h), cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync");

@@ -275,7 +275,9 @@ bool batch_tiled_ok(int n, lbm_ctx* const* ctxs) {
 
 // Whether a member of the list schedule steps by the halo kernel. FP64 members
 // keep the two passes (bound by the FP64 pipe).
-bool batch_halo(const lbm_ctx* c) { return c->halo_ready && c->prm.storage != LBM_STORE_FP64; }
+bool batch_halo(const lbm_ctx* c) {
+  return (c->halo_ready || c->halo_in_plane) && c->prm.storage != LBM_STORE_FP64;
+}
 
 Member member_now(const lbm_ctx* c) {
   return Member{batch_halo(c) ? halo_class(c) : -1, c->n_fluid, c->ph.bc == BC_VAVG ? c->n_iface : 0, c->geometry};
@@ -613,6 +615,7 @@ lbm_status batch_step(lbm_batch* b, int nsteps) {
   for (int s = 0; s < b->n && nsteps > 0; ++s) {
     lbm_ctx* c = b->ctx[s];
     lbm_status cs = clear_virtual(c, b->stream);
+    if (!cs) cs = use_halo_lists(c, !tiled && b->m[s].cls >= 0, b->stream);
     if (cs) return bfail(b, cs, c->err);
     if (c->ph.bc == BC_VAVG && c->n_iface > 0) c->virt_written = true;
     if (tiled && !c->tiles_built && (cs = build_tile_lists(c, b->stream))) return bfail(b, cs, c->err);

@@ -64,15 +64,16 @@ struct lbm_ctx {
   bool tiles_built;     // the tiled schedule's lists match the current geometry
   bool halo_used;       // a halo step ran since the last look at the error word
   bool halo_ready;      // the halo schedule's lists match the current geometry
+  bool halo_in_plane;   // some of them have their place in Pbuf[1] (see use_halo_lists)
   bool hmaps_ok;        // its tensor maps are encoded
   bool halo_smem_set[2];  // k_halo's dynamic shared memory limit raised (one ring, three rings)
   uint32_t tma_extra_tx;  // test hook of the TMA schedule's bounded wait (lbm_debug_tma_expect_extra); 0
   lbm::HaloLists halo;  // halo schedule: per-tile lists, placed by lbm_set_geometry
   char* halo_off;      // the tiles' offsets while the lists are built (null: no lists)
   char* halo_area[2];  // an area of the workspace for these lists (may be empty)
-  char* iface_end;     // end of the interface arrays, whose unused part also holds them
+  char* iface_end;     // end of the interface arrays, whose unused part also holds them, as Pbuf[1] may
   int* scan_counts;    // per-block interface counts / offsets
-  int* small;          // [0] error count, [1] interface total, [2] fluid total
+  int* small;          // 16 words: [0] error count, [1] interface total, [2] fluid total, [4] error word
   double* partial;     // mass partial sums
   double* mass_out;    // 2 doubles
   uint8_t* stage_mask; // lbm_run_host staging
@@ -101,6 +102,9 @@ struct lbm_ctx {
 lbm_status clear_virtual(lbm_ctx* c, cudaStream_t stream);
 // The tiled schedule's lists of the installed geometry (lbm_api.cu).
 lbm_status build_tile_lists(lbm_ctx* c, cudaStream_t stream);
+// Halo lists that have their place in the second density plane: there (use) or
+// out of the way (lbm_api.cu).
+lbm_status use_halo_lists(lbm_ctx* c, bool use, cudaStream_t stream);
 
 // The halo step's arguments for a context whose current state is in buffer
 // cur, its density plane pcur (the spare one takes a 16-bit step's rho(t)).
