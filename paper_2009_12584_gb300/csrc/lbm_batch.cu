@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB)
   const int2 b = blk[blockIdx.x];
   const BatchDesc<C>& D = d[b.x];
   const int cur = D.cur ^ parity, pcur = D.pcur ^ parity;
-  tile_step<T>(b.y, D.n_tiles, (const T*)D.f[cur], (T*)D.f[cur ^ 1], (const C*)D.Pbuf[pcur],
+  tile_step<T, false>(b.y, D.n_tiles, (const T*)D.f[cur], (T*)D.f[cur ^ 1], (const C*)D.Pbuf[pcur],
                (const C*)D.Pbuf[pcur], nullptr, nullptr, (C*)D.Pbuf[pcur ^ 1], D.flags, D.tile_entries,
                D.tile_off, D.tile_cnt, D.g, D.ntx, D.ph);
 }
@@ -95,10 +95,9 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_collide_batch(c
   const BatchDesc<C>& D = d[b.x];
   const int cur = D.cur ^ parity, pcur = D.pcur ^ parity;
   const int t = b.y + threadIdx.x;
-  const bool valid = t < D.n_fluid;
   collide_node<T>((const T*)D.f[cur], (T*)D.f[cur ^ 1], (const C*)D.Pbuf[pcur ^ 1], (const C*)D.Pbuf[pcur],
-                  VR ? D.Ubuf[cur] : nullptr, VR ? D.Ubuf[cur ^ 1] : nullptr, D.flags,
-                  valid ? (unsigned)__ldg(D.fluid_list + t) : 0u, valid, D.g, D.ph);
+                  VR ? D.Ubuf[cur] : nullptr, VR ? D.Ubuf[cur ^ 1] : nullptr, D.flags, D.fluid_list, t,
+                  D.n_fluid, D.g, D.ph);
 }
 
 // The halo step of every member with R rings; 45 simulations of 400 x 200 in

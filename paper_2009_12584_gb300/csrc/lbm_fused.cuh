@@ -39,8 +39,9 @@ struct MarchCfg {
 // Force, velocity and collision of one fluid node in place (fv: f on entry,
 // f* on exit; nbP: density plane at x + c_i; rho: the node's densities on
 // exit; u: the velocity of Eq. 3). The FP32 compute type runs the paired
-// path of the two-pass kernel (same arithmetic, same results).
-template <typename C>
+// path of the two-pass kernel (same arithmetic, same results); PAIRS: see
+// collide2.
+template <typename C, bool PAIRS>
 __device__ __forceinline__ void march_update(C fv[2][9], const C nbP[2][9], uint16_t fl, bool general,
                                              const PhysK<C>& ph, C rho_out[2], C u_out[2]) {
   if constexpr (sizeof(C) == 4) {
@@ -50,8 +51,8 @@ __device__ __forceinline__ void march_update(C fv[2][9], const C nbP[2][9], uint
       fp[i] = f2(fv[0][i], fv[1][i]);
       q[i] = f2(nbP[0][i], nbP[1][i]);
     }
-    const float2 r = general ? update_pair<true>(fp, q, fl, ph, u_out[0], u_out[1])
-                             : update_pair<false>(fp, q, fl, ph, u_out[0], u_out[1]);
+    const float2 r = general ? update_pair<true, PAIRS>(fp, q, fl, ph, u_out[0], u_out[1])
+                             : update_pair<false, PAIRS>(fp, q, fl, ph, u_out[0], u_out[1]);
     rho_out[0] = r.x;
     rho_out[1] = r.y;
 #pragma unroll
@@ -69,8 +70,8 @@ template <typename C>
 __device__ __forceinline__ void update_pairs(typename CPair<C>::V fp[9], const typename CPair<C>::V q[9], uint16_t fl,
                                              bool general, const PhysK<C>& ph, C rho_out[2], C u_out[2]) {
   if constexpr (sizeof(C) == 4) {
-    const float2 r = general ? update_pair<true>(fp, q, fl, ph, u_out[0], u_out[1])
-                             : update_pair<false>(fp, q, fl, ph, u_out[0], u_out[1]);
+    const float2 r = general ? update_pair<true, true>(fp, q, fl, ph, u_out[0], u_out[1])
+                             : update_pair<false, true>(fp, q, fl, ph, u_out[0], u_out[1]);
     rho_out[0] = r.x;
     rho_out[1] = r.y;
   } else {
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(MARCH_WARPS * 32, 4)
     if (fluid) {
       C rho_unused[2];
       C u_unused[2];
-      march_update<C>(fv, nbP, fl, general, ph, rho_unused, u_unused);
+      march_update<C, false>(fv, nbP, fl, general, ph, rho_unused, u_unused);
 #pragma unroll
       for (int s = 0; s < 2; ++s)
 #pragma unroll

@@ -224,7 +224,10 @@ __device__ __forceinline__ void density_node(const T* __restrict__ f, typename P
 
 // VR: whether the velocity planes may be read (16-bit storage with velocity
 // references); without it Uref is never touched and the kernel carries no
-// code for it, and 32 registers give 8 CTAs per SM.
+// code for it, and 32 registers give 8 CTAs per SM. The list entry is loaded
+// while the kernel before it drains (FP64 100 x 50: 14.2 us per step, 14.4 without);
+// with 16-bit storage after that (the pass takes 133 us at 4096^2 porous, 145
+// with the entry loaded before).
 template <typename T, bool VR = false>
 __global__ void __launch_bounds__(256, VR ? 1 : 8) k_density_list(const T* __restrict__ f, typename Pop<T>::C* __restrict__ P,
                                                       const typename Pop<T>::C* __restrict__ Pref,
@@ -233,8 +236,10 @@ __global__ void __launch_bounds__(256, VR ? 1 : 8) k_density_list(const T* __res
                                                       const int* __restrict__ list, int nfluid, Geo g,
                                                       PhysK<typename Pop<T>::C> ph) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const unsigned e = t < nfluid ? (unsigned)__ldg(list + t) : 0u;
+  unsigned e = 0;
+  if (!kDev<T> && t < nfluid) e = (unsigned)__ldg(list + t);
   pdl_wait();
+  if (kDev<T> && t < nfluid) e = (unsigned)__ldg(list + t);
   if (t < nfluid) density_node<T>(f, P, Pref, VR ? Uref : nullptr, flags, e, g);
 }
 
@@ -263,7 +268,8 @@ __device__ __forceinline__ void collide_node_pair(const T* __restrict__ f, T* __
     q[i] = __ldg(reinterpret_cast<const float2*>(P) + m);
   }
   float ux, uy;
-  const float2 rho = warp_edge ? update_pair<true>(fp, q, fl, ph, ux, uy) : update_pair<false>(fp, q, fl, ph, ux, uy);
+  const float2 rho = warp_edge ? update_pair<true, false>(fp, q, fl, ph, ux, uy)
+                                : update_pair<false, false>(fp, q, fl, ph, ux, uy);
   const float rr[2] = {rho.x, rho.y};
   UVal U{};
   if constexpr (kDev<T>) {
@@ -372,6 +378,20 @@ __device__ __forceinline__ void collide_node(const T* __restrict__ f, T* __restr
     store_bounced(fo, g, x, y, fl, fv, ref);
   }
   }
+}
+
+// The same for entry t of a list of nfluid. (Loading the entry in the caller
+// costs the two-pass batches 1.2%.)
+template <typename T>
+__device__ __forceinline__ void collide_node(const T* __restrict__ f, T* __restrict__ fo,
+                                             const typename Pop<T>::C* __restrict__ P,
+                                             const typename Pop<T>::C* __restrict__ Pref,
+                                             const UPair* __restrict__ Uref, UPair* __restrict__ Uo,
+                                             const uint16_t* __restrict__ flags, const int* __restrict__ list, int t,
+                                             int nfluid, const Geo& g, const PhysK<typename Pop<T>::C>& ph) {
+  const bool valid = t < nfluid;
+  const unsigned e = valid ? (unsigned)__ldg(list + t) : 0u;
+  collide_node<T>(f, fo, P, Pref, Uref, Uo, flags, e, valid, g, ph);
 }
 
 // VR as for k_density_list (Uref and Uo untouched without it). FP64: 128

@@ -129,8 +129,48 @@ __device__ __forceinline__ float2 rho_over_9_2(float2 rho) {
 // component changes only by the rounding of the nine final additions.
 // Directions go as opposite pairs, which share c.u, c.F and their products;
 // u is carried in both lanes, so that every operation is a paired one.
+//
+// PAIRS false: one direction at a time, u in one register and not in both lanes.
+// The same bits, more instructions and fewer registers: for kernels held at 56
+// to 64 registers, which spill otherwise (us per step with PAIRS, without:
+// tiled batch of 45 x 400 x 200 FP32 144, 135; 4096^2 porous by k_tile_tma 598,
+// 568, k_tile FP16 559, 550, k_tile FP32 453, 462; two-pass batch of 45 FP16
+// 102.5, 100.7). The halo kernels have 72 and 80.
+template <bool PAIRS>
 __device__ __forceinline__ void collide2(float2 f[9], float2 rho, float ux, float uy, float2 Fx, float2 Fy,
                                          const PhysK<float>& ph) {
+  if constexpr (!PAIRS) {
+    const float nusq15 = -1.5f * fmaf(ux, ux, uy * uy);
+    const float2 r9 = rho_over_9_2(rho);
+    const float2 r36 = mul2(KC.c025, r9);  // exact
+    const float2 om = f2(ph.omega[0], ph.omega[1]);
+    const float2 k9 = mul2(f2(ph.kF[0], ph.kF[1]), KC.w9);
+    const float2 k36 = mul2(f2(ph.kF[0], ph.kF[1]), KC.w36);
+    const float2 nuF3 = mul2(KC.cneg3, fma2(f2(ux), Fx, mul2(f2(uy), Fy)));
+    float2 acc = f2(0.0f);
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      const float cu = float(cx_of(i)) * ux + float(cy_of(i)) * uy;
+      const float p = fmaf(cu, fmaf(4.5f, cu, 3.0f), nusq15);
+      const float cu9 = 9.0f * cu;
+      float2 cF;  // c_i . F (c_i components are -1, 0, 1)
+      if (cx_of(i) == 0)
+        cF = cy_of(i) > 0 ? Fy : neg2(Fy);
+      else if (cy_of(i) == 0)
+        cF = cx_of(i) > 0 ? Fx : neg2(Fx);
+      else {
+        const float2 a = cx_of(i) > 0 ? Fx : neg2(Fx);
+        cF = cy_of(i) > 0 ? add2(a, Fy) : sub2(a, Fy);
+      }
+      const float2 src = mul2(i <= 4 ? k9 : k36, fma2(f2(cu9), cF, fma2(KC.c3, cF, nuF3)));
+      const float2 ri = i <= 4 ? r9 : r36;
+      const float2 delta = fma2(om, fma2(ri, f2(p), sub2(ri, f[i])), src);
+      acc = add2(acc, delta);
+      f[i] = add2(f[i], delta);
+    }
+    f[0] = sub2(f[0], acc);
+    return;
+  }
   const float2 ux2 = f2(ux), uy2 = f2(uy);
   const float2 nusq15 = mul2(KC.cneg15, fma2(ux2, ux2, mul2(uy2, uy2)));
   const float2 r9 = rho_over_9_2(rho);
@@ -194,12 +234,12 @@ __device__ __forceinline__ float2 moments_pair(const float2 fp[9], const float2 
 // neighbours (fl holds the neighbour bits); a node without any gets the
 // same result on either path. Returns rho of both components and, in
 // ux_out, uy_out, the velocity u of Eq. 3 the collision used.
-template <bool GENERAL>
+template <bool GENERAL, bool PAIRS>
 __device__ __forceinline__ float2 update_pair(float2 fp[9], const float2 q[9], uint16_t fl,
                                               const PhysK<float>& ph, float& ux_out, float& uy_out) {
   float2 Fx, Fy;
   const float2 rho = moments_pair<GENERAL>(fp, q, fl, ph, Fx, Fy, ux_out, uy_out);
-  collide2(fp, rho, ux_out, uy_out, Fx, Fy, ph);
+  collide2<PAIRS>(fp, rho, ux_out, uy_out, Fx, Fy, ph);
   return rho;
 }
 

@@ -125,8 +125,9 @@ static __global__ void __launch_bounds__(TILE_LIST_THREADS) k_tile_lists(const u
 // decoded again), so that phase 2 sums exactly what the next step pulls,
 // like the density pass. Pref, Uref and Uo are not used for 4- and 8-byte
 // storage.
-// The work of one CTA on tile `tile` of n_tiles (one simulation).
-template <typename T>
+// The work of one CTA on tile `tile` of n_tiles (one simulation). PAIRS: see
+// collide2.
+template <typename T, bool PAIRS>
 __device__ __forceinline__ void tile_step(int tile, int n_tiles, const T* __restrict__ f, T* __restrict__ fo,
                                           const typename Pop<T>::C* __restrict__ P,
                                           const typename Pop<T>::C* __restrict__ Pref,
@@ -184,7 +185,7 @@ __device__ __forceinline__ void tile_step(int tile, int n_tiles, const T* __rest
         asm volatile("prefetch.global.L2 [%0];" ::"l"(f + pslot(g, i, k2 - cx_of(i) - cy_of(i) * g.px)));
     }
     C rho[2], u[2];
-    march_update<C>(fv, nbP, fl, warp_edge, ph, rho, u);
+    march_update<C, PAIRS>(fv, nbP, fl, warp_edge, ph, rho, u);
     UVal U{};
     if constexpr (kDev<T>) {
       if (Uo) {
@@ -253,7 +254,7 @@ __global__ void __launch_bounds__(TILE_THREADS, TILE_MINB)
            const uint16_t* __restrict__ flags,
            const uint16_t* __restrict__ entries, const int* __restrict__ offsets, const int2* __restrict__ cnt,
            Geo g, int ntx, PhysK<typename Pop<T>::C> ph) {
-  tile_step<T>(blockIdx.x, gridDim.x, f, fo, P, Pref, Uref, Uo, Po, flags, entries, offsets, cnt, g, ntx, ph);
+  tile_step<T, sizeof(T) == 4>(blockIdx.x, gridDim.x, f, fo, P, Pref, Uref, Uo, Po, flags, entries, offsets, cnt, g, ntx, ph);
 }
 
 template <typename T>

@@ -285,7 +285,7 @@ static __global__ void __launch_bounds__(TMA_THREADS, TMA_MINB)
         nbP[1][i] = v.y;
       }
       float rho[2], u[2];
-      march_update<float>(fv, nbP, fl, warp_edge, ph, rho, u);
+      march_update<float, false>(fv, nbP, fl, warp_edge, ph, rho, u);
       if (t < n_own) {
         if (!warp_border) {
 #pragma unroll
