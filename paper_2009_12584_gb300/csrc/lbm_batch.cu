@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_collide_batch(c
 template <typename T, int R, bool VR>
 __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
     k_halo_batch(const HaloArgs<T>* __restrict__ args, const CUtensorMap* __restrict__ maps,
-                 const HaloTile* __restrict__ work, const int4* __restrict__ cur, const int* __restrict__ stop,
+                 const HaloTile* __restrict__ work, const int4* __restrict__ cur, const int* __restrict__ stop_word,
                  int parity) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ HaloArgs<T> a;
@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ?
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
   pdl_wait();  // the launch before; what is read above it does not write
+  const int stop = threadIdx.x == 0 ? *(const volatile int*)stop_word : 0;
   if (threadIdx.x == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(work + blockIdx.x + HALO_AHEAD));
   const HaloArgs<T>* src = args + 2 * h.member + parity;

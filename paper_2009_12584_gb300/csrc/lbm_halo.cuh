@@ -228,18 +228,19 @@ struct HaloSmem {
 // smem_raw: shared memory of HaloSmem::BYTES. The error word is set to 1 when
 // the copies were not seen to complete within the bound; extra_tx: see
 // tma_issue. ready(): called once by every thread before the first use of a.
-// stop: a CTA that finds it set does nothing (it would wait like the one that
-// set it) and sets its own simulation's error word, whose step is missing then
-// (in a batch the words are apart). Another CTA of the same launch may be
-// setting stop, so one thread reads it, and the CTA's first barrier carries the
-// answer: all of its threads go on or none does.
+// stop: the stop word, as thread 0 read it. A CTA that finds it set does nothing
+// (it would wait like the one that set it) and sets its own simulation's error
+// word, whose step is missing then (in a batch the words are apart). Another CTA
+// of the same launch may be setting the word, so one thread reads it, early, and
+// the CTA's first barrier carries the answer: all of its threads go on or none
+// does.
 // eval: an EvalOut that takes the moments (rho^A, rho^B, u of Eq. 3) of the
 // tile's nodes instead of a step, or NoEval; NaN where the wait ran out or the
 // CTA stops, so that nothing older is taken for them.
 struct NoEval {};
 template <typename T, int R, bool VR, typename Ready, typename Eval = NoEval>
 __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* mapf, const CUtensorMap* mapref,
-                                          const uint32_t* entries, const HaloArgs<T>& a, const int* stop, int ntx,
+                                          const uint32_t* entries, const HaloArgs<T>& a, int stop, int ntx,
                                           unsigned char* smem_raw, uint32_t extra_tx, Ready&& ready,
                                           const Eval& eval = Eval{}) {
   using C = typename Pop<T>::C;
@@ -265,9 +266,12 @@ __device__ __forceinline__ void halo_tile(const HaloTile& h, const CUtensorMap* 
       }
     }
   };
-  if (tid == 0 && (stopped = *(const volatile int*)stop) == 0) {
+  if (tid == 0) {
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    stopped = stop;
+  }
+  if (tid == 0 && !stop) {
     // the window's first node: column x0 - O + LP (a multiple of 4 nodes with
     // 16-bit storage, of 2 otherwise: 16-byte aligned), row y0 - R - c_i.y + GH
     const int xw = x0 - S::O + LP, yw = y0 - R + GH;
@@ -467,9 +471,10 @@ __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ?
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
   pdl_wait();  // the step before; what is read above, a geometry's lists, it does not write
+  const int stop = threadIdx.x == 0 ? *(const volatile int*)a.stop : 0;
   if (threadIdx.x == 32 && blockIdx.x + HALO_AHEAD < gridDim.x)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(work + blockIdx.x + HALO_AHEAD));
-  halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, a.stop, a.ntx, smem_raw, extra_tx, [] {});
+  halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, stop, a.ntx, smem_raw, extra_tx, [] {});
 }
 
 // The moments of the current state at fluid nodes, one launch where the
@@ -486,7 +491,8 @@ __global__ void __launch_bounds__(halo_threads<R>, R == 1 ? 4 : 3)
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
   pdl_wait();
-  halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, a.stop, a.ntx, smem_raw, extra_tx, [] {}, out);
+  const int stop = threadIdx.x == 0 ? *(const volatile int*)a.stop : 0;
+  halo_tile<T, R, VR>(h, &mapf, &mapref, a.entries, a, stop, a.ntx, smem_raw, extra_tx, [] {}, out);
 }
 
 }  // namespace lbm
