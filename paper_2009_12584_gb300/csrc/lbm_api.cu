@@ -720,6 +720,17 @@ lbm_status do_eval(lbm_ctx* c, const EvalOut<O>& out, bool solid = true) {
   return after_launch(c, "k_collide(eval)");
 }
 
+// Whether a kernel may write doubles at p: memory of the context's device, on 8
+// bytes.
+bool on_device(const lbm_ctx* c, const void* p) {
+  cudaPointerAttributes at;
+  if ((uintptr_t)p % 8 || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == c->device;
+}
+
 // Four consecutive fields of n values.
 template <typename O>
 EvalOut<O> fields(O* base, int64_t n) {
@@ -1065,9 +1076,11 @@ lbm_status lbm_moments(lbm_ctx* c, double* rA, double* rB, double* ux, double* u
   const int64_t N = (int64_t)c->g.nx * c->g.ny;
   double* outs[4] = {rA, rB, ux, uy};
   EvalOut<double> out{{rA, rB, ux, uy}};
-  // an array that is not on 8 bytes gets its field as a copy
+  // the kernel writes arrays in this device's memory; any other (pinned host
+  // memory, another device's, not on 8 bytes) gets its field as a copy, which
+  // also refuses what is no address
   for (int a = 0; a < 4; ++a)
-    if ((uintptr_t)outs[a] % 8) out.p[a] = c->stage + a * N;
+    if (outs[a] && !on_device(c, outs[a])) out.p[a] = c->stage + a * N;
   lbm_status s;
   LBM_DISPATCH(c, s = (do_eval<T, 1>(c, out)); break);
   for (int a = 0; a < 4 && !s; ++a)
