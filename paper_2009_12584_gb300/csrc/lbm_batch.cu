@@ -116,6 +116,8 @@ __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ?
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ HaloArgs<T> a;
   static_assert(sizeof(a) % 4 == 0 && sizeof(a) / 4 <= halo_threads<R>, "one thread per word");
+  __shared__ __align__(8) uint64_t bar;
+  halo_bar_init(bar);
   HaloTile h;
   h.n = __ldg(&work[blockIdx.x].n);
   *(int4*)&h.e0 = __ldg((const int4*)&work[blockIdx.x].e0);
@@ -135,7 +137,7 @@ __global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ?
     if (kDev<T>) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(mr) : "memory");
   }
   const uint32_t* entries = (const uint32_t*)__ldg((const unsigned long long*)&src->entries);
-  halo_tile<T, R, VR>(h, mf, mr, entries, a, stop, __ldg(&src->ntx), smem_raw, extra_tx,
+  halo_tile<T, R, VR>(h, mf, mr, entries, a, stop, __ldg(&src->ntx), smem_raw, bar, extra_tx,
                       [&] {
                         if (threadIdx.x < sizeof(a) / 4)
                           ((uint32_t*)&a)[threadIdx.x] = __ldg((const uint32_t*)src + threadIdx.x);

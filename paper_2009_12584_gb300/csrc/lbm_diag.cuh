@@ -158,6 +158,7 @@ static __global__ void __launch_bounds__(32 * DIAG_NQ) k_diag_final(const double
     if (lane == 0) out[q] = v;
     return;
   }
+  const int e = *err;
   double br = 0.0;
   if (a.bridge_x >= 0) {
     // rho^A on the column, 0 at solid nodes
@@ -184,7 +185,7 @@ static __global__ void __launch_bounds__(32 * DIAG_NQ) k_diag_final(const double
   }
   if (lane == 0) {
     out[16] = br;
-    out[DIAG_NQ] = *err;
+    out[DIAG_NQ] = e;
   }
 }
 
