@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 2 : 4) k_collide_batch(c
 // memory, hence the fence. cur: per member two indices into its maps, and its
 // extra_tx.
 template <typename T, int R, bool VR>
-__global__ void __launch_bounds__(halo_threads<R>, sizeof(T) == 8 ? 1 : R == 1 ? 4 : 3)
+__global__ void __launch_bounds__(halo_threads<R>, R == 1 ? 4 : 3)
     k_halo_batch(const HaloArgs<T>* __restrict__ args, const CUtensorMap* __restrict__ maps,
                  const HaloTile* __restrict__ work, const int4* __restrict__ cur, const int* __restrict__ stop_word,
                  int parity) {
@@ -261,9 +261,9 @@ struct BLayout {
   size_t desc, fblk, iblk, tblk, hargs, hmaps, hcur, hwork, stop, total;
   int64_t table;  // entries of the longest block table
 };
+// (none for FP64 members, which step by the two passes)
 size_t hargs_bytes(int storage) {
-  return storage == LBM_STORE_FP64 ? sizeof(HaloArgs<double>)
-                                   : storage == LBM_STORE_FP32 ? sizeof(HaloArgs<float>) : sizeof(HaloArgs<__half>);
+  return storage == LBM_STORE_FP64 ? 0 : storage == LBM_STORE_FP32 ? sizeof(HaloArgs<float>) : sizeof(HaloArgs<__half>);
 }
 
 // The tiled schedule runs when the storage is 4 or 8 bytes and every member
@@ -293,7 +293,8 @@ BLayout blayout(int n, lbm_ctx* const* ctxs) {
     nf += ((int64_t)c->g.nx * c->g.ny + 127) / 128;
     ni += (c->if_capacity + 127) / 128;
     nt += tiled ? c->n_tiles : 0;
-    nw += c->prm.storage != LBM_STORE_FP64 ? halo_tile_count(c->g, halo_rows(c->prm.storage == LBM_STORE_FP32 ? 4 : 2)) : 0;
+    if (c->prm.storage != LBM_STORE_FP64)
+      nw += halo_tile_count(c->g, halo_rows(c->prm.storage == LBM_STORE_FP32 ? 4 : 2));
   }
   BLayout L;
   size_t off = 0;
@@ -746,7 +747,7 @@ lbm_status lbm_batch_create(int32_t n, lbm_ctx* const* ctxs, void* d_workspace, 
   b->h_desc = malloc((size_t)n * desc_bytes(b->storage));
   b->h_tab = (int2*)malloc((size_t)(L.table + 1) * sizeof(int2));
   b->m = (Member*)malloc((size_t)n * sizeof(Member));
-  b->h_hargs = malloc(2 * (size_t)n * hargs_bytes(b->storage));
+  b->h_hargs = malloc(2 * (size_t)n * hargs_bytes(b->storage) + 1);
   b->h_hcur = (int4*)malloc((size_t)n * sizeof(int4));
   b->d_hargs = b->ws + L.hargs;
   b->d_hmaps = (CUtensorMap*)(b->ws + L.hmaps);

@@ -235,9 +235,10 @@ __device__ __forceinline__ void halo_bar_init(uint64_t& bar) {
 // populations (pairs; x in units of Pop<T>::V, FP64 of 8 bytes), with a box of
 // one tile's window; mapref: of the references. a: the simulation's arguments,
 // and entries its list, which the thread that issues the copies has at hand.
-// smem_raw: shared memory of HaloSmem::BYTES; bar: see halo_bar_init. The error word is set to 1 when
-// the copies were not seen to complete within the bound; extra_tx: see
-// tma_issue. ready(): called once by every thread before the first use of a.
+// smem_raw: shared memory of HaloSmem::BYTES; bar: see halo_bar_init. The error
+// word is set to 1 when the copies were not seen to complete within the bound;
+// extra_tx: see tma_issue. ready(): called once by every thread before the first
+// use of a.
 // stop: the stop word, as thread 0 read it. A CTA that finds it set does nothing
 // (it would wait like the one that set it) and sets its own simulation's error
 // word, whose step is missing then (in a batch the words are apart). Another CTA
