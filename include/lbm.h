@@ -124,8 +124,8 @@ typedef enum {
  * AUTO picks the schedule measured fastest on GB300: TWO_PASS for FP64 storage
  * (bound by the FP64 pipe: the single passes compute densities around a tile
  * again) and HALO for the others (porous 4096^2, us per step under the
- * improved scheme / LLKC: FP32 398 / 357 against 449 / 427 for TILED and 514 /
- * 488 for TWO_PASS; FP16 367 / 315 against 434 / 412 for TWO_PASS); the
+ * improved scheme / LLKC: FP32 390 / 357 against 449 / 427 for TILED and 521 /
+ * 498 for TWO_PASS; FP16 362 / 313 against 433 / 413 for TWO_PASS); the
  * workspace of 4- and 8-byte storage also keeps room for the tiled lists,
  * which batches use. */
 typedef enum {

@@ -649,10 +649,9 @@ lbm_status do_step(lbm_ctx* c, int nsteps) {
   }
   const int k = c->prm.kernel;
   // AUTO with FP64 storage: bound by the FP64 pipe, so the schedule that
-  // sums and updates every node once. Before the update's operations were
-  // halved too, 100 x 50 took 20.5 us per step against 61 for the single
-  // passes, 800 x 600 207 against 298 us, 1400 x 1000 553 against 701 us
-  // (with the operations halved 15.5 us and, at 800 x 600, 132 us).
+  // sums and updates every node once (walled boxes, us per step by two passes /
+  // halo / tiles: 100 x 50 18 / 44 / 57, 800 x 600 226 / 284 / 309, 1400 x 1000
+  // 631 / 732 / 800).
   const bool halo = k == LBM_KERNEL_HALO || (k == LBM_KERNEL_AUTO && sizeof(T) != 8);
   if (halo) {
     lbm_status s = use_halo_lists(c, true, c->stream);
@@ -896,7 +895,7 @@ lbm_status lbm_create(const lbm_params* params, void* d_workspace, size_t bytes,
                          "cudaDeviceGetAttribute");
   if (!s) s = check_cuda(c, cudaMemsetAsync(c->ws, 0, L.total, c->stream), "cudaMemsetAsync");
   if (!s && c->tma && !encode_tma_maps(c)) s = LBM_ERR_CUDA;
-  if (!s) c->hmaps_ok = encode_halo_maps(c);  // without them the two-pass schedule runs
+  if (!s) c->hmaps_ok = encode_halo_maps(c);  // without them do_step falls back
   if (s) {
     delete c;
     return s;

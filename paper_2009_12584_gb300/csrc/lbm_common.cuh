@@ -465,11 +465,12 @@ __device__ __forceinline__ double rho_over_9(double rho) {
 //   g = 3 w_i (1 - 1/(2 tau)) c.F, E = 3 c.u g - 3 w_i (1 - 1/(2 tau)) u.F
 // along c and -c, which share e, g and E. FP64 instructions run at 1/32 of the
 // FP32 rate on this GPU and bound every FP64 pass: about 230 per node, where
-// one direction at a time took 366 (800 x 600, two passes: 402 -> 226 us per
-// step). Relaxing the sum and the difference of a pair instead (180; 190 us)
-// rounds the O(1) part of each increment: against long double, after 300 steps
-// of 320 droplets, 1.0 to 1.7 times the error in rho and 1.25 to 1.37 times in
-// the momentum; this form 0.97 to 1.00 times.
+// one direction at a time took 366 (45 simulations of 400 x 200 by two passes:
+// 1290 -> 1005 us per step). Relaxing the sum and the difference of a pair
+// instead (180; 839 us) rounds the O(1) part of each increment: against long
+// double, after 300 steps of 160 droplets each, 0.76 to 1.7 times the error in
+// rho (tau 1.6 to 0.6) and 1.25 to 1.37 times in the momentum; this form 0.68 to
+// 1.005 and 0.94 to 1.005 times.
 template <typename C>
 __device__ __forceinline__ void update_node(C f[2][9], const C nbP[2][9], uint16_t fl, bool walls,
                                             const PhysK<C>& ph, C rho[2], C u[2]) {
