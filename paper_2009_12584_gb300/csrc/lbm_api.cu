@@ -585,6 +585,8 @@ lbm_status write_halo_lists(lbm_ctx* c, const int* totals) {
       }
     return nullptr;
   };
+  // the records first: contexts with the area have room for them there, so that a
+  // batch may gather them whether the rest is in the plane or out of the way
   HaloTile* work = (HaloTile*)take((size_t)totals[2] * sizeof(HaloTile));
   uint32_t* entries = (uint32_t*)take((size_t)totals[0] * 4);
   uint2* cells = (uint2*)take((size_t)(totals[1] > 0 ? totals[1] : 1) * 8);

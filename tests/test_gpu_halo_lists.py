@@ -34,7 +34,7 @@ def _interface_cells(mask, per_x, per_y):
 def _masks():
     open_box = inputs.flat_wall_mask(200, 96)
     wells = np.ones((66, 99), np.uint8)
-    wells[1::3, 1::3] = 0  # eight nodes in nine are interface cells
+    wells[1::3, 1::3] = 0  # eight nodes in nine are interface cells (here the planes' padding holds their lists)
     return {"wall": open_box, "30%": inputs.random_solid_mask(131, 83, 1, 0.3),
             "45%": inputs.random_solid_mask(131, 83, 2, 0.45), "60%": inputs.random_solid_mask(131, 83, 3, 0.6),
             "wells": wells}
@@ -63,8 +63,7 @@ def test_lists_find_room(storage, kernel, wet, exact, geometry):
     b = _sim(mask, storage, "two_pass", wet, exact)
     n0 = a.launch_count
     a.step(3)
-    if geometry != "wells":  # (where they need not fit)
-        assert a.launch_count - n0 == 3
+    assert a.launch_count - n0 == 3
     b.step(3)
     assert torch.equal(a.forces(), b.forces())
     for x, y in zip(a.moments(), b.moments()):
@@ -119,5 +118,37 @@ def test_lists_give_way_to_batches(storage, kernel, graph):
             a.set_populations(f)
             b.set_populations(f)
         both(1, True)
+        # the halo launches are put together anew while the lists may be away
+        for (a, b), (kind, kw) in zip(pairs, (LLKC, IMPROVED, LLKC)):
+            a.set_wetting(kind, **kw)
+            b.set_wetting(kind, **kw)
+        both(2, True)
+        if schedule == "tiled":
+            batch.set_schedule("two_pass")
+            both(3, True)
         both(1, False)
     batch.close()
+
+
+@pytest.mark.parametrize("kernel,launches", [("auto", 2), ("halo", 3)])
+def test_without_any_room(kernel, launches):
+    """Eight nodes in nine are interface cells, on a grid with little padding:
+    the lists fit nowhere. AUTO runs tiles (Eq. 8 and the tiles, after a first
+    step that builds their lists and sums the densities), HALO the two passes."""
+    nx, ny = 2016, 699
+    mask = np.ones((ny, nx), np.uint8)
+    mask[1::3, 1::3] = 0
+    cap = _interface_cells(mask, True, True)
+    sims = []
+    for k, c in ((kernel, cap), ("two_pass", 0)):
+        sim = lbm.Simulation(nx, ny, storage="fp32", kernel=k, periodic_x=True, periodic_y=True, max_interface=c)
+        sim.set_geometry(mask).set_wetting(IMPROVED[0], **IMPROVED[1])
+        sims.append(sim.init_fields(*inputs.random_fields(nx, ny, 3, umax=0.05)))
+    a, b = sims
+    a.step(1)
+    n0 = a.launch_count
+    a.step(2)
+    assert a.launch_count - n0 == 2 * launches
+    assert torch.equal(a.populations(), b.step(3).populations())
+    assert torch.equal(a.moments()[0], b.moments()[0])
+    assert torch.equal(a.step(2).populations(), b.step(2).populations())
